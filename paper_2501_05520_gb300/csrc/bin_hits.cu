@@ -37,6 +37,8 @@ __global__ void k_clear(Buffers b, int32_t phi_bins) {
     b.cnt[CNT_SV] = 0;
     b.cnt[CNT_CELLS_USED] = 0;
     b.cnt[CNT_LINKS_USED] = 0;
+    b.cnt[CNT_DBL_WORK] = 0;
+    b.cnt[CNT_LNK_WORK] = 0;
     b.cnt[CNT_SCAN_BINS] = (unsigned long long)nb;
     b.cnt[CNT_SCAN_HITS] = (unsigned long long)N;
   }

@@ -114,16 +114,16 @@ struct ConnWarp {
   float4 qp0[kQueue];        // window pairs: the source's inner hit (x, y, z, r)
   uint4 q[kQueue];           //   source cell, target (outer hit | slot << 29), middle hit,
                              //   inner hit on layer 0
-  float4 p1;                 // middle hit
-  uint4 rg[kMaxOuter];       //   its forward windows, one per outer slot
+  uint4 rg[kMaxOuter];       // middle hit: its forward windows, one per outer slot
   uint32_t so[kMaxInner];    //   its incoming segments: first cell
   uint32_t sc[kMaxInner];    //   and number of cells
   uint32_t sb[kMaxInner + 1];  //   incoming cells before each segment (the last: all)
   float tmin, scale, m;      // the staged piece: slope origin and scale of the buckets,
                              //   smallest r2 - r1
   int piece;                 // the staged piece (-1: none)
-  unsigned long long chunk_next, chunk_end, used;  // link slots
-  uint32_t chunk_size;
+  unsigned long long chunk_next, chunk_end;  // link slots
+  uint32_t used;             //   handed out
+  float ahead;               //   search_ahead of the warp's hits
 };
 
 // Bucket of a slope (monotone non-decreasing in x): the same correctly rounded
@@ -137,7 +137,7 @@ __device__ __forceinline__ int slope_bucket(float x, float tmin, float scale) {
 // unused (a hole), and link slots are scanned by the later stages.
 constexpr uint32_t kLinkChunkMax = 256;
 
-// Warp chunk reservation with the chunk state in shared memory, lane 0 acting.
+// Warp chunk reservation (as chunk_take) with the chunk state in shared memory, lane 0 acting.
 __device__ __forceinline__ unsigned long long chunk_take_shared(
     ConnWarp& W, unsigned long long* counter, uint32_t n, unsigned long long* hlo,
     unsigned long long* hhi) {
@@ -147,15 +147,14 @@ __device__ __forceinline__ unsigned long long chunk_take_shared(
     if (next + n > end) {
       lo = next;
       hi = end;
-      const uint32_t size = W.chunk_size;
-      const uint32_t want = size == 0 ? n : (n > size ? n : size);
-      W.chunk_size = size == 0 ? (n > kChunkMin ? n : kChunkMin) : min(2 * size, kLinkChunkMax);
+      const uint32_t want = chunk_size(n, W.used, W.ahead, kLinkChunkMax);
       next = atomicAdd(counter, (unsigned long long)want);
       end = next + want;
     }
     r = next;
     W.chunk_next = next + n;
     W.chunk_end = end;
+    W.used += n;
   }
   r = __shfl_sync(kFull, r, 0);
   *hlo = __shfl_sync(kFull, lo, 0);
@@ -175,8 +174,8 @@ __global__ void __launch_bounds__(kConnWarps * 32, kConnBlocksPerSm)
   const float bins_per_rad = (float)B / kTwoPi;
   if (lane == 0) {
     W.chunk_next = W.chunk_end = 0;
-    W.chunk_size = 0;
     W.used = 0;
+    W.ahead = 0.0f;
   }
   __syncwarp();
   auto mark_link_hole = [&](unsigned long long lo, unsigned long long hi) {
@@ -213,7 +212,6 @@ __global__ void __launch_bounds__(kConnWarps * 32, kConnBlocksPerSm)
       unsigned long long hlo, hhi;
       const unsigned long long base = chunk_take_shared(W, &b.cnt[CNT_LINKS], n, &hlo, &hhi);
       mark_link_hole(hlo, hhi);
-      if (lane == 0) W.used += n;
       if (base + n > cap_links) {
         if (lane == 0) atomicOr(&b.cnt[CNT_STATUS], ST_LINKS);
         mark_link_hole(base, base + n);  // slots below the capacity stay readable
@@ -231,23 +229,26 @@ __global__ void __launch_bounds__(kConnWarps * 32, kConnBlocksPerSm)
     __syncwarp();
   };
 
+  const uint32_t n_warps = gridDim.x * kConnWarps;
+  const uint32_t per = search_chunk(n_sorted, n_warps);
+  // chunks of sorted middle hits, the first by the warp's number, the others from a work
+  // counter
+  uint32_t chunk = blockIdx.x * kConnWarps + (threadIdx.x >> 5);
   for (;;) {
-    unsigned long long chunk = 0;
-    if (lane == 0) chunk = atomicAdd(&b.cnt[CNT_LNK_WORK], 1ull);
-    const uint64_t s0 = __shfl_sync(kFull, chunk, 0) * 32ull;
+    const uint32_t s0 = chunk * per;  // < n_sorted + 2 * per * n_warps < 2^32
     if (s0 >= n_sorted) break;
     // one round of loads finds the hits with incoming cells and outer layers
     uint32_t my_gb = 0;
     bool work = false;
     {
-      const uint64_t s = s0 + lane;
-      if (s < n_sorted) {
+      const uint32_t s = s0 + lane;
+      if ((uint32_t)lane < per && s < n_sorted) {
         my_gb = b.hbin[s];
         const int L = (my_gb / (uint32_t)B) % kLayers;
         if (pt.n_outer[L] > 0) {
           uint32_t any = 0;
           // slots past the layer's own inner layers are written empty
-          for (int k = 0; k < pt.n_inner[L]; ++k) any |= b.seg[s * pt.max_inner + k].y;
+          for (int k = 0; k < pt.n_inner[L]; ++k) any |= b.seg[(uint64_t)s * pt.max_inner + k].y;
           work = any != 0;
         }
       }
@@ -256,7 +257,7 @@ __global__ void __launch_bounds__(kConnWarps * 32, kConnBlocksPerSm)
     while (todo) {
       const int src = __ffs(todo) - 1;
       todo &= todo - 1;
-      const uint32_t h1 = (uint32_t)s0 + src;
+      const uint32_t h1 = s0 + src;
       const uint32_t gb = __shfl_sync(kFull, my_gb, src);
       const int L1 = (gb / (uint32_t)B) % kLayers;
       const float4 p1 = b.hit4[h1];
@@ -283,7 +284,7 @@ __global__ void __launch_bounds__(kConnWarps * 32, kConnBlocksPerSm)
         W.rg[lane] = rg;
       }
       if (lane == 0) {
-        W.p1 = p1;
+        W.ahead = search_ahead(n_sorted, h1 + 1);
         W.piece = -1;
       }
       __syncwarp();
@@ -489,11 +490,13 @@ __global__ void __launch_bounds__(kConnWarps * 32, kConnBlocksPerSm)
         if (valid_next) p0_next = b.hit4[h0_next];
       }
     }
+    if (lane == 0) chunk = n_warps + (uint32_t)atomicAdd(&b.cnt[CNT_LNK_WORK], 1ull);
+    chunk = __shfl_sync(kFull, chunk, 0);
   }
   while (qtail != qhead) process(min(32u, qtail - qhead));
   __syncwarp();
   mark_link_hole(W.chunk_next, W.chunk_end);
-  if (lane == 0 && W.used) atomicAdd(&b.cnt[CNT_LINKS_USED], W.used);
+  if (lane == 0 && W.used) atomicAdd(&b.cnt[CNT_LINKS_USED], (unsigned long long)W.used);
 }
 
 // Position of inner hit h in the cells [lo, hi) of one segment (ordered by inner hit, each
@@ -592,7 +595,6 @@ __global__ void k_link_targets(Buffers b, pt_cuts cuts, int32_t B, int max_inner
 
 void launch_connect(const Buffers& b, const Params& p, const Launch& l, cudaStream_t s,
                     bool gated) {
-  cudaMemsetAsync(&b.cnt[CNT_LNK_WORK], 0, sizeof(unsigned long long), s);  // work counter
   if (gated) {
     PT_TRACE(l, s, "k_connect",
              k_connect<true><<<l.sms * kConnBlocksPerSm, kConnWarps * 32, 0, s>>>(

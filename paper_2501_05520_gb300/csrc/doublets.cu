@@ -86,8 +86,8 @@ __device__ __forceinline__ uint4 reverse_window(const Buffers& b, const pt_cuts&
   return r;
 }
 
-// Warps take chunks of 32 consecutive sorted (outer) hits from a work counter.  The
-// chunk's windows are found lane-parallel (one hit per lane, all of its loads in flight
+// Warps take chunks of a few consecutive sorted (outer) hits (search_chunk), the first
+// by their own number, the others from a work counter.  The chunk's windows are found lane-parallel (one hit per lane, all of its loads in flight
 // at once) and kept in shared memory; the warp then searches them hit by hit.
 __global__ void __launch_bounds__(kWarpsPerBlock * 32, 5)
     k_doublets(Buffers b, pt_cuts cuts, PairTable pt, int32_t B, uint64_t cap_cells) {
@@ -103,21 +103,20 @@ __global__ void __launch_bounds__(kWarpsPerBlock * 32, 5)
   const uint32_t n_sorted = b.bin_start[E * kLayers * B];
   const float bins_per_rad = (float)B / kTwoPi;
   WarpChunk ch;
-  unsigned long long used = 0;
   auto mark_hole = [&](unsigned long long lo, unsigned long long hi) {
     hi = min(hi, (unsigned long long)cap_cells);
     for (unsigned long long i = lo + lane; i < hi; i += 32) b.cell_out[i] = kHole;
   };
 
-  for (;;) {
-    unsigned long long chunk = 0;
-    if (lane == 0) chunk = atomicAdd(&b.cnt[CNT_DBL_WORK], 1ull);
-    const uint64_t s0 = __shfl_sync(kFull, chunk, 0) * 32ull;
+  const uint32_t n_warps = gridDim.x * kWarpsPerBlock;
+  const uint32_t per = search_chunk(n_sorted, n_warps);
+  for (uint32_t chunk = blockIdx.x * kWarpsPerBlock + wib;;) {
+    const uint32_t s0 = chunk * per;  // < n_sorted + 2 * per * n_warps < 2^32
     if (s0 >= n_sorted) break;
-    const uint32_t nh = (uint32_t)min((uint64_t)32, (uint64_t)n_sorted - s0);
+    const uint32_t nh = min(per, n_sorted - s0);
     __syncwarp();
     if ((uint32_t)lane < nh) {
-      const uint32_t s = (uint32_t)s0 + lane;
+      const uint32_t s = s0 + lane;
       const uint32_t gb = b.hbin[s];
       const float4 ho = b.hit4[s];
       const float a = 0.5f * cuts.kmax * ho.w;
@@ -136,7 +135,7 @@ __global__ void __launch_bounds__(kWarpsPerBlock * 32, 5)
     __syncwarp();
 
     for (uint32_t j = 0; j < nh; ++j) {
-      const uint32_t s = (uint32_t)s0 + j;
+      const uint32_t s = s0 + j;
       const float4 ho = st_hit[wib][j];
       const int nin = st_nin[wib][j];
       // the slots the hit's layer does not use are written empty, so readers need not
@@ -174,9 +173,9 @@ __global__ void __launch_bounds__(kWarpsPerBlock * 32, 5)
         uint32_t seg_off = 0, seg_cnt = 0;
         if (cnt > 0) {
           unsigned long long hlo, hhi;
-          const unsigned long long base = chunk_take(ch, &b.cnt[CNT_CELLS], cnt, &hlo, &hhi);
+          const unsigned long long base = chunk_take(ch, &b.cnt[CNT_CELLS], cnt,
+                                                     search_ahead(n_sorted, s + 1), &hlo, &hhi);
           mark_hole(hlo, hhi);
-          used += cnt;
           if (base + cnt > cap_cells) {
             if (lane == 0) atomicOr(&b.cnt[CNT_STATUS], ST_CELLS);
             mark_hole(base, base + cnt);  // slots below the capacity stay readable
@@ -210,15 +209,16 @@ __global__ void __launch_bounds__(kWarpsPerBlock * 32, 5)
         __syncwarp();
       }
     }
+    if (lane == 0) chunk = n_warps + (uint32_t)atomicAdd(&b.cnt[CNT_DBL_WORK], 1ull);
+    chunk = __shfl_sync(kFull, chunk, 0);
   }
   mark_hole(ch.next, ch.end);
-  if (lane == 0 && used) atomicAdd(&b.cnt[CNT_CELLS_USED], used);
+  if (lane == 0 && ch.total) atomicAdd(&b.cnt[CNT_CELLS_USED], (unsigned long long)ch.total);
 }
 
 }  // namespace
 
 void launch_doublets(const Buffers& b, const Params& p, const Launch& l, cudaStream_t s) {
-  cudaMemsetAsync(&b.cnt[CNT_DBL_WORK], 0, sizeof(unsigned long long), s);  // work counter
   PT_TRACE(l, s, "k_doublets",
            k_doublets<<<l.sgrid, kWarpsPerBlock * 32, 0, s>>>(b, p.cuts, p.pairs, p.phi_bins,
                                                                (uint64_t)p.max_cells));

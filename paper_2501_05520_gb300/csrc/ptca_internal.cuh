@@ -39,7 +39,7 @@ enum : int {
   CNT_SCORE_STATUS = 9,  // status bits of the standalone gate scoring (pt_gate_score)
   CNT_CELLS_USED = 10,  // cells written (CNT_CELLS counts reserved slots incl. holes)
   CNT_LINKS_USED = 11,  // links written (CNT_LINKS counts reserved slots incl. holes)
-  CNT_DBL_WORK = 12,    // doublet search: next chunk of 32 sorted hits
+  CNT_DBL_WORK = 12,    // doublet search: next chunk of sorted hits
   CNT_SCAN_EV = 13,     // events (size of the scan over per-event vertex counts)
   CNT_VTX = 14,         // vertices of the batch
   CNT_RAW_STATUS = 15,  // raw input: status bits (RAW_*), not reset by the chain
@@ -47,7 +47,7 @@ enum : int {
   CNT_RAW_RUNS = 17,    // raw input: module runs (size of the hit-count scan)
   CNT_RAW_HITS = 18,    // raw input: hits made from the digis
   CNT_RAW_BIG = 19,     // raw input: long module runs listed for the block-per-run launch
-  CNT_LNK_WORK = 20,    // link search: next chunk of 32 sorted middle hits
+  CNT_LNK_WORK = 20,    // link search: next chunk of sorted middle hits
   CNT_DEBUG_SITE = 22,  // debug build: the first failing bounds check (DebugSite)
   CNT_N = 24
 };
@@ -522,29 +522,52 @@ __device__ __forceinline__ unsigned warp_incl_scan(unsigned v) {
 
 constexpr uint32_t kHole = 0xffffffffu;  // marks a reserved but unused slot
 
-// Per-warp bump allocator over a global counter.  The first chunk is exactly the first
-// request (a warp that makes one request wastes nothing); later chunks double from
-// kChunkMin up to kChunkMax, so a busy warp takes a global atomic about once per
-// kChunkMax slots instead of once per request.  The unused tail of a chunk becomes a
-// hole that the owner marks.  All members are warp-uniform.
+// Sorted hits that a warp of the two searches takes at once, of n_sorted hits over `warps`
+// warps.  A search warp handles its hits one after the other, so large chunks leave most
+// of the GPU idle on a single event (41k hits in chunks of 32 keep 1281 of 6080 warps
+// busy), and uneven hits leave the last warps of a batch running alone.  The chunk gives
+// every warp 16, at most 8 hits.  Doublet / link search in us with 32, 16, 8, 4 and 2 hits
+// at most: 64 pileup-200 events 1719 / 3576, 1631 / 3358, 1607 / 3315, 1661 / 3382,
+// 1854 / 3655; and for 2, 4, 8, 16 and 32 chunks per warp, 7 gap-pair events (217k hits)
+// 320 / 1498, 277 / 1096, 264 / 883, 269 / 753, 304 / 747.
+__device__ __forceinline__ uint32_t search_chunk(uint32_t n_sorted, uint32_t warps) {
+  return min(8u, max(1u, n_sorted / (16u * warps)));
+}
+
+// How much a search warp still has to do, as half of the hits after `done` over the hits
+// up to it: times what the warp has handed out so far, half of what it may still need.
+__device__ __forceinline__ float search_ahead(uint32_t n_sorted, uint32_t done) {
+  return done < n_sorted ? __fdividef(0.5f * (float)(n_sorted - done), (float)done) : 0.0f;
+}
+
+// Size of the chunk of slots that a warp takes for a request of n, having handed out
+// `total`: as much again up to `most`, but no more than it may still need.
+__device__ __forceinline__ uint32_t chunk_size(uint32_t n, uint32_t total, float ahead,
+                                               uint32_t most) {
+  return max(n, min(min(total, most), (uint32_t)fminf((float)total * ahead, (float)most)));
+}
+
+// Per-warp bump allocator over a global counter.  A warp that makes one request wastes
+// nothing; a busy warp takes a global atomic about once per kChunkMax slots instead of
+// once per request.  The unused tail of a chunk becomes a hole that the owner marks.  All
+// members are warp-uniform.
 struct WarpChunk {
   unsigned long long next = 0, end = 0;
-  uint32_t size = 0;
+  uint32_t total = 0;  // slots handed out
 };
-constexpr uint32_t kChunkMin = 32;
 constexpr uint32_t kChunkMax = 2048;
 
 // Reserves n contiguous slots; returns the first.  The caller marks [old next, old end)
 // as a hole when a new chunk is taken (reported through *hole_lo / *hole_hi).
 __device__ __forceinline__ unsigned long long chunk_take(WarpChunk& ch, unsigned long long* counter,
-                                                         uint32_t n, unsigned long long* hole_lo,
+                                                         uint32_t n, float ahead,
+                                                         unsigned long long* hole_lo,
                                                          unsigned long long* hole_hi) {
   *hole_lo = *hole_hi = 0;
   if (ch.next + n > ch.end) {
     *hole_lo = ch.next;
     *hole_hi = ch.end;
-    const uint32_t want = ch.size == 0 ? n : (n > ch.size ? n : ch.size);
-    ch.size = ch.size == 0 ? (n > kChunkMin ? n : kChunkMin) : min(2 * ch.size, kChunkMax);
+    const uint32_t want = chunk_size(n, ch.total, ahead, kChunkMax);
     unsigned long long base = 0;
     if ((threadIdx.x & 31) == 0) base = atomicAdd(counter, (unsigned long long)want);
     base = __shfl_sync(0xffffffffu, base, 0);
@@ -553,6 +576,7 @@ __device__ __forceinline__ unsigned long long chunk_take(WarpChunk& ch, unsigned
   }
   const unsigned long long r = ch.next;
   ch.next += n;
+  ch.total += n;
   return r;
 }
 

@@ -695,7 +695,7 @@ void reset_counters(pt_ctx* c, std::initializer_list<int> which) {
 }
 
 pt_status pt_build_doublets(pt_ctx* c, int64_t* n_cells) {
-  STAGE_BODY((reset_counters(c, {CNT_CELLS, CNT_CELLS_USED}),
+  STAGE_BODY((reset_counters(c, {CNT_CELLS, CNT_CELLS_USED, CNT_DBL_WORK}),
               launch_doublets(c->B, c->P, c->L, c->stream)),
              CNT_CELLS_USED, n_cells)
 }
@@ -703,14 +703,14 @@ pt_status pt_build_doublets(pt_ctx* c, int64_t* n_cells) {
 pt_status pt_connect_cells(pt_ctx* c, int64_t* n_links) {
   if (c) c->links_masked = c->masked();
   if (c && c->masked()) {
-    STAGE_BODY((reset_counters(c, {CNT_LINKS, CNT_LINKS_USED, CNT_GATE_KEPT}),
+    STAGE_BODY((reset_counters(c, {CNT_LINKS, CNT_LINKS_USED, CNT_GATE_KEPT, CNT_LNK_WORK}),
                 launch_connect(c->B, c->P, c->L, c->stream, c->gate_on),
                 c->gate_on ? launch_gate(c->B, c->P, c->L, c->gate, c->stream) : (void)0,
                 c->fishbone_on ? launch_fishbone(c->B, c->P, c->L, c->stream, c->gate_on)
                                : (void)0),
                CNT_GATE_KEPT, n_links)
   }
-  STAGE_BODY((reset_counters(c, {CNT_LINKS, CNT_LINKS_USED, CNT_GATE_KEPT}),
+  STAGE_BODY((reset_counters(c, {CNT_LINKS, CNT_LINKS_USED, CNT_GATE_KEPT, CNT_LNK_WORK}),
               launch_connect(c->B, c->P, c->L, c->stream)),
              CNT_LINKS_USED, n_links)
 }
