@@ -24,8 +24,13 @@ __global__ void k_clear(Buffers b, int32_t phi_bins) {
     b.layer_zmin[i] = 0xffffffffu;
     b.layer_zmax[i] = 0u;
   }
-  for (int i = t0; i <= N; i += stride) b.bucket_cnt[i] = 0;
-  for (int i = t0; i < N; i += stride) b.used[i] = 0;
+  if (b.nt_head) {  // a caller that stops at the doublets has no ntuplet arrays
+    for (int i = t0; i < N; i += stride) {
+      b.nt_head[i] = kHole;
+      b.used[i] = 0;
+    }
+    for (int i = t0; i <= N; i += stride) b.sv_cnt[i] = 0;
+  }
   if (t0 == 0) {
     b.cnt[CNT_CELLS] = 0;
     b.cnt[CNT_LINKS] = 0;
@@ -35,6 +40,8 @@ __global__ void k_clear(Buffers b, int32_t phi_bins) {
     b.cnt[CNT_GATE_KEPT] = 0;
     b.cnt[CNT_SCAN_NT] = 0;
     b.cnt[CNT_SV] = 0;
+    b.cnt[CNT_NT_BEST] = 0;
+    b.cnt[CNT_NT_TIES] = 0;
     b.cnt[CNT_CELLS_USED] = 0;
     b.cnt[CNT_LINKS_USED] = 0;
     b.cnt[CNT_DBL_WORK] = 0;

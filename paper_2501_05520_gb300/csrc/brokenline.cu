@@ -122,7 +122,7 @@ __device__ __forceinline__ void ldl_solve(double (&A)[M][M], double (&r)[M]) {
 __device__ __forceinline__ bool refit_pass(const Buffers& b, uint64_t j, double bfield,
                                            double x0b, double x0d, bool* more) {
   *more = false;
-  const uint32_t t = b.ord[b.sv[j]];
+  const uint32_t t = b.sv[j];
   const int n = b.nt_n[t];
   pt_track tr = b.tracks[j];
   if (n < 3 || n > kN) return false;

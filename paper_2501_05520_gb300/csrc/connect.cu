@@ -27,13 +27,13 @@
 // so the queue runs on across incoming groups and middle hits, and C1, C2 and C3 are
 // tested only once 32 pairs are waiting, all lanes busy (about six pairs fall in the
 // windows of a group of 32 incoming cells).  A link takes the next slot of the warp's
-// reservation and is pushed onto its source's out-link list (cell_head, link_next),
-// the list the ntuplet search walks; a cell's list head is cleared by the lane that
-// holds the cell before any of its pairs is queued.
+// reservation and is pushed onto its source's out-link list (CellState::head, Link::next),
+// the list the ntuplet search walks; a cell's state is set up by the lane that holds the
+// cell before any of its pairs is queued, and only then: three of four cells have no pair.
 //
 // The target cell (h1, h2) of a link is found afterwards, one thread per link, in h2's
-// incoming segment from h1's layer (ordered by inner hit) by binary search: in the
-// warp's own path those dependent loads would hold up the search.  A middle hit with
+// incoming segment from h1's layer (ordered by inner hit): in the warp's own path those
+// dependent loads would hold up the search.  A middle hit with
 // more outgoing cells than the stage holds is handled piece by piece, every incoming
 // group visiting every piece.
 #include "ptca_internal.cuh"
@@ -162,7 +162,6 @@ __device__ __forceinline__ unsigned long long chunk_take_shared(
   return r;
 }
 
-template <bool GATE>
 __global__ void __launch_bounds__(kConnWarps * 32, kConnBlocksPerSm)
     k_connect(Buffers b, pt_cuts cuts, PairTable pt, int32_t B, uint64_t cap_links) {
   __shared__ ConnWarp s_w[kConnWarps];
@@ -180,7 +179,7 @@ __global__ void __launch_bounds__(kConnWarps * 32, kConnBlocksPerSm)
   __syncwarp();
   auto mark_link_hole = [&](unsigned long long lo, unsigned long long hi) {
     hi = min(hi, (unsigned long long)cap_links);
-    for (unsigned long long i = lo + lane; i < hi; i += 32) b.link_src[i] = kHole;
+    for (unsigned long long i = lo + lane; i < hi; i += 32) b.link[i].src = kHole;
   };
   // C1, C2 and C3 on nt queued pairs, one per lane, all of them carrying what they need
   // (the source cell and the target's outer hit and slot), so that pairs of different
@@ -218,11 +217,8 @@ __global__ void __launch_bounds__(kConnWarps * 32, kConnBlocksPerSm)
       } else if (ok) {
         const uint64_t slot = base + __popc(pm & lt_mask);
         if (PT_CHECK(b.cnt, slot < cap_links, DBG_CON_LINK)) {
-          b.link_src[slot] = src;
-          b.link_dst[slot] = e.y;  // outer hit | slot << 29, made a cell id by k_link_targets
-          b.link_q[slot] = q;
-          b.link_next[slot] = atomicExch(&b.cell_head[src], (uint32_t)slot);
-          if (!GATE) b.has_out[src] = 1;  // gated form: the gate sets the flags of kept links
+          *link_hi(&b.link[slot]) = make_uint4(src, e.y, e.z, __float_as_uint(q));
+          b.link[slot].next = atomicExch(&b.cell[src].head, (uint32_t)slot);
         }
       }
     }
@@ -439,7 +435,7 @@ __global__ void __launch_bounds__(kConnWarps * 32, kConnBlocksPerSm)
         const float ua = cuts.rz0 + cuts.rz1 * fabsf(ta);
         const float shrink = 1.0f - cuts.rz1 * id1;
 
-        bool inited = false;  // the lane's cell had its out-link list cleared
+        bool inited = false;  // the lane's cell had its state set up
 #pragma unroll 1
         for (int piece = 0; piece < npieces; ++piece) {
           if (W.piece != piece) stage_piece(piece);
@@ -470,7 +466,8 @@ __global__ void __launch_bounds__(kConnWarps * 32, kConnBlocksPerSm)
                 const uint32_t st = W.perm[pos];
                 code = W.code[st];
                 if (!inited) {
-                  b.cell_head[c] = kHole;  // before any of its pairs is tested
+                  // before any of its pairs is tested: no links, no flags
+                  *(uint2*)&b.cell[c] = make_uint2(kHole, 0u);
                   inited = true;
                 }
               }
@@ -548,39 +545,46 @@ __device__ __forceinline__ uint32_t find_inner(const Buffers& b, uint32_t lo, ui
   return lo;
 }
 
-// The target cell (h1, h2) of every link: h1 (the outer hit of the source cell) in h2's
-// incoming segment from h1's layer, which is ordered by inner hit (find_inner);
-// one thread per link slot.  Plain form: the target's incoming-link flag is set and the
-// link records the target's out-link list head and outer hit.  Gated
-// form: the link's bf16 feature row for the gate's MLP is computed here, one thread per
-// link with every lane busy, from the three hits (mostly still in L2).  A
-// target can be missing only when the doublet stage ran out of cell slots (its status
-// bit is set then); the link then points back to its source, a valid cell, so that the
-// later stages stay within their arrays.
+// The target cell (h1, h2) of every link: h1 in h2's incoming segment from h1's layer,
+// which is ordered by inner hit (find_inner); one thread per link slot.  The link is
+// completed for the ntuplet walk.  The target has links of its own when the list head in
+// its state names a link that starts from it: a cell without links may hold anything
+// there, but no link then names it as its source.  Such a leaf gets its state here, named
+// by whichever of its in-links writes last.  The cleaning keys start here too.  Plain form: the flag of the target's incoming link is set (a leaf needs
+// none: only cells with links can be roots).  Gated form: the link's bf16 feature row for
+// the gate's MLP is computed, one thread per link with every lane busy, from the three
+// hits (mostly still in L2).  A target can be missing only when the doublet stage ran out
+// of cell slots (its status bit is set then); the link then points back to its source, a
+// valid cell, so that the later stages stay within their arrays.
+//
+// Bound by its random sectors.  64 pileup-200 events (5.3M links): 0.32 ms, against 0.27
+// when it left the walk's other fields and the cleaning keys to the stages that now read
+// or reduce them in one sector (A4 to A6 1.00 against 1.62 ms).
 template <bool GATE>
 __global__ void k_link_targets(Buffers b, pt_cuts cuts, int32_t B, int max_inner,
                                uint64_t cap_links) {
   const uint64_t nl = min(b.cnt[CNT_LINKS], (unsigned long long)cap_links);
   const uint64_t stride = (uint64_t)gridDim.x * blockDim.x;
   for (uint64_t l = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x; l < nl; l += stride) {
-    const uint32_t a = b.link_src[l];
+    const uint4 hi = *link_hi(&b.link[l]);
+    const uint32_t a = hi.x, t = hi.y, h1 = hi.z;
     if (a == kHole) continue;
-    const uint32_t t = b.link_dst[l];
-    const uint32_t h1 = b.cell_out[a];
+    const uint32_t next = b.link[l].next;
+    *(uint4*)&b.link_best[l] = make_uint4(~0u, ~0u, ~0u, ~0u);
     uint2 sg = b.seg[(uint64_t)(t & 0x1fffffffu) * max_inner + (t >> 29)];
     if (!PT_CHECK(b.cnt, (uint64_t)sg.x + sg.y <= b.cnt[CNT_CELLS], DBG_TGT_SEGMENT))
       sg = make_uint2(0u, 0u);
     bool found;
     const uint32_t pos = find_inner(b, sg.x, sg.x + sg.y, h1, found);
     const uint32_t c = found ? pos : a;
-    b.link_dst[l] = c;
-    if (!GATE) {
-      if (found) b.has_in[c] = 1;
-      // the target's list (complete: every link was pushed by the link kernel; kHole
-      // when the target has none) and outer hit, for the ntuplet walk
-      b.link_walk[l] = make_uint2(b.has_out[c] ? b.cell_head[c] : kHole,
-                                  found ? (t & 0x1fffffffu) : b.cell_out[c]);
+    uint32_t head = b.cell[c].head;
+    if (head >= nl || b.link[head].src != c) {
+      head = kHole;
+      *(uint2*)&b.cell[c] = make_uint2((uint32_t)l, 0u);
+    } else if (!GATE && found) {
+      b.cell[c].has_in = 1;
     }
+    *link_lo(&b.link[l]) = make_uint4(next, c, head, found ? (t & 0x1fffffffu) : h1);
     if (GATE) {
       const uint32_t h0 = b.cell_in[a], h2 = t & 0x1fffffffu;
       float f[kGateFeat];
@@ -595,21 +599,17 @@ __global__ void k_link_targets(Buffers b, pt_cuts cuts, int32_t B, int max_inner
 
 void launch_connect(const Buffers& b, const Params& p, const Launch& l, cudaStream_t s,
                     bool gated) {
-  if (gated) {
-    PT_TRACE(l, s, "k_connect",
-             k_connect<true><<<l.sms * kConnBlocksPerSm, kConnWarps * 32, 0, s>>>(
-                 b, p.cuts, p.pairs, p.phi_bins, (uint64_t)p.max_links));
+  PT_TRACE(l, s, "k_connect",
+           k_connect<<<l.sms * kConnBlocksPerSm, kConnWarps * 32, 0, s>>>(
+               b, p.cuts, p.pairs, p.phi_bins, (uint64_t)p.max_links));
+  if (gated)
     PT_TRACE(l, s, "k_link_targets",
              k_link_targets<true><<<l.grid, 256, 0, s>>>(b, p.cuts, p.phi_bins, p.pairs.max_inner,
                                                          (uint64_t)p.max_links));
-  } else {
-    PT_TRACE(l, s, "k_connect",
-             k_connect<false><<<l.sms * kConnBlocksPerSm, kConnWarps * 32, 0, s>>>(
-                 b, p.cuts, p.pairs, p.phi_bins, (uint64_t)p.max_links));
+  else
     PT_TRACE(l, s, "k_link_targets",
              k_link_targets<false><<<l.grid, 256, 0, s>>>(b, p.cuts, p.phi_bins, p.pairs.max_inner,
                                                           (uint64_t)p.max_links));
-  }
 }
 
 }  // namespace ptca

@@ -18,7 +18,9 @@
 // increasing index order.  Lanes stride over it, test the exact float32 cuts and stage
 // the passing inner hits in shared memory; the segment is then appended with one
 // reservation per (hit, inner slot).  Slots are reserved through a per-warp chunk
-// allocator; unused slots are marked as holes.
+// allocator; a slot that no segment covers is a hole.  A cell is written as its inner hit
+// alone (4 bytes): the segment names its outer hit, and its link state starts with its
+// first link.
 #include "ptca_internal.cuh"
 
 namespace ptca {
@@ -28,14 +30,6 @@ namespace {
 constexpr float kTwoPi = 6.28318530717958647692f;
 constexpr float kHalfPi = 1.57079632679489661923f;
 constexpr int kWarpsPerBlock = 8;
-
-// Writes one cell; its two link flags start cleared.
-__device__ __forceinline__ void write_cell(const Buffers& b, uint64_t c, uint32_t in, uint32_t out) {
-  b.cell_in[c] = in;
-  b.cell_out[c] = out;
-  b.has_in[c] = 0;
-  b.has_out[c] = 0;
-}
 
 // Azimuthal window of outer hit `ho` (global bin gb, asin_o = asin(kmax*ro/2), +inf where
 // kmax*ro/2 >= 0.7) towards inner slot k: up to two ranges [r.x, r.y) and [r.z, r.w) of
@@ -103,10 +97,6 @@ __global__ void __launch_bounds__(kWarpsPerBlock * 32, 5)
   const uint32_t n_sorted = b.bin_start[E * kLayers * B];
   const float bins_per_rad = (float)B / kTwoPi;
   WarpChunk ch;
-  auto mark_hole = [&](unsigned long long lo, unsigned long long hi) {
-    hi = min(hi, (unsigned long long)cap_cells);
-    for (unsigned long long i = lo + lane; i < hi; i += 32) b.cell_out[i] = kHole;
-  };
 
   const uint32_t n_warps = gridDim.x * kWarpsPerBlock;
   const uint32_t per = search_chunk(n_sorted, n_warps);
@@ -172,18 +162,15 @@ __global__ void __launch_bounds__(kWarpsPerBlock * 32, 5)
 
         uint32_t seg_off = 0, seg_cnt = 0;
         if (cnt > 0) {
-          unsigned long long hlo, hhi;
-          const unsigned long long base = chunk_take(ch, &b.cnt[CNT_CELLS], cnt,
-                                                     search_ahead(n_sorted, s + 1), &hlo, &hhi);
-          mark_hole(hlo, hhi);
+          const unsigned long long base =
+              chunk_take(ch, &b.cnt[CNT_CELLS], cnt, search_ahead(n_sorted, s + 1));
           if (base + cnt > cap_cells) {
             if (lane == 0) atomicOr(&b.cnt[CNT_STATUS], ST_CELLS);
-            mark_hole(base, base + cnt);  // slots below the capacity stay readable
           } else if (cnt <= (uint32_t)kStage) {
             __syncwarp();
             for (uint32_t i = lane; i < cnt; i += 32)
               if (PT_CHECK(b.cnt, base + i < cap_cells, DBG_DBL_CELL))
-                write_cell(b, base + i, sval[i], s);
+                b.cell_in[base + i] = sval[i];
             seg_off = (uint32_t)base;
             seg_cnt = cnt;
           } else {
@@ -197,7 +184,7 @@ __global__ void __launch_bounds__(kWarpsPerBlock * 32, 5)
                 const unsigned bal = __ballot_sync(kFull, pass);
                 if (pass && PT_CHECK(b.cnt, base + pos0 + __popc(bal & lt_mask) < cap_cells,
                                      DBG_DBL_CELL))
-                  write_cell(b, base + pos0 + __popc(bal & lt_mask), i, s);
+                  b.cell_in[base + pos0 + __popc(bal & lt_mask)] = i;
                 pos0 += __popc(bal);
               }
             }
@@ -212,7 +199,6 @@ __global__ void __launch_bounds__(kWarpsPerBlock * 32, 5)
     if (lane == 0) chunk = n_warps + (uint32_t)atomicAdd(&b.cnt[CNT_DBL_WORK], 1ull);
     chunk = __shfl_sync(kFull, chunk, 0);
   }
-  mark_hole(ch.next, ch.end);
   if (lane == 0 && ch.total) atomicAdd(&b.cnt[CNT_CELLS_USED], (unsigned long long)ch.total);
 }
 

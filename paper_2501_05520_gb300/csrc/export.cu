@@ -15,17 +15,16 @@ __device__ __forceinline__ void to_local(const Buffers& b, int E, const int32_t*
   *ev = e;
 }
 
+// Cleaned ntuplets (the stage path; the whole-batch graph's cleaning writes them itself).
 __global__ void k_export_ntuplets(Buffers b) {
   const uint64_t S = b.cnt[CNT_SV];
   const int E = b.hdr->n_events;
   const uint64_t stride = (uint64_t)gridDim.x * blockDim.x;
   for (uint64_t j = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x; j < S; j += stride) {
-    const uint32_t t = b.ord[b.sv[j]];
+    const uint32_t t = b.sv[j];
     int32_t ev;
     to_local(b, E, b.nt_hits + (uint64_t)t * kMaxHits, b.exp_hits + j * kMaxHits, &ev);
     b.exp_n[j] = b.nt_n[t];
-    b.exp_q[j] = b.nt_q[t];
-    b.exp_ev[j] = ev;
   }
 }
 
@@ -37,25 +36,32 @@ __global__ void k_export_candidates(Buffers b) {
     int32_t ev;
     to_local(b, E, b.nt_hits + t * kMaxHits, b.exp_hits + t * kMaxHits, &ev);
     b.exp_n[t] = b.nt_n[t];
-    b.exp_q[t] = b.nt_q[t];
+    b.exp_q[t] = fabsf(b.nt_q[t]);
     b.exp_ev[t] = ev;
   }
 }
 
-__global__ void k_export_cells(Buffers b, uint64_t cap_cells, int32_t* out3) {
+// One warp per sorted hit: the cells of its incoming segments, at their own slots (the
+// caller has marked every slot a hole).
+__global__ void k_export_cells(Buffers b, int32_t B, int max_inner, uint64_t cap_cells,
+                               int32_t* out3) {
   const uint64_t nc = min(b.cnt[CNT_CELLS], (unsigned long long)cap_cells);
   const int E = b.hdr->n_events;
-  const uint64_t stride = (uint64_t)gridDim.x * blockDim.x;
-  for (uint64_t c = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x; c < nc; c += stride) {
-    if (b.cell_out[c] == kHole) {
-      out3[c * 3 + 0] = out3[c * 3 + 1] = out3[c * 3 + 2] = -1;
-      continue;
+  const uint32_t n_sorted = b.bin_start[E * kLayers * B];
+  const uint32_t nw = gridDim.x * (blockDim.x >> 5);
+  for (uint32_t s = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5); s < n_sorted; s += nw) {
+    const int32_t go = (int32_t)b.perm[s];
+    const int e = find_event(b.hit_off, E, go);
+    for (int k = 0; k < max_inner; ++k) {
+      const uint2 sg = b.seg[(uint64_t)s * max_inner + k];
+      for (uint32_t i = lane_id(); i < sg.y; i += 32) {
+        const uint64_t c = (uint64_t)sg.x + i;
+        if (c >= nc) break;
+        out3[c * 3 + 0] = (int32_t)b.perm[b.cell_in[c]] - b.hit_off[e];
+        out3[c * 3 + 1] = go - b.hit_off[e];
+        out3[c * 3 + 2] = e;
+      }
     }
-    const int32_t gi = (int32_t)b.perm[b.cell_in[c]], go = (int32_t)b.perm[b.cell_out[c]];
-    const int e = find_event(b.hit_off, E, gi);
-    out3[c * 3 + 0] = gi - b.hit_off[e];
-    out3[c * 3 + 1] = go - b.hit_off[e];
-    out3[c * 3 + 2] = e;
   }
 }
 
@@ -65,17 +71,17 @@ __global__ void k_export_links(Buffers b, uint64_t cap_links, int32_t* out4, flo
   const int E = b.hdr->n_events;
   const uint64_t stride = (uint64_t)gridDim.x * blockDim.x;
   for (uint64_t l = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x; l < nl; l += stride) {
-    const uint32_t a = b.link_src[l];
-    if (a == kHole || (gated && !b.gate_keep[l])) continue;  // hole or removed link
-    const int32_t g0 = (int32_t)b.perm[b.cell_in[a]], g1 = (int32_t)b.perm[b.cell_out[a]];
-    const int32_t g2 = (int32_t)b.perm[b.cell_out[b.link_dst[l]]];
+    const Link k = b.link[l];
+    if (k.src == kHole || (gated && !b.gate_keep[l])) continue;  // hole or removed link
+    const int32_t g0 = (int32_t)b.perm[b.cell_in[k.src]], g1 = (int32_t)b.perm[k.h1];
+    const int32_t g2 = (int32_t)b.perm[k.h2];
     const int e = find_event(b.hit_off, E, g0);
     const int32_t off = b.hit_off[e];
     out4[l * 4 + 0] = g0 - off;
     out4[l * 4 + 1] = g1 - off;
     out4[l * 4 + 2] = g2 - off;
     out4[l * 4 + 3] = e;
-    outq[l] = b.link_q[l];
+    outq[l] = k.q;
   }
 }
 
@@ -89,7 +95,8 @@ void launch_export_candidates(const Buffers& b, const Launch& l, cudaStream_t s)
 }
 void launch_export_cells(const Buffers& b, const Params& p, const Launch& l, int32_t* out3,
                          cudaStream_t s) {
-  k_export_cells<<<l.grid, 256, 0, s>>>(b, (uint64_t)p.max_cells, out3);
+  k_export_cells<<<l.grid, 256, 0, s>>>(b, p.phi_bins, p.pairs.max_inner, (uint64_t)p.max_cells,
+                                        out3);
 }
 void launch_export_links(const Buffers& b, const Params& p, const Launch& l, int32_t* out4,
                          float* outq, cudaStream_t s, bool gated) {

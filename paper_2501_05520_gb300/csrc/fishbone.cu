@@ -21,8 +21,8 @@
 // stands for its source.  They are grouped by outer
 // hit with a counting sort (k_fb_count, a scan, k_fb_scatter, which also writes each
 // cell's comparison record), and k_fb_compare takes one active cell per thread and
-// compares it with the other records of its group.  The removal
-// flags are zeroed for every cell first and set only for the removed ones.
+// compares it with the other records of its group.  The removal flags are part of the
+// cells' states, which the link stage and its target pass leave cleared.
 // k_fb_filter_clear / k_fb_filter_set: one thread per link slot; the keep mask of the
 //   ntuplet search becomes (gate keep, if any) and neither end removed, and the link
 //   flags of the ntuplet search are rebuilt from the kept links (cleared for every end
@@ -42,7 +42,7 @@ struct alignas(16) FbCell {
   uint32_t key;   // input index of the inner hit
   uint32_t lay;   // layer of the inner hit
   float sensor;   // the inner hit's radius (barrel) or |z| (disk)
-  uint32_t cell;  // the cell
+  uint32_t link;  // the link slot that heads the cell's out-link list
 };
 static_assert(sizeof(FbCell) == 32, "two float4 per record");
 
@@ -56,7 +56,8 @@ __device__ __forceinline__ bool fb_loses(const FbCell& a, const FbCell& c) {
   return a.lay == c.lay ? a.u.w < c.u.w : a.u.w > c.u.w;
 }
 
-__device__ __forceinline__ FbCell fb_cell(const Buffers& b, float4 ph, uint32_t c, int32_t B) {
+__device__ __forceinline__ FbCell fb_cell(const Buffers& b, float4 ph, uint32_t c, uint32_t l,
+                                          int32_t B) {
   const uint32_t hi = b.cell_in[c];
   const float4 pi = b.hit4[hi];
   FbCell f;
@@ -67,24 +68,27 @@ __device__ __forceinline__ FbCell fb_cell(const Buffers& b, float4 ph, uint32_t 
   f.key = b.perm[hi];
   f.lay = (b.hbin[hi] / (uint32_t)B) % kLayers;
   f.sensor = f.lay < 4 ? pi.w : fabsf(pi.z);
-  f.cell = c;
+  f.link = l;
   return f;
 }
 
-// The source of link slot l when l heads an active source's out-link list, else kHole.
-__device__ __forceinline__ uint32_t run_source(const Buffers& b, uint64_t l, bool gated) {
-  const uint32_t a = b.link_src[l];
-  if (a == kHole || b.cell_head[a] != (uint32_t)l) return kHole;
-  if (gated && !b.has_out[a]) return kHole;  // no link of the run passed the gate
-  return a;
+// The source of link slot l when l heads an active source's out-link list, else kHole;
+// h: its outer hit.
+__device__ __forceinline__ uint32_t run_source(const Buffers& b, uint64_t l, bool gated,
+                                               uint32_t& h) {
+  const uint4 hi = *link_hi(&b.link[l]);
+  h = hi.z;
+  if (hi.x == kHole || b.cell[hi.x].head != (uint32_t)l) return kHole;
+  if (gated && !b.cell[hi.x].has_out) return kHole;  // no link of the run passed the gate
+  return hi.x;
 }
 
 __global__ void k_fb_count(Buffers b, uint64_t cap_links, bool gated) {
   const uint64_t nl = min(b.cnt[CNT_LINKS], (unsigned long long)cap_links);
   const uint64_t stride = (uint64_t)gridDim.x * blockDim.x;
   for (uint64_t l = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x; l < nl; l += stride) {
-    const uint32_t a = run_source(b, l, gated);
-    if (a != kHole) atomicAdd(&b.fb_cnt[b.cell_out[a]], 1u);
+    uint32_t h;
+    if (run_source(b, l, gated, h) != kHole) atomicAdd(&b.fb_cnt[h], 1u);
   }
 }
 
@@ -92,12 +96,12 @@ __global__ void k_fb_scatter(Buffers b, int32_t B, uint64_t cap_links, bool gate
   const uint64_t nl = min(b.cnt[CNT_LINKS], (unsigned long long)cap_links);
   const uint64_t stride = (uint64_t)gridDim.x * blockDim.x;
   for (uint64_t l = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x; l < nl; l += stride) {
-    const uint32_t a = run_source(b, l, gated);
+    uint32_t h;
+    const uint32_t a = run_source(b, l, gated, h);
     if (a == kHole) continue;
-    const uint32_t h = b.cell_out[a];
     const uint32_t pos = b.fb_start[h] + atomicSub(&b.fb_cnt[h], 1u) - 1u;
     if (!PT_CHECK(b.cnt, pos < cap_links, DBG_FB_RECORD)) continue;
-    reinterpret_cast<FbCell*>(b.fb_rec)[pos] = fb_cell(b, b.hit4[h], a, B);
+    reinterpret_cast<FbCell*>(b.fb_rec)[pos] = fb_cell(b, b.hit4[h], a, (uint32_t)l, B);
   }
 }
 
@@ -109,12 +113,12 @@ __global__ void k_fb_compare(Buffers b) {
   const FbCell* rec = reinterpret_cast<const FbCell*>(b.fb_rec);
   for (uint32_t p = blockIdx.x * blockDim.x + threadIdx.x; p < n_act; p += stride) {
     const FbCell ca = rec[p];
-    const uint32_t h = b.cell_out[ca.cell];
+    const uint32_t h = b.link[ca.link].h1;
     const uint32_t g0 = b.fb_start[h], g1 = b.fb_start[h + 1];
     bool lose = false;
     for (uint32_t q = g0; q < g1 && !lose; ++q)
       if (q != p) lose = fb_loses(ca, rec[q]);
-    if (lose) b.fb_kill[ca.cell] = 1;
+    if (lose) b.cell[b.link[ca.link].src].kill = 1;
   }
 }
 
@@ -125,13 +129,13 @@ __global__ void k_fb_filter_clear(Buffers b, uint64_t cap_links, bool gated) {
   const uint64_t stride = (uint64_t)gridDim.x * blockDim.x;
   uint32_t kept = 0;
   for (uint64_t l = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x; l < nl; l += stride) {
-    const uint32_t a = b.link_src[l];
+    const uint32_t a = b.link[l].src;
     bool k = false;
     if (a != kHole) {
-      const uint32_t d = b.link_dst[l];
-      k = (!gated || b.gate_keep[l]) && !b.fb_kill[a] && !b.fb_kill[d];
-      b.has_out[a] = 0;
-      b.has_in[d] = 0;
+      const uint32_t d = b.link[l].dst;
+      k = (!gated || b.gate_keep[l]) && !b.cell[a].kill && !b.cell[d].kill;
+      b.cell[a].has_out = 0;
+      b.cell[d].has_in = 0;
     }
     b.gate_keep[l] = k ? 1 : 0;
     kept += k ? 1u : 0u;
@@ -146,8 +150,8 @@ __global__ void k_fb_filter_set(Buffers b, uint64_t cap_links) {
   const uint64_t stride = (uint64_t)gridDim.x * blockDim.x;
   for (uint64_t l = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x; l < nl; l += stride) {
     if (!b.gate_keep[l]) continue;
-    b.has_out[b.link_src[l]] = 1;
-    b.has_in[b.link_dst[l]] = 1;
+    b.cell[b.link[l].src].has_out = 1;
+    b.cell[b.link[l].dst].has_in = 1;
   }
 }
 
@@ -156,7 +160,6 @@ __global__ void k_fb_filter_set(Buffers b, uint64_t cap_links) {
 void launch_fishbone(const Buffers& b, const Params& p, const Launch& l, cudaStream_t s,
                      bool gated) {
   cudaMemsetAsync(&b.cnt[CNT_GATE_KEPT], 0, sizeof(unsigned long long), s);  // recounted
-  cudaMemsetAsync(b.fb_kill, 0, (size_t)p.max_cells, s);
   cudaMemsetAsync(b.fb_cnt, 0, (size_t)(p.max_hits + 1) * 4, s);
   PT_TRACE(l, s, "k_fb_count",
            k_fb_count<<<l.grid, 256, 0, s>>>(b, (uint64_t)p.max_links, gated));

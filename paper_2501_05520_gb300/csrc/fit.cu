@@ -76,7 +76,7 @@ __global__ void __launch_bounds__(256) k_fit(Buffers b, float bfield) {
     float x = 0.0f, y = 0.0f, z = 0.0f;
     uint32_t t = 0;
     if (active) {
-      t = b.ord[b.sv[j]];
+      t = b.sv[j];
       n = b.nt_n[t];
       if (!PT_CHECK(b.cnt, n >= 3 && n <= kMaxHits, DBG_FIT_HITS)) n = 3;
       if (sub < n) {

@@ -190,7 +190,7 @@ __global__ void __launch_bounds__(kTileM, kMlpCtasPerSm)
     src = kHole;
     if (tt >= n_tiles || r >= n) return;
     if (PIPE) {
-      src = b.link_src[r];
+      src = b.link[r].src;
       if (src == kHole) return;
     }
     const uint4* srcp = (const uint4*)((PIPE ? b.gate_x : X) + r * kGateK1);
@@ -277,8 +277,8 @@ __global__ void __launch_bounds__(kTileM, kMlpCtasPerSm)
         if (src_cell == kHole) {
           kp = false;
         } else if (kp) {
-          b.has_in[b.link_dst[row]] = 1;
-          b.has_out[src_cell] = 1;
+          b.cell[b.link[row].dst].has_in = 1;
+          b.cell[src_cell].has_out = 1;
         }
       }
       score[row] = acc;
@@ -311,15 +311,14 @@ __global__ void k_gate_features_f32(Buffers b, pt_cuts cuts, int32_t B, uint64_t
   const uint64_t nl = min(b.cnt[CNT_LINKS], (unsigned long long)cap_links);
   const uint64_t stride = (uint64_t)gridDim.x * blockDim.x;
   for (uint64_t l = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x; l < nl; l += stride) {
-    const uint32_t a = b.link_src[l];
-    if (a == kHole || (gated && !b.gate_keep[l])) continue;
-    const uint32_t h0 = b.cell_in[a], h1 = b.cell_out[a];
-    const uint32_t h2 = b.cell_out[b.link_dst[l]];
+    const Link k = b.link[l];
+    if (k.src == kHole || (gated && !b.gate_keep[l])) continue;
+    const uint32_t h0 = b.cell_in[k.src], h1 = k.h1, h2 = k.h2;
     float f[kGateFeat];
     gate_link_features(cuts, b.hit4[h0], b.hit4[h1], b.hit4[h2], (b.hbin[h0] / B) % kLayers,
                        (b.hbin[h1] / B) % kLayers, (b.hbin[h2] / B) % kLayers, f);
 #pragma unroll
-    for (int k = 0; k < kGateFeat; ++k) out[l * kGateFeat + k] = f[k];
+    for (int i = 0; i < kGateFeat; ++i) out[l * kGateFeat + i] = f[i];
   }
 }
 

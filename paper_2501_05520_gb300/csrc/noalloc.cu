@@ -20,8 +20,7 @@ constexpr size_t kNaNb = (size_t)kLayers * kNaBins + 1;
 // Bytes of each scratch buffer, in the order na_layout carves them.
 enum NaPart {
   NA_HDR, NA_CNT, NA_OFF, NA_IN_BIN, NA_IN_RANK, NA_HIT4, NA_PERM, NA_HBIN, NA_BIN_CNT,
-  NA_BIN_START, NA_RMAX, NA_ASIN, NA_RMIN, NA_ASIN_LO, NA_ZMIN, NA_ZMAX, NA_BUCKET_CNT, NA_USED,
-  NA_SCAN,
+  NA_BIN_START, NA_RMAX, NA_ASIN, NA_RMIN, NA_ASIN_LO, NA_ZMIN, NA_ZMAX, NA_SCAN,
   NA_PARTS
 };
 constexpr size_t kNaPart[NA_PARTS] = {
@@ -31,7 +30,6 @@ constexpr size_t kNaPart[NA_PARTS] = {
     kNaNb * 4, kNaNb * 4, kLayers * 4, kLayers * 4,          // bins, layer r max, layer asin
     kLayers * 4, kLayers * 4,                                // layer r min, its asin
     kLayers * 4, kLayers * 4,                                // layer z min, max
-    (kNaMaxHits + 1) * 4, kNaMaxHits,                        // cleared: bucket, used
     (kScanBlocks + 1) * 4};                                  // scan partials
 constexpr size_t na_offset(int part) {
   size_t off = 0;
@@ -64,8 +62,6 @@ Buffers na_layout(char* base, const float* x, const float* y, const float* z,
   b.layer_asin_lo = (float*)at(NA_ASIN_LO);
   b.layer_zmin = (uint32_t*)at(NA_ZMIN);
   b.layer_zmax = (uint32_t*)at(NA_ZMAX);
-  b.bucket_cnt = (uint32_t*)at(NA_BUCKET_CNT);
-  b.used = (uint8_t*)at(NA_USED);
   b.scan_part = (uint32_t*)at(NA_SCAN);
   b.in_x = (float*)x;
   b.in_y = (float*)y;

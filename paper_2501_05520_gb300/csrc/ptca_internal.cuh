@@ -33,7 +33,7 @@ enum : int {
   CNT_STATUS = 3,
   CNT_SCAN_BINS = 4,  // sizes for the device-wide scans
   CNT_SCAN_HITS = 5,
-  CNT_SCAN_NT = 6,
+  CNT_SCAN_NT = 6,    // ntuplets before cleaning that were stored
   CNT_GATE_KEPT = 7,
   CNT_SV = 8,         // cleaned ntuplets
   CNT_SCORE_STATUS = 9,  // status bits of the standalone gate scoring (pt_gate_score)
@@ -48,7 +48,9 @@ enum : int {
   CNT_RAW_HITS = 18,    // raw input: hits made from the digis
   CNT_RAW_BIG = 19,     // raw input: long module runs listed for the block-per-run launch
   CNT_LNK_WORK = 20,    // link search: next chunk of sorted middle hits
+  CNT_NT_BEST = 21,     // ntuplets on best_list
   CNT_DEBUG_SITE = 22,  // debug build: the first failing bounds check (DebugSite)
+  CNT_NT_TIES = 23,     // nonzero: ntuplets of the same hit count and q met in a cell
   CNT_N = 24
 };
 // raw-input status bits (cnt[CNT_RAW_STATUS])
@@ -100,6 +102,44 @@ struct GateWeights {
   float w3[kGateHidden];
   float b3;
   float tau;
+};
+
+// Link state of a cell, one record because the later stages reach the cells at random (161M
+// cells on 64 pileup-200 events, one of 16 on a link).  Written for the cells that take part
+// in links only: the link stage sets up its sources, the target pass the targets without
+// links of their own (leaves).
+struct alignas(8) CellState {
+  uint32_t head;    // a source's latest out-link slot, the head of its out-link list (kHole:
+                    //   no link passed); a leaf: one of the links that end on it
+  uint8_t has_in;   // a link ends on the cell (masked forms: a kept link; sources only)
+  uint8_t has_out;  // masked forms: a kept link starts from the cell
+  uint8_t kill;     // removed by the fishbone step
+  uint8_t pad;
+};
+static_assert(sizeof(CellState) == 8, "one 8-byte record");
+
+// A link in one memory sector, all that a step of the ntuplet walk needs.  The link stage
+// writes `next` and the second half, the target pass the rest.
+struct alignas(32) Link {
+  uint32_t next;  // the source's next out-link slot (kHole: last)
+  uint32_t dst;   // target cell
+  uint32_t head;  // the target's out-link list head (kHole: a leaf)
+  uint32_t h2;    // the target's outer hit (sorted index)
+  uint32_t src;   // source cell (kHole: an unused slot)
+  uint32_t code;  // the target before the target pass: outer hit | slot << 29
+  uint32_t h1;    // middle hit (sorted index)
+  float q;        // link quality
+};
+static_assert(sizeof(Link) == 32, "one memory sector");
+__device__ __forceinline__ uint4* link_lo(Link* l) { return (uint4*)l; }
+__device__ __forceinline__ uint4* link_hi(Link* l) { return (uint4*)l + 1; }
+
+// Duplicate-cleaning keys.  A cell of an ntuplet is named by a link slot, a source by its
+// list's head and a leaf by the in-link in its state, so the keys lie in 16 bytes per link
+// (85 MB on 64 pileup-200 events, which stays in L2) instead of among all cells (2.6 GB).
+// Reading them back (k_dedup_best) takes 0.13 instead of 0.38 ms.
+struct alignas(16) LinkBest {
+  unsigned long long src, leaf;  // of the source headed by the slot, of the leaf named by it
 };
 
 struct BatchHeader {
@@ -171,42 +211,35 @@ struct Buffers {
   // max_inner slots per hit, all written
   uint2* seg;                // [max_hits*kMaxInner]
   // cells
-  uint32_t* cell_in;         // [max_cells] sorted hit index
-  uint32_t* cell_out;        // [max_cells]
-  uint8_t* has_in;           // [max_cells] an accepted link ends on the cell
-  uint8_t* has_out;          // [max_cells] an accepted link starts from the cell
-  uint8_t* fb_kill;          // [max_cells] removed by the fishbone step (zeroed for every
-                             //   cell when the step runs)
-  uint32_t* fb_cnt;          // [max_hits + 1] fishbone: active cells per outer hit
-  uint32_t* fb_start;        // [max_hits + 1]   and their first position in fb_list
+  uint32_t* cell_in;         // [max_cells] inner hit (sorted index); the outer hit is the
+                             //   one whose segment holds the cell
+  CellState* cell;           // [max_cells] cells that take part in links
+  uint32_t* fb_cnt;          // [max_hits + 1] fishbone: active cells per outer hit (all zero
+                             //   again after the step)
+  uint32_t* fb_start;        // [max_hits + 1]   and their first position in fb_rec
   float4* fb_rec;            // [max_links * 2] active cells grouped by outer hit: vector to
-                             //   the hit and |.|^2; cell, inner hit's input index, layer, sensor
-  uint32_t* cell_head;       // [max_cells] the cell's latest out-link slot, the head of
-                             //   its out-link list (valid where it has links)
-  unsigned long long* best;  // [max_cells] duplicate-cleaning key (cells on ntuplets)
-  // links
-  uint32_t* link_dst;        // [max_links]
-  uint32_t* link_next;       // [max_links] the source's next out-link slot (kHole: last)
-  uint2* link_walk;          // [max_links] plain form: the target cell's out-link list head
-                             //   (kHole: a leaf) and its outer hit (sorted index), written
-                             //   with the target so that the ntuplet walk reads each step
-                             //   from the link alone
-  float* link_q;             // [max_links]
+                             //   the hit and |.|^2; list head, inner hit's input index,
+                             //   layer, sensor (the memory of gate_x, free by then)
+  Link* link;                // [max_links]
+  LinkBest* link_best;       // [max_links]
   // ntuplets before cleaning
   int32_t* nt_hits;          // [max_ntuplets*6] batch input index, -1 pad
-  uint32_t* nt_cells;        // [max_ntuplets*5]
+  uint32_t* nt_cells;        // [max_ntuplets*5] link slots naming the cells (LinkBest), kHole
+                             //   padded; the last one names a leaf, or a source where nt_q
+                             //   is negative (masked forms: none of its links was kept)
   uint8_t* nt_n;             // [max_ntuplets]
-  float* nt_q;               // [max_ntuplets]
-  uint32_t* nt_rank;         // [max_ntuplets] rank within its first-hit bucket, then (after
-                             //   the canonical sort) its sorted position
-  // canonical order
-  uint32_t* bucket_cnt;      // [max_hits + 1]
-  uint32_t* bucket_start;    // [max_hits + 1]
-  uint32_t* ord;             // [max_ntuplets] sorted position -> ntuplet
-  uint32_t* alive;           // [max_ntuplets]
-  uint32_t* alive_scan;      // [max_ntuplets + 1]
-  uint8_t* used;             // [max_hits]
-  uint32_t* sv;              // [max_ntuplets] survivor -> sorted position
+  float* nt_q;               // [max_ntuplets] quality q >= 0, or -q (see nt_cells)
+  uint32_t* nt_next;         // [max_ntuplets] next survivor with the same first hit (kHole:
+                             //   none)
+  // duplicate cleaning and canonical order (hits are batch input indices here)
+  uint32_t* nt_head;         // [max_hits] list of the survivors that start at the hit (kHole:
+                             //   none)
+  uint32_t* sv_cnt;          // [max_hits + 1] surviving ntuplets that start at the hit (the
+                             //   memory of fb_cnt)
+  uint32_t* sv_start;        // [max_hits + 1]   and the first one's place
+  uint32_t* best_list;       // [max_ntuplets] ntuplets that may survive (kHole: it did not)
+  uint8_t* used;             // [max_hits] on a surviving ntuplet of four or more hits
+  uint32_t* sv;              // [max_ntuplets] cleaned ntuplets in canonical order
   int64_t* ev_nt_off;        // [max_events + 1]
   pt_track* tracks;          // [max_ntuplets]
   // primary vertices (pt_find_vertices)
@@ -220,8 +253,6 @@ struct Buffers {
   uint16_t* gate_x;          // [max_links*16] bf16 features per link slot (12 used)
   float* gate_score;         // [max_links] logit per link slot
   uint8_t* gate_keep;        // [max_links] 1 where the link passes the gate
-  uint32_t* link_src;        // [max_links] source cell of each link slot, kHole for unused
-                             //   slots
   int32_t* exp_hits;         // [max_ntuplets*6] export staging (event-local indices)
   uint8_t* exp_n;            // [max_ntuplets]
   float* exp_q;              // [max_ntuplets]
@@ -297,8 +328,14 @@ void launch_fishbone(const Buffers& b, const Params& p, const Launch& l, cudaStr
                      bool gated);
 // Debug build: records a failure of bounds check `site` as a failing check does.
 cudaError_t launch_debug_inject(const Buffers& b, unsigned site, cudaStream_t s);
+// Ntuplet search, cleaning and order; gated: the search follows the keep mask.  The first
+// form is the whole-batch graph's (the cells' cleaning keys and the lists must be as the
+// link stage and launch_clear leave them; the ntuplets go to the export staging too), the
+// second the stage call's, which may run again on the same links.
 void launch_ntuplets(const Buffers& b, const Params& p, const Launch& l, cudaStream_t s,
-                     bool gated = false);
+                     bool gated);
+void launch_ntuplet_steps(const Buffers& b, const Params& p, const Launch& l, cudaStream_t s,
+                          bool gated);
 void launch_fit(const Buffers& b, const Params& p, const Launch& l, cudaStream_t s);
 // raw digis -> hits in the chain's input arrays, per-event offsets and header
 cudaError_t launch_raw(const RawBuffers& r, const Buffers& b, const pt_module* mods, int n_mod,
@@ -549,24 +586,18 @@ __device__ __forceinline__ uint32_t chunk_size(uint32_t n, uint32_t total, float
 
 // Per-warp bump allocator over a global counter.  A warp that makes one request wastes
 // nothing; a busy warp takes a global atomic about once per kChunkMax slots instead of
-// once per request.  The unused tail of a chunk becomes a hole that the owner marks.  All
-// members are warp-uniform.
+// once per request.  The unused tail of a chunk becomes a hole.  All members are
+// warp-uniform.
 struct WarpChunk {
   unsigned long long next = 0, end = 0;
   uint32_t total = 0;  // slots handed out
 };
 constexpr uint32_t kChunkMax = 2048;
 
-// Reserves n contiguous slots; returns the first.  The caller marks [old next, old end)
-// as a hole when a new chunk is taken (reported through *hole_lo / *hole_hi).
+// Reserves n contiguous slots; returns the first.
 __device__ __forceinline__ unsigned long long chunk_take(WarpChunk& ch, unsigned long long* counter,
-                                                         uint32_t n, float ahead,
-                                                         unsigned long long* hole_lo,
-                                                         unsigned long long* hole_hi) {
-  *hole_lo = *hole_hi = 0;
+                                                         uint32_t n, float ahead) {
   if (ch.next + n > ch.end) {
-    *hole_lo = ch.next;
-    *hole_hi = ch.end;
     const uint32_t want = chunk_size(n, ch.total, ahead, kChunkMax);
     unsigned long long base = 0;
     if ((threadIdx.x & 31) == 0) base = atomicAdd(counter, (unsigned long long)want);

@@ -182,29 +182,20 @@ size_t layout(const pt_capacity& c, char* base, Buffers* b, GateWeights** gate =
   t.layer_zmax = (uint32_t*)take(E * kLayers * 4);
   t.seg = (uint2*)take(N * kMaxInner * sizeof(uint2));  // the table's max_inner slots used
   t.cell_in = (uint32_t*)take(C * 4);
-  t.cell_out = (uint32_t*)take(C * 4);
-  t.has_in = (uint8_t*)take(C);
-  t.has_out = (uint8_t*)take(C);
-  t.fb_kill = (uint8_t*)take(C);
+  t.cell = (CellState*)take(C * sizeof(CellState));
   t.fb_cnt = (uint32_t*)take((N + 1) * 4);
   t.fb_start = (uint32_t*)take((N + 1) * 4);
-  t.fb_rec = (float4*)take(L * 32);
-  t.cell_head = (uint32_t*)take(C * 4);
-  t.best = (unsigned long long*)take(C * 8);
-  t.link_dst = (uint32_t*)take(L * 4);
-  t.link_next = (uint32_t*)take(L * 4);
-  t.link_walk = (uint2*)take(L * 8);
-  t.link_q = (float*)take(L * 4);
+  t.link = (Link*)take(L * sizeof(Link));
+  t.link_best = (LinkBest*)take(L * sizeof(LinkBest));
   t.nt_hits = (int32_t*)take(T * kMaxHits * 4);
   t.nt_cells = (uint32_t*)take(T * kMaxCellsPerNt * 4);
   t.nt_n = (uint8_t*)take(T);
   t.nt_q = (float*)take(T * 4);
-  t.nt_rank = (uint32_t*)take(T * 4);
-  t.bucket_cnt = (uint32_t*)take((N + 1) * 4);
-  t.bucket_start = (uint32_t*)take((N + 1) * 4);
-  t.ord = (uint32_t*)take(T * 4);
-  t.alive = (uint32_t*)take(T * 4);
-  t.alive_scan = (uint32_t*)take((T + 1) * 4);
+  t.nt_next = (uint32_t*)take(T * 4);
+  t.nt_head = (uint32_t*)take(N * 4);
+  t.sv_cnt = t.fb_cnt;
+  t.sv_start = (uint32_t*)take((N + 1) * 4);
+  t.best_list = (uint32_t*)take(T * 4);
   t.used = (uint8_t*)take(N);
   t.sv = (uint32_t*)take(T * 4);
   t.ev_nt_off = (int64_t*)take((E + 1) * 8);
@@ -216,9 +207,9 @@ size_t layout(const pt_capacity& c, char* base, Buffers* b, GateWeights** gate =
   t.ev_v_scan = (uint32_t*)take((E + 1) * 4);
   t.ev_vtx_off = (int64_t*)take((E + 1) * 8);
   t.gate_x = (uint16_t*)take(L * 16 * 2);
+  t.fb_rec = (float4*)t.gate_x;
   t.gate_score = (float*)take(L * 4);
   t.gate_keep = (uint8_t*)take(L);
-  t.link_src = (uint32_t*)take(L * 4);
   t.exp_hits = (int32_t*)take(T * kMaxHits * 4);
   t.exp_n = (uint8_t*)take(T);
   t.exp_q = (float*)take(T * 4);
@@ -419,7 +410,6 @@ void enqueue_pipeline(pt_ctx* c, cudaStream_t s) {
   if (c->fishbone_on) launch_fishbone(c->B, c->P, L, s, c->gate_on);
   launch_ntuplets(c->B, c->P, L, s, c->masked());
   launch_fit(c->B, c->P, L, s);
-  launch_export_ntuplets(c->B, L, s);
 }
 
 pt_status ensure_graph(pt_ctx* c) {
@@ -717,9 +707,9 @@ pt_status pt_connect_cells(pt_ctx* c, int64_t* n_links) {
 
 pt_status pt_find_ntuplets(pt_ctx* c, int64_t* n_ntuplets) {
   STAGE_BODY((reset_counters(c, {CNT_NT, CNT_SCAN_NT, CNT_SV}),
-              cudaMemsetAsync(c->B.bucket_cnt, 0, (size_t)(loaded_hits(c) + 1) * 4, c->stream),
+              cudaMemsetAsync(c->B.sv_cnt, 0, (size_t)(loaded_hits(c) + 1) * 4, c->stream),
               cudaMemsetAsync(c->B.used, 0, (size_t)loaded_hits(c), c->stream),
-              launch_ntuplets(c->B, c->P, c->L, c->stream, c->links_masked)),
+              launch_ntuplet_steps(c->B, c->P, c->L, c->stream, c->links_masked)),
              CNT_SV, n_ntuplets)
 }
 
@@ -955,6 +945,7 @@ pt_status pt_get_cells(pt_ctx* c, int32_t* inner, int32_t* outer, int32_t* event
                            (long long)C);
   if (C == 0) return PT_OK;
   PT_TRY(val_staging(c, (size_t)slots * 12));
+  PT_CUDA(cudaMemsetAsync(c->val, 0xff, (size_t)slots * 12, c->stream));  // holes: event -1
   launch_export_cells(c->B, c->P, c->L, (int32_t*)c->val, c->stream);
   PT_TRY(last_launch());
   std::vector<int32_t> tmp((size_t)slots * 3);
