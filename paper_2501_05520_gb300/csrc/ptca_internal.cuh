@@ -40,7 +40,6 @@ enum : int {
   CNT_CELLS_USED = 10,  // cells written (CNT_CELLS counts reserved slots incl. holes)
   CNT_LINKS_USED = 11,  // links written (CNT_LINKS counts reserved slots incl. holes)
   CNT_DBL_WORK = 12,    // doublet search: next chunk of sorted hits
-  CNT_SCAN_EV = 13,     // events (size of the scan over per-event vertex counts)
   CNT_VTX = 14,         // vertices of the batch
   CNT_RAW_STATUS = 15,  // raw input: status bits (RAW_*), not reset by the chain
   CNT_RAW_DIGIS = 16,   // raw input: digis of the batch (size of the run-flag scan)
@@ -247,8 +246,7 @@ struct Buffers {
   pt_vertex* vtx;            // [max_ntuplets / 2 + 1] the batch's vertices, events in order
   int32_t* trk_vtx;          // [max_ntuplets] vertex of each track, -1 for none
   uint32_t* ev_nv;           // [max_events + 1] vertices per event
-  uint32_t* ev_v_scan;       // [max_events + 1] exclusive scan of ev_nv
-  int64_t* ev_vtx_off;       // [max_events + 1] the same as int64
+  int64_t* ev_vtx_off;       // [max_events + 1] vertices before each event
   // learned gate (valid when enabled)
   uint16_t* gate_x;          // [max_links*16] bf16 features per link slot (12 used)
   float* gate_score;         // [max_links] logit per link slot
@@ -342,8 +340,8 @@ cudaError_t launch_raw(const RawBuffers& r, const Buffers& b, const pt_module* m
                        int64_t cap_hits, const Launch& l, cudaStream_t s);
 // primary vertices of the fitted tracks of n_events events (tracks with >= min_hits
 // hits, groups cut at z0 steps > dz)
-cudaError_t launch_vertices(const Buffers& b, int n_events, int32_t min_hits, float dz,
-                            uint64_t cap_nt, const Launch& l, cudaStream_t s);
+cudaError_t launch_vertices(const Buffers& b, const Params& p, int n_events, int32_t min_hits,
+                            float dz, const Launch& l, cudaStream_t s);
 // scan of n+1 entries: out[i] = sum(in[0..i)), n = *n_dev
 void launch_scan(const uint32_t* in, uint32_t* out, const unsigned long long* n_dev,
                  uint32_t* part, cudaStream_t s);

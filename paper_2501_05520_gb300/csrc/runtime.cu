@@ -204,7 +204,6 @@ size_t layout(const pt_capacity& c, char* base, Buffers* b, GateWeights** gate =
   t.vtx = (pt_vertex*)take((T / 2 + 1) * sizeof(pt_vertex));
   t.trk_vtx = (int32_t*)take(T * 4);
   t.ev_nv = (uint32_t*)take((E + 1) * 4);
-  t.ev_v_scan = (uint32_t*)take((E + 1) * 4);
   t.ev_vtx_off = (int64_t*)take((E + 1) * 8);
   t.gate_x = (uint16_t*)take(L * 16 * 2);
   t.fb_rec = (float4*)t.gate_x;
@@ -901,8 +900,7 @@ pt_status pt_find_vertices(pt_ctx* c, int min_hits, float dz, int64_t* n_vertice
   if (!(dz > 0.0f) || !std::isfinite(dz)) return fail(PT_ERR_INVALID, "dz must be finite and > 0");
   DeviceGuard guard(c->device);
   if (!c->fitted) return fail(PT_ERR_INVALID, "pt_fit_tracks has not run on this batch");
-  PT_CUDA(launch_vertices(c->B, c->n_events, min_hits, dz, (uint64_t)c->cap.max_ntuplets, c->L,
-                          c->stream));
+  PT_CUDA(launch_vertices(c->B, c->P, c->n_events, min_hits, dz, c->L, c->stream));
   c->vtx_ready = true;
   if (n_vertices) {
     PT_TRY(sync_counters(c));
