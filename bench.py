@@ -774,7 +774,7 @@ def run_ours(args):
             trace = ctx.pt_get_trace()
             ctx.pt_set_tracing(False)
             kernels[form] = {k: round(ms / n, 4) for k, (ms, n) in trace.items()}
-            launches[form] = sum(n * (3 if k == "scan" else 1)
+            launches[form] = sum(n * (2 if k == "scan" else 1)
                                  for k, (_, n) in trace.items()) // TRACE_STEPS
         total_s = max_over_ranks(sum(step_ms) / 1000.0, dist, dev)
         # end to end through the public call: pinned host in, host out; E2E_THREADS host

@@ -13,6 +13,7 @@ constexpr float kPi = 3.14159265358979323846f;
 
 // Reset per-batch counters and the histogram / flag arrays, sized from the header.
 __global__ void k_clear(Buffers b, int32_t phi_bins) {
+  pdl_sync();
   const int E = b.hdr->n_events, N = b.hdr->n_hits;
   const int nb = E * kLayers * phi_bins;
   const int stride = gridDim.x * blockDim.x;
@@ -58,6 +59,7 @@ __device__ __forceinline__ float hit_radius(float x, float y) {
 // Histogram: global bin of every input hit and its rank inside the bin; the r and z
 // ranges per (event, layer), reduced within the warp before the atomics.
 __global__ void k_bin_count(Buffers b, int32_t B) {
+  pdl_sync();
   const int E = b.hdr->n_events, N = b.hdr->n_hits;
   const float scale = (float)B / (2.0f * kPi);
   const int stride = gridDim.x * blockDim.x;
@@ -102,6 +104,7 @@ __global__ void k_bin_count(Buffers b, int32_t B) {
 }
 
 __global__ void k_bin_scatter(Buffers b, float kmax) {
+  pdl_sync();
   const int N = b.hdr->n_hits;
   const int stride = gridDim.x * blockDim.x;
   // per event layer: the outer- and inner-radius terms of the azimuthal windows of the
@@ -145,70 +148,92 @@ __device__ __forceinline__ uint32_t block_excl_scan(uint32_t v, uint32_t* warp_s
   return r;
 }
 
+// A block's share of n entries, a multiple of four so that aligned arrays are read four at a
+// time.
 __device__ __forceinline__ void chunk_of(uint64_t n, uint64_t* lo, uint64_t* hi) {
-  const uint64_t per = (n + gridDim.x - 1) / gridDim.x;
+  const uint64_t per = ((n + gridDim.x - 1) / gridDim.x + 3) & ~3ull;
   *lo = min(n, per * blockIdx.x);
   *hi = min(n, *lo + per);
 }
 
+__device__ __forceinline__ uint4 scan_load(const uint32_t* in, uint64_t i, uint64_t hi, bool vec) {
+  if (vec && i + 4 <= hi) return *(const uint4*)(in + i);
+  return make_uint4(i < hi ? in[i] : 0u, i + 1 < hi ? in[i + 1] : 0u, i + 2 < hi ? in[i + 2] : 0u,
+                    i + 3 < hi ? in[i + 3] : 0u);
+}
+
+// Sum of each block's share.
 __global__ void __launch_bounds__(kScanThreads) k_scan_partial(const uint32_t* in, uint32_t* part,
                                                                const unsigned long long* n_dev) {
+  pdl_sync();
   __shared__ uint32_t ws[kScanThreads / 32];
   __shared__ uint32_t tot;
   uint64_t lo, hi;
   chunk_of(*n_dev, &lo, &hi);
+  const bool vec = ((uintptr_t)in & 15u) == 0;
   uint32_t acc = 0;
-  for (uint64_t i = lo + threadIdx.x; i < hi; i += kScanThreads) acc += in[i];
+#pragma unroll 4
+  for (uint64_t i = lo + 4 * threadIdx.x; i < hi; i += 4 * kScanThreads) {
+    const uint4 v = scan_load(in, i, hi, vec);
+    acc += v.x + v.y + v.z + v.w;
+  }
   block_excl_scan(acc, ws, &tot);
   if (threadIdx.x == 0) part[blockIdx.x] = tot;
 }
 
-__global__ void __launch_bounds__(kScanThreads) k_scan_top(uint32_t* part, int nparts) {
-  __shared__ uint32_t ws[kScanThreads / 32];
-  __shared__ uint32_t tot;
-  // nparts <= kScanThreads
-  const uint32_t v = threadIdx.x < nparts ? part[threadIdx.x] : 0u;
-  const uint32_t ex = block_excl_scan(v, ws, &tot);
-  if (threadIdx.x < nparts) part[threadIdx.x] = ex;
-  if (threadIdx.x == 0) part[nparts] = tot;
-}
-
+// Each block adds up the shares before its own (no third launch for them) and scans its
+// share, four entries per thread at a time.
 __global__ void __launch_bounds__(kScanThreads) k_scan_final(const uint32_t* in, uint32_t* out,
                                                              const uint32_t* part,
                                                              const unsigned long long* n_dev) {
+  pdl_sync();
   __shared__ uint32_t ws[kScanThreads / 32];
   __shared__ uint32_t tot;
+  static_assert(kScanBlocks <= kScanThreads, "one partial sum per thread");
   const uint64_t n = *n_dev;
   uint64_t lo, hi;
   chunk_of(n, &lo, &hi);
-  uint32_t carry = part[blockIdx.x];
-  for (uint64_t base = lo; base < hi; base += kScanThreads) {
-    const uint64_t i = base + threadIdx.x;
-    const uint32_t v = i < hi ? in[i] : 0u;
-    const uint32_t ex = block_excl_scan(v, ws, &tot);
-    if (i < hi) out[i] = carry + ex;
+  block_excl_scan(threadIdx.x < blockIdx.x ? part[threadIdx.x] : 0u, ws, &tot);
+  uint32_t carry = tot;
+  const bool vec_in = ((uintptr_t)in & 15u) == 0, vec_out = ((uintptr_t)out & 15u) == 0;
+  for (uint64_t base = lo; base < hi; base += 4 * kScanThreads) {
+    __syncthreads();  // tot has been read
+    const uint64_t i = base + 4 * threadIdx.x;
+    const uint4 v = scan_load(in, i, hi, vec_in);
+    uint4 r;
+    r.x = carry + block_excl_scan(v.x + v.y + v.z + v.w, ws, &tot);
+    r.y = r.x + v.x;
+    r.z = r.y + v.y;
+    r.w = r.z + v.z;
+    if (vec_out && i + 4 <= hi) {
+      *(uint4*)(out + i) = r;
+    } else {
+      if (i < hi) out[i] = r.x;
+      if (i + 1 < hi) out[i + 1] = r.y;
+      if (i + 2 < hi) out[i + 2] = r.z;
+      if (i + 3 < hi) out[i + 3] = r.w;
+    }
     carry += tot;
   }
-  if (blockIdx.x == gridDim.x - 1 && threadIdx.x == 0) out[n] = part[gridDim.x];
+  if (blockIdx.x == gridDim.x - 1 && threadIdx.x == 0) out[n] = carry;
 }
 
 }  // namespace
 
 void launch_scan(const uint32_t* in, uint32_t* out, const unsigned long long* n_dev,
                  uint32_t* part, cudaStream_t s) {
-  k_scan_partial<<<kScanBlocks, kScanThreads, 0, s>>>(in, part, n_dev);
-  k_scan_top<<<1, kScanThreads, 0, s>>>(part, kScanBlocks);
-  k_scan_final<<<kScanBlocks, kScanThreads, 0, s>>>(in, out, part, n_dev);
+  launch_pdl(k_scan_partial, kScanBlocks, kScanThreads, 0, s, in, part, n_dev);
+  launch_pdl(k_scan_final, kScanBlocks, kScanThreads, 0, s, in, out, part, n_dev);
 }
 
 void launch_clear(const Buffers& b, const Params& p, const Launch& l, cudaStream_t s) {
-  PT_TRACE(l, s, "k_clear", k_clear<<<l.grid, 256, 0, s>>>(b, p.phi_bins));
+  PT_TRACE(l, s, "k_clear", launch_pdl(k_clear, l.grid, 256, 0, s, b, p.phi_bins));
 }
 
 void launch_bin_hits(const Buffers& b, const Params& p, const Launch& l, cudaStream_t s) {
-  PT_TRACE(l, s, "k_bin_count", k_bin_count<<<l.grid, 256, 0, s>>>(b, p.phi_bins));
+  PT_TRACE(l, s, "k_bin_count", launch_pdl(k_bin_count, l.grid, 256, 0, s, b, p.phi_bins));
   PT_TRACE(l, s, "scan", launch_scan(b.bin_cnt, b.bin_start, &b.cnt[CNT_SCAN_BINS], b.scan_part, s));
-  PT_TRACE(l, s, "k_bin_scatter", k_bin_scatter<<<l.grid, 256, 0, s>>>(b, p.cuts.kmax));
+  PT_TRACE(l, s, "k_bin_scatter", launch_pdl(k_bin_scatter, l.grid, 256, 0, s, b, p.cuts.kmax));
 }
 
 namespace {

@@ -515,6 +515,7 @@ __global__ void __launch_bounds__(kThreads, kBlocksPerSm)
     k_refit_bl(Buffers b, float bfield, float x0b, float x0d, const uint32_t* in_list,
                const unsigned long long* in_n, uint32_t* out_list, unsigned long long* out_n,
                uint64_t cap) {
+  pdl_sync();
   namespace cg = cooperative_groups;
   extern __shared__ __align__(16) unsigned char rsm[];
   RefitSmem& S = *(RefitSmem*)rsm;
@@ -552,8 +553,8 @@ cudaError_t launch_refit_broken_line(const Buffers& b, const Params& p, float x0
     uint32_t* out = pass + 1 < kMaxPasses ? lists[pass & 1] : nullptr;
     unsigned long long* out_n = pass + 1 < kMaxPasses ? &counters[pass] : nullptr;
     PT_TRACE(l, s, "k_refit_bl",
-             k_refit_bl<<<l.sms * kBlocksPerSm, kThreads, sizeof(RefitSmem), s>>>(b, p.bfield, x0_barrel, x0_disk, in, in_n, out,
-                                                   out_n, cap));
+             launch_pdl(k_refit_bl, l.sms * kBlocksPerSm, kThreads, sizeof(RefitSmem), s, b,
+                        p.bfield, x0_barrel, x0_disk, in, in_n, out, out_n, cap));
   }
   return cudaGetLastError();
 }

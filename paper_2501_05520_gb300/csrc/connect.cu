@@ -164,6 +164,7 @@ __device__ __forceinline__ unsigned long long chunk_take_shared(
 
 __global__ void __launch_bounds__(kConnWarps * 32, kConnBlocksPerSm)
     k_connect(Buffers b, pt_cuts cuts, PairTable pt, int32_t B, uint64_t cap_links) {
+  pdl_wait();
   __shared__ ConnWarp s_w[kConnWarps];
   const int lane = lane_id();
   ConnWarp& W = s_w[threadIdx.x >> 5];
@@ -563,6 +564,7 @@ __device__ __forceinline__ uint32_t find_inner(const Buffers& b, uint32_t lo, ui
 template <bool GATE>
 __global__ void k_link_targets(Buffers b, pt_cuts cuts, int32_t B, int max_inner,
                                uint64_t cap_links) {
+  pdl_wait();
   const uint64_t nl = min(b.cnt[CNT_LINKS], (unsigned long long)cap_links);
   const uint64_t stride = (uint64_t)gridDim.x * blockDim.x;
   for (uint64_t l = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x; l < nl; l += stride) {
@@ -600,16 +602,16 @@ __global__ void k_link_targets(Buffers b, pt_cuts cuts, int32_t B, int max_inner
 void launch_connect(const Buffers& b, const Params& p, const Launch& l, cudaStream_t s,
                     bool gated) {
   PT_TRACE(l, s, "k_connect",
-           k_connect<<<l.sms * kConnBlocksPerSm, kConnWarps * 32, 0, s>>>(
-               b, p.cuts, p.pairs, p.phi_bins, (uint64_t)p.max_links));
+           launch_pdl(k_connect, l.sms * kConnBlocksPerSm, kConnWarps * 32, 0, s, b, p.cuts,
+                      p.pairs, p.phi_bins, (uint64_t)p.max_links));
   if (gated)
     PT_TRACE(l, s, "k_link_targets",
-             k_link_targets<true><<<l.grid, 256, 0, s>>>(b, p.cuts, p.phi_bins, p.pairs.max_inner,
-                                                         (uint64_t)p.max_links));
+             launch_pdl(k_link_targets<true>, l.grid, 256, 0, s, b, p.cuts, p.phi_bins,
+                        p.pairs.max_inner, (uint64_t)p.max_links));
   else
     PT_TRACE(l, s, "k_link_targets",
-             k_link_targets<false><<<l.grid, 256, 0, s>>>(b, p.cuts, p.phi_bins, p.pairs.max_inner,
-                                                          (uint64_t)p.max_links));
+             launch_pdl(k_link_targets<false>, l.grid, 256, 0, s, b, p.cuts, p.phi_bins,
+                        p.pairs.max_inner, (uint64_t)p.max_links));
 }
 
 }  // namespace ptca

@@ -85,6 +85,7 @@ __device__ __forceinline__ uint4 reverse_window(const Buffers& b, const pt_cuts&
 // at once) and kept in shared memory; the warp then searches them hit by hit.
 __global__ void __launch_bounds__(kWarpsPerBlock * 32, 5)
     k_doublets(Buffers b, pt_cuts cuts, PairTable pt, int32_t B, uint64_t cap_cells) {
+  pdl_wait();
   __shared__ uint32_t st_val[kWarpsPerBlock][kStage];
   __shared__ uint4 st_rng[kWarpsPerBlock][32][kMaxInner];
   __shared__ float4 st_hit[kWarpsPerBlock][32];
@@ -206,8 +207,8 @@ __global__ void __launch_bounds__(kWarpsPerBlock * 32, 5)
 
 void launch_doublets(const Buffers& b, const Params& p, const Launch& l, cudaStream_t s) {
   PT_TRACE(l, s, "k_doublets",
-           k_doublets<<<l.sgrid, kWarpsPerBlock * 32, 0, s>>>(b, p.cuts, p.pairs, p.phi_bins,
-                                                               (uint64_t)p.max_cells));
+           launch_pdl(k_doublets, l.sgrid, kWarpsPerBlock * 32, 0, s, b, p.cuts, p.pairs,
+                      p.phi_bins, (uint64_t)p.max_cells));
 }
 
 }  // namespace ptca

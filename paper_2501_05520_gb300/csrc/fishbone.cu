@@ -84,6 +84,7 @@ __device__ __forceinline__ uint32_t run_source(const Buffers& b, uint64_t l, boo
 }
 
 __global__ void k_fb_count(Buffers b, uint64_t cap_links, bool gated) {
+  pdl_sync();
   const uint64_t nl = min(b.cnt[CNT_LINKS], (unsigned long long)cap_links);
   const uint64_t stride = (uint64_t)gridDim.x * blockDim.x;
   for (uint64_t l = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x; l < nl; l += stride) {
@@ -93,6 +94,7 @@ __global__ void k_fb_count(Buffers b, uint64_t cap_links, bool gated) {
 }
 
 __global__ void k_fb_scatter(Buffers b, int32_t B, uint64_t cap_links, bool gated) {
+  pdl_sync();
   const uint64_t nl = min(b.cnt[CNT_LINKS], (unsigned long long)cap_links);
   const uint64_t stride = (uint64_t)gridDim.x * blockDim.x;
   for (uint64_t l = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x; l < nl; l += stride) {
@@ -108,6 +110,7 @@ __global__ void k_fb_scatter(Buffers b, int32_t B, uint64_t cap_links, bool gate
 // One active cell per thread against the other active cells ending on its outer hit
 // (the records of its group, consecutive in fb_rec).
 __global__ void k_fb_compare(Buffers b) {
+  pdl_sync();
   const uint32_t n_act = b.fb_start[b.cnt[CNT_SCAN_HITS]];
   const uint32_t stride = gridDim.x * blockDim.x;
   const FbCell* rec = reinterpret_cast<const FbCell*>(b.fb_rec);
@@ -125,6 +128,7 @@ __global__ void k_fb_compare(Buffers b) {
 // Keep mask of every link slot: the gate's (gated) and neither end removed; the flags
 // of both ends cleared.  The kept links are counted.
 __global__ void k_fb_filter_clear(Buffers b, uint64_t cap_links, bool gated) {
+  pdl_sync();
   const uint64_t nl = min(b.cnt[CNT_LINKS], (unsigned long long)cap_links);
   const uint64_t stride = (uint64_t)gridDim.x * blockDim.x;
   uint32_t kept = 0;
@@ -146,6 +150,7 @@ __global__ void k_fb_filter_clear(Buffers b, uint64_t cap_links, bool gated) {
 
 // Flags of the ends of every kept link.
 __global__ void k_fb_filter_set(Buffers b, uint64_t cap_links) {
+  pdl_sync();
   const uint64_t nl = min(b.cnt[CNT_LINKS], (unsigned long long)cap_links);
   const uint64_t stride = (uint64_t)gridDim.x * blockDim.x;
   for (uint64_t l = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x; l < nl; l += stride) {
@@ -162,15 +167,16 @@ void launch_fishbone(const Buffers& b, const Params& p, const Launch& l, cudaStr
   cudaMemsetAsync(&b.cnt[CNT_GATE_KEPT], 0, sizeof(unsigned long long), s);  // recounted
   cudaMemsetAsync(b.fb_cnt, 0, (size_t)(p.max_hits + 1) * 4, s);
   PT_TRACE(l, s, "k_fb_count",
-           k_fb_count<<<l.grid, 256, 0, s>>>(b, (uint64_t)p.max_links, gated));
+           launch_pdl(k_fb_count, l.grid, 256, 0, s, b, (uint64_t)p.max_links, gated));
   PT_TRACE(l, s, "scan", launch_scan(b.fb_cnt, b.fb_start, &b.cnt[CNT_SCAN_HITS], b.scan_part, s));
   PT_TRACE(l, s, "k_fb_scatter",
-           k_fb_scatter<<<l.grid, 256, 0, s>>>(b, p.phi_bins, (uint64_t)p.max_links, gated));
-  PT_TRACE(l, s, "k_fb_compare", k_fb_compare<<<l.grid, 256, 0, s>>>(b));
+           launch_pdl(k_fb_scatter, l.grid, 256, 0, s, b, p.phi_bins, (uint64_t)p.max_links,
+                      gated));
+  PT_TRACE(l, s, "k_fb_compare", launch_pdl(k_fb_compare, l.grid, 256, 0, s, b));
   PT_TRACE(l, s, "k_fb_filter_clear",
-           k_fb_filter_clear<<<l.grid, 256, 0, s>>>(b, (uint64_t)p.max_links, gated));
+           launch_pdl(k_fb_filter_clear, l.grid, 256, 0, s, b, (uint64_t)p.max_links, gated));
   PT_TRACE(l, s, "k_fb_filter_set",
-           k_fb_filter_set<<<l.grid, 256, 0, s>>>(b, (uint64_t)p.max_links));
+           launch_pdl(k_fb_filter_set, l.grid, 256, 0, s, b, (uint64_t)p.max_links));
 }
 
 }  // namespace ptca

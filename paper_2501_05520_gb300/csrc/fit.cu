@@ -63,6 +63,7 @@ __device__ __forceinline__ float gsum(float v) {
 }
 
 __global__ void __launch_bounds__(256) k_fit(Buffers b, float bfield) {
+  pdl_wait();
   const uint64_t S = b.cnt[CNT_SV];
   const int lane = lane_id();
   const int sub = lane & 7;
@@ -181,7 +182,7 @@ __global__ void __launch_bounds__(256) k_fit(Buffers b, float bfield) {
 }  // namespace
 
 void launch_fit(const Buffers& b, const Params& p, const Launch& l, cudaStream_t s) {
-  PT_TRACE(l, s, "k_fit", k_fit<<<l.grid, 256, 0, s>>>(b, p.bfield));
+  PT_TRACE(l, s, "k_fit", launch_pdl(k_fit, l.grid, 256, 0, s, b, p.bfield));
 }
 
 }  // namespace ptca

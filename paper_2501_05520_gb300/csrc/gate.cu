@@ -141,9 +141,6 @@ __global__ void __launch_bounds__(kTileM, kMlpCtasPerSm)
   uint64_t* mbar = (uint64_t*)(sm + kOffBar);
   uint32_t* tslot = (uint32_t*)(sm + kOffTmem);
   volatile uint32_t* flag = (volatile uint32_t*)(sm + kOffFlag);
-  // rows: n_max, or the device count clamped to n_max
-  const uint64_t n = n_dev ? min((uint64_t)*n_dev, (uint64_t)n_max) : (uint64_t)n_max;
-
   // weights -> shared memory (already in the operand layout)
   {
     const uint4* w1 = (const uint4*)gw->w1;
@@ -170,6 +167,9 @@ __global__ void __launch_bounds__(kTileM, kMlpCtasPerSm)
                  : "memory");
     asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
   }
+  pdl_sync();  // the weights were uploaded before any of this stream's work was launched
+  // rows: n_max, or the device count clamped to n_max
+  const uint64_t n = n_dev ? min((uint64_t)*n_dev, (uint64_t)n_max) : (uint64_t)n_max;
   fence_async_smem();
   tc_before_sync();
   __syncthreads();
@@ -324,6 +324,7 @@ __global__ void k_gate_features_f32(Buffers b, pt_cuts cuts, int32_t B, uint64_t
 
 // float32 feature rows -> bf16 rows padded to 16.
 __global__ void k_gate_pack(const float* feat, int64_t n, uint16_t* X) {
+  pdl_sync();
   const int64_t stride = (int64_t)gridDim.x * blockDim.x;
   for (int64_t r = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; r < n; r += stride) {
     float f[kGateFeat];
@@ -347,17 +348,17 @@ cudaError_t gate_prepare() {
 void launch_gate(const Buffers& b, const Params& p, const Launch& l, const GateWeights* w,
                  cudaStream_t s) {
   PT_TRACE(l, s, "k_gate_mlp",
-           k_gate_mlp<true><<<l.sms * kMlpCtasPerSm, kTileM, kMlpSmem, s>>>(
-               w, b, p.cuts, p.phi_bins, nullptr, &b.cnt[CNT_LINKS], p.max_links, b.gate_score,
-               b.gate_keep, &b.cnt[CNT_STATUS], &b.cnt[CNT_GATE_KEPT], p.wait_cycles));
+           launch_pdl(k_gate_mlp<true>, l.sms * kMlpCtasPerSm, kTileM, kMlpSmem, s, w, b, p.cuts,
+                      p.phi_bins, nullptr, &b.cnt[CNT_LINKS], p.max_links, b.gate_score,
+                      b.gate_keep, &b.cnt[CNT_STATUS], &b.cnt[CNT_GATE_KEPT], p.wait_cycles));
 }
 
 void launch_gate_score(const GateWeights* w, const float* feat, int64_t n, float* out,
                        uint16_t* xbuf, unsigned long long* status, int sms, long long wait_cycles,
                        cudaStream_t s) {
-  k_gate_pack<<<sms * 4, 256, 0, s>>>(feat, n, xbuf);
-  k_gate_mlp<false><<<sms * kMlpCtasPerSm, kTileM, kMlpSmem, s>>>(w, Buffers{}, pt_cuts{}, 1, xbuf, nullptr, n,
-                                                        out, nullptr, status, nullptr, wait_cycles);
+  launch_pdl(k_gate_pack, sms * 4, 256, 0, s, feat, n, xbuf);
+  launch_pdl(k_gate_mlp<false>, sms * kMlpCtasPerSm, kTileM, kMlpSmem, s, w, Buffers{}, pt_cuts{}, 1,
+             xbuf, nullptr, n, out, nullptr, status, nullptr, wait_cycles);
 }
 
 void launch_export_link_features(const Buffers& b, const Params& p, const Launch& l, bool gated,

@@ -200,6 +200,7 @@ __device__ uint32_t walk(const Buffers& b, uint32_t l0, unsigned long long t0, u
 template <bool GATED, bool CLEAN>
 __global__ void __launch_bounds__(kNtWarps * 32, kNtBlocksPerSm)
     k_find_ntuplets(Buffers b, uint64_t cap_links, uint64_t cap_nt) {
+  pdl_wait();
   __shared__ NtWarp s_w[kNtWarps];
   NtWarp& W = s_w[threadIdx.x >> 5];
   const uint64_t nl = min(b.cnt[CNT_LINKS], (unsigned long long)cap_links);
@@ -301,6 +302,7 @@ __device__ __noinline__ void take_tied_cell(const Buffers& b, uint32_t t, unsign
 // Ntuplets that no cell ranks behind another hit count or q go to best_list (one
 // reservation per warp); cells where two of the same meet are decided on the way.
 __global__ void k_dedup_best(Buffers b, uint64_t cap_nt) {
+  pdl_wait();
   const uint64_t T = min(b.cnt[CNT_NT], (unsigned long long)cap_nt);
   if (blockIdx.x == 0 && threadIdx.x == 0) b.cnt[CNT_SCAN_NT] = T;
   const uint64_t stride = (uint64_t)gridDim.x * blockDim.x;
@@ -356,6 +358,7 @@ __device__ __forceinline__ bool holds_all(const Buffers& b, uint64_t t, uint32_t
 // The listed ntuplets that hold all their cells (where cells were tied, that is looked up
 // again) and have four or more hits mark their hits used.
 __global__ void k_used_hits(Buffers b) {
+  pdl_sync();
   const uint64_t N = b.cnt[CNT_NT_BEST];
   const bool ties = b.cnt[CNT_NT_TIES] != 0;
   const uint64_t stride = (uint64_t)gridDim.x * blockDim.x;
@@ -374,6 +377,7 @@ __global__ void k_used_hits(Buffers b) {
 // Survivors: the listed ntuplets of four or more hits, and the triplets that share no hit
 // with them; each goes on its first hit's list and is counted there.
 __global__ void k_survivors(Buffers b) {
+  pdl_sync();
   const uint64_t N = b.cnt[CNT_NT_BEST];
   const uint64_t stride = (uint64_t)gridDim.x * blockDim.x;
   for (uint64_t i = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x; i < N; i += stride) {
@@ -393,6 +397,7 @@ __global__ void k_survivors(Buffers b) {
 // hit's list.  Per-event offsets and the total come from the places of the events' first
 // hits.  The ntuplet also goes to the export staging, with event-local indices.
 __global__ void k_order(Buffers b) {
+  pdl_sync();
   const uint64_t N = b.cnt[CNT_NT_BEST];
   const int E = b.hdr->n_events;
   const uint64_t stride = (uint64_t)gridDim.x * blockDim.x;
@@ -542,20 +547,20 @@ static void launch_search(const Buffers& b, const Params& p, const Launch& l, cu
   const int grid = l.sms * kNtBlocksPerSm, block = kNtWarps * 32;
   if (gated)
     PT_TRACE(l, s, "k_find_ntuplets",
-             k_find_ntuplets<true, CLEAN><<<grid, block, 0, s>>>(b, cap_links, cap_nt));
+             launch_pdl(k_find_ntuplets<true, CLEAN>, grid, block, 0, s, b, cap_links, cap_nt));
   else
     PT_TRACE(l, s, "k_find_ntuplets",
-             k_find_ntuplets<false, CLEAN><<<grid, block, 0, s>>>(b, cap_links, cap_nt));
+             launch_pdl(k_find_ntuplets<false, CLEAN>, grid, block, 0, s, b, cap_links, cap_nt));
 }
 
 void launch_ntuplets(const Buffers& b, const Params& p, const Launch& l, cudaStream_t s,
                      bool gated) {
   launch_search<true>(b, p, l, s, gated);
-  k_dedup_best<<<l.grid, 256, 0, s>>>(b, (uint64_t)p.max_ntuplets);
-  k_used_hits<<<l.grid, 256, 0, s>>>(b);
-  k_survivors<<<l.grid, 256, 0, s>>>(b);
+  launch_pdl(k_dedup_best, l.grid, 256, 0, s, b, (uint64_t)p.max_ntuplets);
+  launch_pdl(k_used_hits, l.grid, 256, 0, s, b);
+  launch_pdl(k_survivors, l.grid, 256, 0, s, b);
   launch_scan(b.sv_cnt, b.sv_start, &b.cnt[CNT_SCAN_HITS], b.scan_part, s);
-  k_order<<<l.grid, 256, 0, s>>>(b);
+  launch_pdl(k_order, l.grid, 256, 0, s, b);
 }
 
 void launch_ntuplet_steps(const Buffers& b, const Params& p, const Launch& l, cudaStream_t s,

@@ -73,6 +73,7 @@ __device__ __forceinline__ int digi_event(const int64_t* off, int E, int64_t i) 
 // flag[i] = 1 where a module run starts; every digi is checked against the table.
 __global__ void k_raw_runs(RawBuffers r, const pt_module* mods, int n_mod, int E,
                            unsigned long long* status) {
+  pdl_sync();
   const int64_t n = r.digi_off[E];
   if (blockIdx.x == 0 && threadIdx.x == 0) {
     r.cnt[CNT_RAW_DIGIS] = (unsigned long long)n;
@@ -93,6 +94,7 @@ __global__ void k_raw_runs(RawBuffers r, const pt_module* mods, int n_mod, int E
 
 // run_first[run] = its first digi (from the scan of the flags); run_first[R] = n.
 __global__ void k_raw_run_starts(RawBuffers r, int E) {
+  pdl_sync();
   const int64_t n = r.digi_off[E];
   for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n;
        i += (int64_t)gridDim.x * blockDim.x)
@@ -293,6 +295,7 @@ __device__ __forceinline__ void cluster_run(const G& g, RawWarp<CAP>& W, const R
 // launch's list.
 __global__ void __launch_bounds__(kSmallWarps * 32, kSmallBlocksPerSm)
     k_raw_cluster(RawBuffers r, const pt_module* mods, int n_mod, unsigned long long* status) {
+  pdl_sync();
   __shared__ RawWarp<kRunSmall> s_w[kSmallWarps];
   RawWarp<kRunSmall>& W = s_w[threadIdx.x >> 5];
   const uint32_t R = r.run_scan[r.digi_off[r.n_events]];
@@ -325,6 +328,7 @@ __global__ void __launch_bounds__(kSmallWarps * 32, kSmallBlocksPerSm)
 // One block per listed run of more than kRunSmall digis (at most kRunMax).
 __global__ void __launch_bounds__(kBigThreads, kBigBlocksPerSm)
     k_raw_cluster_big(RawBuffers r, const pt_module* mods, int n_mod, unsigned long long* status) {
+  pdl_sync();
   __shared__ RawWarp<kRunMax> W;
   __shared__ uint32_t s_count[kBigThreads / 32];
   const BlockGroup<kBigThreads> g{s_count};
@@ -346,6 +350,7 @@ __global__ void __launch_bounds__(kBigThreads, kBigBlocksPerSm)
 // Hits of run `run` to the chain's inputs at run_hoff[run]; per-event hit offsets (an
 // event's first run; events without digis own no hits) and the batch header.
 __global__ void k_raw_place(RawBuffers r, Buffers b, int64_t cap_hits, unsigned long long* status) {
+  pdl_sync();
   const int E = r.n_events;
   const uint32_t R = r.run_scan[r.digi_off[E]];
   const uint32_t H = r.run_hoff[R];
@@ -388,18 +393,21 @@ __global__ void k_raw_place(RawBuffers r, Buffers b, int64_t cap_hits, unsigned 
 cudaError_t launch_raw(const RawBuffers& r, const Buffers& b, const pt_module* mods, int n_mod,
                        int64_t cap_hits, const Launch& l, cudaStream_t s) {
   unsigned long long* status = &b.cnt[CNT_RAW_STATUS];
-  PT_TRACE(l, s, "k_raw_runs", k_raw_runs<<<l.grid, 256, 0, s>>>(r, mods, n_mod, r.n_events, status));
+  PT_TRACE(l, s, "k_raw_runs",
+           launch_pdl(k_raw_runs, l.grid, 256, 0, s, r, mods, n_mod, r.n_events, status));
   // run numbers: run_scan[i] = runs starting before digi i
   PT_TRACE(l, s, "scan", launch_scan(r.flag, r.run_scan, &r.cnt[CNT_RAW_DIGIS], r.scan_part, s));
-  PT_TRACE(l, s, "k_raw_run_starts", k_raw_run_starts<<<l.grid, 256, 0, s>>>(r, r.n_events));
+  PT_TRACE(l, s, "k_raw_run_starts",
+           launch_pdl(k_raw_run_starts, l.grid, 256, 0, s, r, r.n_events));
   PT_TRACE(l, s, "k_raw_cluster",
-           k_raw_cluster<<<l.sms * kSmallBlocksPerSm, kSmallWarps * 32, 0, s>>>(r, mods, n_mod,
-                                                                                status));
+           launch_pdl(k_raw_cluster, l.sms * kSmallBlocksPerSm, kSmallWarps * 32, 0, s, r, mods,
+                      n_mod, status));
   PT_TRACE(l, s, "k_raw_cluster_big",
-           k_raw_cluster_big<<<l.sms * kBigBlocksPerSm, kBigThreads, 0, s>>>(r, mods, n_mod,
-                                                                             status));
+           launch_pdl(k_raw_cluster_big, l.sms * kBigBlocksPerSm, kBigThreads, 0, s, r, mods, n_mod,
+                      status));
   PT_TRACE(l, s, "scan", launch_scan(r.run_nh, r.run_hoff, &r.cnt[CNT_RAW_RUNS], r.scan_part, s));
-  PT_TRACE(l, s, "k_raw_place", k_raw_place<<<l.grid, 256, 0, s>>>(r, b, cap_hits, status));
+  PT_TRACE(l, s, "k_raw_place",
+           launch_pdl(k_raw_place, l.grid, 256, 0, s, r, b, cap_hits, status));
   return cudaGetLastError();
 }
 

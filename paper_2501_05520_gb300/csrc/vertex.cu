@@ -94,6 +94,7 @@ __device__ __noinline__ void vtx_bitonic(unsigned long long* key, uint32_t n) {
 __global__ void __launch_bounds__(kVtxThreads) k_vertex_event(Buffers b, int32_t min_hits,
                                                               float dz, float z_range,
                                                               uint64_t cap_nt) {
+  pdl_sync();
   extern __shared__ unsigned char vsm[];
   unsigned long long* key = reinterpret_cast<unsigned long long*>(vsm);  // [kVtxMax]
   uint32_t* vf = reinterpret_cast<uint32_t*>(vsm + (size_t)kVtxMax * 8);  // [kVtxMax]
@@ -256,6 +257,7 @@ __global__ void __launch_bounds__(kVtxThreads) k_vertex_event(Buffers b, int32_t
 constexpr int kPlaceThreads = 256;
 constexpr int kPlaceBlocks = 8;
 __global__ void __launch_bounds__(kPlaceThreads) k_vertex_compact(Buffers b, uint64_t cap_nt) {
+  pdl_sync();
   __shared__ uint32_t s_sum[kPlaceThreads / 32];
   const int e = blockIdx.x, E = gridDim.x;
   const int64_t S = (int64_t)min(b.cnt[CNT_SV], (unsigned long long)cap_nt);
@@ -297,10 +299,11 @@ cudaError_t launch_vertices(const Buffers& b, const Params& p, int n_events, int
                                          cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kVtxSmem);
   if (err != cudaSuccess) return err;
   PT_TRACE(l, s, "k_vertex_event",
-           k_vertex_event<<<n_events, kVtxThreads, kVtxSmem, s>>>(b, min_hits, dz,
-                                                                  1.25f * p.cuts.z0max, cap_nt));
+           launch_pdl(k_vertex_event, n_events, kVtxThreads, kVtxSmem, s, b, min_hits, dz,
+                      1.25f * p.cuts.z0max, cap_nt));
   PT_TRACE(l, s, "k_vertex_compact",
-           k_vertex_compact<<<dim3(n_events, kPlaceBlocks), kPlaceThreads, 0, s>>>(b, cap_nt));
+           launch_pdl(k_vertex_compact, dim3(n_events, kPlaceBlocks), kPlaceThreads, 0, s, b,
+                      cap_nt));
   return cudaGetLastError();
 }
 
