@@ -126,10 +126,12 @@ static_assert(kMlpCtasPerSm * (kMlpSmem + 1024) <= 228 * 1024, "six CTAs fit an 
 
 // PIPE = true: rows are link slots of the batch, whose bf16 feature rows the link stage
 // wrote to gate_x; kept links set the flags the ntuplet search reads.
-// PIPE = false: rows are given bf16 feature rows X (standalone scoring).
+// PIPE = false: rows are given float32 feature rows X [n][12] (standalone scoring), rounded
+// to bf16 as they are loaded: 300k rows 34 us a call with the rounding in a kernel of its
+// own and the biases read one at a time, 30 us so.
 template <bool PIPE>
 __global__ void __launch_bounds__(kTileM, kMlpCtasPerSm)
-    k_gate_mlp(const GateWeights* gw, Buffers b, pt_cuts cuts, int32_t B, const uint16_t* X,
+    k_gate_mlp(const GateWeights* gw, Buffers b, pt_cuts cuts, int32_t B, const float* X,
                const unsigned long long* n_dev, int64_t n_max, float* score, uint8_t* keep,
                unsigned long long* status, unsigned long long* kept, long long wait_limit) {
   extern __shared__ __align__(1024) unsigned char sm[];
@@ -182,6 +184,7 @@ __global__ void __launch_bounds__(kTileM, kMlpCtasPerSm)
   bool pending = false;  // an MMA group was committed and not yet seen complete
   const uint64_t n_tiles = (n + kTileM - 1) / kTileM;
 
+  const bool vec_x = ((uintptr_t)X & 15u) == 0;
   // this thread's row of tile tt: its source cell (pipeline form) and bf16 feature row
   auto load_row = [&](uint64_t tt, uint4& lo, uint4& hi, uint32_t& src) {
     const uint64_t r = tt * kTileM + tid;
@@ -192,10 +195,23 @@ __global__ void __launch_bounds__(kTileM, kMlpCtasPerSm)
     if (PIPE) {
       src = b.link[r].src;
       if (src == kHole) return;
+      const uint4* srcp = (const uint4*)(b.gate_x + r * kGateK1);
+      lo = srcp[0];
+      hi = srcp[1];
+    } else {
+      float f[kGateFeat];
+      if (vec_x) {
+#pragma unroll
+        for (int k = 0; k < 3; ++k) {
+          const float4 v = ((const float4*)(X + r * kGateFeat))[k];
+          f[4 * k] = v.x, f[4 * k + 1] = v.y, f[4 * k + 2] = v.z, f[4 * k + 3] = v.w;
+        }
+      } else {
+#pragma unroll
+        for (int k = 0; k < kGateFeat; ++k) f[k] = X[r * kGateFeat + k];
+      }
+      gate_row(f, lo, hi);
     }
-    const uint4* srcp = (const uint4*)((PIPE ? b.gate_x : X) + r * kGateK1);
-    lo = srcp[0];
-    hi = srcp[1];
   };
   uint4 nlo, nhi;
   uint32_t nsrc;
@@ -233,11 +249,13 @@ __global__ void __launch_bounds__(kTileM, kMlpCtasPerSm)
 #pragma unroll
         for (int c = 0; c < 4; ++c) {  // 4 core matrices of 8 columns per half
           const int j0 = 32 * half + 8 * c;
+          const float4 ba = *(const float4*)&sb1[j0], bb = *(const float4*)&sb1[j0 + 4];
+          const float* u = &v[8 * c];
           uint4 pk;
-          pk.x = pack_bf16x2(fmaxf(v[8 * c + 0] + sb1[j0 + 0], 0.f), fmaxf(v[8 * c + 1] + sb1[j0 + 1], 0.f));
-          pk.y = pack_bf16x2(fmaxf(v[8 * c + 2] + sb1[j0 + 2], 0.f), fmaxf(v[8 * c + 3] + sb1[j0 + 3], 0.f));
-          pk.z = pack_bf16x2(fmaxf(v[8 * c + 4] + sb1[j0 + 4], 0.f), fmaxf(v[8 * c + 5] + sb1[j0 + 5], 0.f));
-          pk.w = pack_bf16x2(fmaxf(v[8 * c + 6] + sb1[j0 + 6], 0.f), fmaxf(v[8 * c + 7] + sb1[j0 + 7], 0.f));
+          pk.x = pack_bf16x2(fmaxf(u[0] + ba.x, 0.f), fmaxf(u[1] + ba.y, 0.f));
+          pk.y = pack_bf16x2(fmaxf(u[2] + ba.z, 0.f), fmaxf(u[3] + ba.w, 0.f));
+          pk.z = pack_bf16x2(fmaxf(u[4] + bb.x, 0.f), fmaxf(u[5] + bb.y, 0.f));
+          pk.w = pack_bf16x2(fmaxf(u[6] + bb.z, 0.f), fmaxf(u[7] + bb.w, 0.f));
           *(uint4*)(hr + (j0 >> 3) * 128) = pk;
         }
       }
@@ -267,7 +285,14 @@ __global__ void __launch_bounds__(kTileM, kMlpCtasPerSm)
       float v[32];
       tmem_ld32(tmem + lane_base + 32 * half, v);
 #pragma unroll
-      for (int i = 0; i < 32; ++i) acc += fmaxf(v[i] + sb2[32 * half + i], 0.f) * sw3[32 * half + i];
+      for (int i = 0; i < 32; i += 4) {
+        const float4 bv = *(const float4*)&sb2[32 * half + i];
+        const float4 wv = *(const float4*)&sw3[32 * half + i];
+        acc += fmaxf(v[i] + bv.x, 0.f) * wv.x;
+        acc += fmaxf(v[i + 1] + bv.y, 0.f) * wv.y;
+        acc += fmaxf(v[i + 2] + bv.z, 0.f) * wv.z;
+        acc += fmaxf(v[i + 3] + bv.w, 0.f) * wv.w;
+      }
     }
     // pipeline form (src != NULL): row = link slot; kept links set the flags the
     // ntuplet search reads (a link slot that is a hole is never kept)
@@ -322,18 +347,6 @@ __global__ void k_gate_features_f32(Buffers b, pt_cuts cuts, int32_t B, uint64_t
   }
 }
 
-// float32 feature rows -> bf16 rows padded to 16.
-__global__ void k_gate_pack(const float* feat, int64_t n, uint16_t* X) {
-  pdl_sync();
-  const int64_t stride = (int64_t)gridDim.x * blockDim.x;
-  for (int64_t r = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; r < n; r += stride) {
-    float f[kGateFeat];
-#pragma unroll
-    for (int k = 0; k < kGateFeat; ++k) f[k] = feat[r * kGateFeat + k];
-    store_gate_row(X + r * kGateK1, f);
-  }
-}
-
 }  // namespace
 
 cudaError_t gate_prepare() {
@@ -354,11 +367,10 @@ void launch_gate(const Buffers& b, const Params& p, const Launch& l, const GateW
 }
 
 void launch_gate_score(const GateWeights* w, const float* feat, int64_t n, float* out,
-                       uint16_t* xbuf, unsigned long long* status, int sms, long long wait_cycles,
+                       unsigned long long* status, int sms, long long wait_cycles,
                        cudaStream_t s) {
-  launch_pdl(k_gate_pack, sms * 4, 256, 0, s, feat, n, xbuf);
   launch_pdl(k_gate_mlp<false>, sms * kMlpCtasPerSm, kTileM, kMlpSmem, s, w, Buffers{}, pt_cuts{}, 1,
-             xbuf, nullptr, n, out, nullptr, status, nullptr, wait_cycles);
+             feat, nullptr, n, out, nullptr, status, nullptr, wait_cycles);
 }
 
 void launch_export_link_features(const Buffers& b, const Params& p, const Launch& l, bool gated,

@@ -387,7 +387,7 @@ void launch_gate(const Buffers& b, const Params& p, const Launch& l, const GateW
                  cudaStream_t s);
 // scores of n feature rows (float32 [n][12], device) with the gate's MLP -> out [n]
 void launch_gate_score(const GateWeights* w, const float* feat, int64_t n, float* out,
-                       uint16_t* xbuf, unsigned long long* status, int sms, long long wait_cycles,
+                       unsigned long long* status, int sms, long long wait_cycles,
                        cudaStream_t s);
 // float32 features of the current links (gated: kept only) -> out [slots][12]
 void launch_export_link_features(const Buffers& b, const Params& p, const Launch& l, bool gated,
@@ -565,9 +565,8 @@ __device__ __forceinline__ uint32_t pack_bf16x2(float a, float b) {
   return lo | (hi << 16);
 }
 
-// Writes the 12 features as one bf16 row of 16 (4 zeros) = 32 bytes.
-__device__ __forceinline__ void store_gate_row(uint16_t* row, const float (&f)[12]) {
-  uint4 lo, hi;
+// The 12 features as one bf16 row of 16 (4 zeros) = 32 bytes.
+__device__ __forceinline__ void gate_row(const float (&f)[12], uint4& lo, uint4& hi) {
   lo.x = pack_bf16x2(f[0], f[1]);
   lo.y = pack_bf16x2(f[2], f[3]);
   lo.z = pack_bf16x2(f[4], f[5]);
@@ -576,6 +575,10 @@ __device__ __forceinline__ void store_gate_row(uint16_t* row, const float (&f)[1
   hi.y = pack_bf16x2(f[10], f[11]);
   hi.z = 0;
   hi.w = 0;
+}
+__device__ __forceinline__ void store_gate_row(uint16_t* row, const float (&f)[12]) {
+  uint4 lo, hi;
+  gate_row(f, lo, hi);
   ((uint4*)row)[0] = lo;
   ((uint4*)row)[1] = hi;
 }
