@@ -47,6 +47,7 @@ __global__ void k_clear(Buffers b, int32_t phi_bins) {
     b.cnt[CNT_LINKS_USED] = 0;
     b.cnt[CNT_DBL_WORK] = 0;
     b.cnt[CNT_LNK_WORK] = 0;
+    if (!b.hdr->raw) b.cnt[CNT_RAW_STATUS] = 0;
     b.cnt[CNT_SCAN_BINS] = (unsigned long long)nb;
     b.cnt[CNT_SCAN_HITS] = (unsigned long long)N;
   }
@@ -57,11 +58,18 @@ __device__ __forceinline__ float hit_radius(float x, float y) {
 }
 
 // Histogram: global bin of every input hit and its rank inside the bin; the r and z
-// ranges per (event, layer), reduced within the warp before the atomics.
+// ranges per (event, layer), reduced within the warp before the atomics.  Inputs that the
+// caller has on the device (or that came up with the header) are read where they are and
+// copied to the context's arrays here, instead of by four copies of their own.
 __global__ void k_bin_count(Buffers b, int32_t B) {
   pdl_sync();
   const int E = b.hdr->n_events, N = b.hdr->n_hits;
   const float scale = (float)B / (2.0f * kPi);
+  const bool copy = b.hdr->x != nullptr;
+  const float* X = copy ? b.hdr->x : b.in_x;
+  const float* Y = copy ? b.hdr->y : b.in_y;
+  const float* Z = copy ? b.hdr->z : b.in_z;
+  const uint8_t* LAY = copy ? b.hdr->layer : b.in_layer;
   const int stride = gridDim.x * blockDim.x;
   for (int base = blockIdx.x * blockDim.x; base < N; base += stride) {
     const int g = base + threadIdx.x;
@@ -70,15 +78,21 @@ __global__ void k_bin_count(Buffers b, int32_t B) {
     float r = 0.0f;
     uint32_t zk = 0;
     if (valid) {
-      const int L = b.in_layer[g];
+      const int L = LAY[g];
+      const float x = X[g], y = Y[g], z = Z[g];
+      if (copy) {
+        b.in_x[g] = x;
+        b.in_y[g] = y;
+        b.in_z[g] = z;
+        b.in_layer[g] = (uint8_t)L;
+      }
       if (L >= kLayers) {
         atomicOr(&b.cnt[CNT_STATUS], ST_LAYER);
         b.in_bin[g] = 0xffffffffu;
       } else {
         const int e = find_event(b.hit_off, E, g);
-        const float x = b.in_x[g], y = b.in_y[g];
         r = hit_radius(x, y);
-        zk = float_order_key(b.in_z[g]);
+        zk = float_order_key(z);
         int bin = (int)floorf((atan2f(y, x) + kPi) * scale);
         bin = bin < 0 ? 0 : (bin >= B ? B - 1 : bin);
         key = (uint32_t)(e * kLayers + L);

@@ -62,9 +62,10 @@ __device__ __forceinline__ float gsum(float v) {
   return v;
 }
 
-__global__ void __launch_bounds__(256) k_fit(Buffers b, float bfield) {
+__global__ void __launch_bounds__(256) k_fit(Buffers b, float bfield, bool results) {
   pdl_wait();
   const uint64_t S = b.cnt[CNT_SV];
+  pt_track* out = results && results_go_out(b, S) ? b.hdr->out_tracks : nullptr;
   const int lane = lane_id();
   const int sub = lane & 7;
   const int gbase = lane & ~7;
@@ -175,14 +176,16 @@ __global__ void __launch_bounds__(256) k_fit(Buffers b, float bfield) {
       tr.nhits = (uint8_t)n;
       tr.pad[0] = tr.pad[1] = 0;
       b.tracks[j] = tr;
+      if (out) out[j] = tr;
     }
   }
 }
 
 }  // namespace
 
-void launch_fit(const Buffers& b, const Params& p, const Launch& l, cudaStream_t s) {
-  PT_TRACE(l, s, "k_fit", launch_pdl(k_fit, l.grid, 256, 0, s, b, p.bfield));
+void launch_fit(const Buffers& b, const Params& p, const Launch& l, cudaStream_t s,
+                bool results) {
+  PT_TRACE(l, s, "k_fit", launch_pdl(k_fit, l.grid, 256, 0, s, b, p.bfield, results));
 }
 
 }  // namespace ptca

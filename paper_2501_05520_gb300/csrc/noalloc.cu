@@ -72,6 +72,7 @@ Buffers na_layout(char* base, const float* x, const float* y, const float* z,
 
 __global__ void k_na_header(Buffers b, int32_t n) {
   if (threadIdx.x == 0 && blockIdx.x == 0) {
+    *b.hdr = BatchHeader{};  // the inputs are read in place
     b.hdr->n_events = 1;
     b.hdr->n_hits = n;
     b.hit_off[0] = 0;

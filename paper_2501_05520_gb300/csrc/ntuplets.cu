@@ -395,16 +395,25 @@ __global__ void k_survivors(Buffers b) {
 
 // Place of every survivor: its first hit's, plus the survivors with a smaller tuple on that
 // hit's list.  Per-event offsets and the total come from the places of the events' first
-// hits.  The ntuplet also goes to the export staging, with event-local indices.
+// hits.  The ntuplet also goes out, with event-local indices: to the caller's arrays or, if
+// they do not hold the batch, to the export staging.
 __global__ void k_order(Buffers b) {
   pdl_sync();
   const uint64_t N = b.cnt[CNT_NT_BEST];
   const int E = b.hdr->n_events;
   const uint64_t stride = (uint64_t)gridDim.x * blockDim.x;
   const uint64_t tid = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (tid == 0) b.cnt[CNT_SV] = b.sv_start[b.hdr->n_hits];
-  for (uint64_t e = tid; e <= (uint64_t)E; e += stride)
-    b.ev_nt_off[e] = (int64_t)b.sv_start[b.hit_off[e]];
+  const uint32_t S = b.sv_start[b.hdr->n_hits];
+  if (tid == 0) b.cnt[CNT_SV] = S;
+  const bool direct = results_go_out(b, S);
+  int32_t* out_hits = direct ? b.hdr->out_hits : b.exp_hits;
+  uint8_t* out_n = direct ? b.hdr->out_n : b.exp_n;
+  int64_t* out_off = direct ? b.hdr->out_off : nullptr;
+  for (uint64_t e = tid; e <= (uint64_t)E; e += stride) {
+    const int64_t first = (int64_t)b.sv_start[b.hit_off[e]];
+    b.ev_nt_off[e] = first;
+    if (out_off) out_off[e] = first;
+  }
   for (uint64_t i = tid; i < N; i += stride) {
     const uint32_t t = b.best_list[i];
     if (t == kHole) continue;
@@ -421,13 +430,13 @@ __global__ void k_order(Buffers b) {
       for (uint32_t o = b.nt_head[h[0]]; o != kHole; o = b.nt_next[o])
         if (tuple_less(b.nt_hits + (uint64_t)o * kMaxHits, h)) ++pos;
     b.sv[pos] = t;
-    const int32_t off = b.hit_off[find_event(b.hit_off, E, h[0])];
-    int2* ep = (int2*)(b.exp_hits + (uint64_t)pos * kMaxHits);
+    if (out_hits) {
+      const int32_t off = b.hit_off[find_event(b.hit_off, E, h[0])];
+      int32_t* ep = out_hits + (uint64_t)pos * kMaxHits;  // a caller's array: any 4-byte place
 #pragma unroll
-    for (int k = 0; k < kMaxHits / 2; ++k)
-      ep[k] = make_int2(h[2 * k] >= 0 ? h[2 * k] - off : -1,
-                        h[2 * k + 1] >= 0 ? h[2 * k + 1] - off : -1);
-    b.exp_n[pos] = b.nt_n[t];
+      for (int k = 0; k < kMaxHits; ++k) ep[k] = h[k] >= 0 ? h[k] - off : -1;
+    }
+    if (out_n) out_n[pos] = b.nt_n[t];
   }
 }
 

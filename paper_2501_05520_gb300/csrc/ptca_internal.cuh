@@ -141,10 +141,30 @@ struct alignas(16) LinkBest {
   unsigned long long src, leaf;  // of the source headed by the slot, of the leaf named by it
 };
 
+// What a call says about its batch; the kernels read it, so that one captured graph serves
+// any batch, its inputs wherever they lie and its outputs wherever they go.
 struct BatchHeader {
   int32_t n_events;
   int32_t n_hits;
+  int32_t raw;  // the hits were made from raw digis
+  int32_t pad;
+  // where the binning pass takes the hits from, copying them to in_x, ...  (x NULL: they
+  // are there)
+  const float *x, *y, *z;
+  const uint8_t* layer;
+  // where the whole-batch graph writes the cleaned ntuplets and tracks (each may be NULL)
+  // when there are at most out_cap of them and nothing went wrong; otherwise the ntuplets
+  // go to the export staging
+  int32_t* out_hits;
+  uint8_t* out_n;
+  pt_track* out_tracks;
+  int64_t* out_off;
+  int64_t out_cap;
 };
+constexpr size_t kHeaderBytes = 256;  // hit_off follows, and small host inputs follow that
+static_assert(sizeof(BatchHeader) <= kHeaderBytes, "header fits its place");
+constexpr int64_t kSmallHits = 4096;    // host inputs of up to so many hits go up in one copy
+constexpr int64_t kSmallTracks = 4096;  // up to so many results come back without a copy
 
 // The layer-pair table of a context, as the kernels read it (a kernel argument):
 // outer[L][k], k < n_outer[L], are the outer layers paired with inner layer L, inner[L][k],
@@ -187,7 +207,8 @@ struct Buffers {
   float* in_y;
   float* in_z;
   uint8_t* in_layer;
-  int32_t* hit_off;          // [max_events + 1]
+  int32_t* hit_off;          // [max_events + 1], directly after the header; then room for
+                             //   the inputs of a small batch
   uint32_t* in_bin;          // [max_hits] global bin of input hit (or ~0)
   uint32_t* in_rank;         // [max_hits] rank within the bin
   // hits sorted by (event, layer, phi bin)
@@ -369,7 +390,9 @@ void launch_ntuplets(const Buffers& b, const Params& p, const Launch& l, cudaStr
                      bool gated);
 void launch_ntuplet_steps(const Buffers& b, const Params& p, const Launch& l, cudaStream_t s,
                           bool gated);
-void launch_fit(const Buffers& b, const Params& p, const Launch& l, cudaStream_t s);
+// results: the tracks also go where the batch header says
+void launch_fit(const Buffers& b, const Params& p, const Launch& l, cudaStream_t s,
+                bool results = false);
 // raw digis -> hits in the chain's input arrays, per-event offsets and header
 cudaError_t launch_raw(const RawBuffers& r, const Buffers& b, const pt_module* mods, int n_mod,
                        int64_t cap_hits, const Launch& l, cudaStream_t s);
@@ -645,6 +668,11 @@ __device__ __forceinline__ unsigned long long chunk_take(WarpChunk& ch, unsigned
   ch.next += n;
   ch.total += n;
   return r;
+}
+
+// Whether the batch's S results are written to the arrays in the header.
+__device__ __forceinline__ bool results_go_out(const Buffers& b, unsigned long long S) {
+  return (int64_t)S <= b.hdr->out_cap && b.cnt[CNT_STATUS] == 0;
 }
 
 // Event owning batch hit g: largest e with off[e] <= g (empty events are skipped).

@@ -358,6 +358,8 @@ __global__ void k_raw_place(RawBuffers r, Buffers b, int64_t cap_hits, unsigned 
   const int64_t tid = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (tid == 0) {
     if ((int64_t)H > cap_hits) atomicOr(status, RAW_HIT_CAPACITY);
+    *b.hdr = BatchHeader{};
+    b.hdr->raw = 1;
     b.hdr->n_events = E;
     b.hdr->n_hits = (int32_t)min((int64_t)H, cap_hits);
     r.cnt[CNT_RAW_HITS] = H;

@@ -147,6 +147,13 @@ pt_status fail(pt_status st, const char* fmt, ...) {
 
 constexpr size_t kAlign = 256;
 
+// The header, the events' offsets and the inputs of a small batch, which go up in one copy
+// from a pinned block of the same layout.
+size_t stage_bytes(const pt_capacity& c) {
+  return kHeaderBytes + (size_t)(c.max_events + 1) * 4 +
+         (size_t)std::min(c.max_hits, kSmallHits) * 13;
+}
+
 // Carves the workspace; with base == nullptr only computes the size.
 size_t layout(const pt_capacity& c, char* base, Buffers* b, GateWeights** gate = nullptr) {
   size_t off = 0;
@@ -160,13 +167,13 @@ size_t layout(const pt_capacity& c, char* base, Buffers* b, GateWeights** gate =
   const size_t L = (size_t)c.max_links, T = (size_t)c.max_ntuplets;
   const size_t NB = E * kLayers * (size_t)c.phi_bins + 1;
   Buffers t{};
-  t.hdr = (BatchHeader*)take(sizeof(BatchHeader));
+  t.hdr = (BatchHeader*)take(stage_bytes(c));
+  t.hit_off = (int32_t*)(base ? base + kHeaderBytes : nullptr);
   t.cnt = (unsigned long long*)take(CNT_N * 8);
   t.in_x = (float*)take(N * 4);
   t.in_y = (float*)take(N * 4);
   t.in_z = (float*)take(N * 4);
   t.in_layer = (uint8_t*)take(N);
-  t.hit_off = (int32_t*)take((E + 1) * 4);
   t.in_bin = (uint32_t*)take(N * 4);
   t.in_rank = (uint32_t*)take(N * 4);
   t.hit4 = (float4*)take(N * 16);
@@ -257,10 +264,16 @@ struct pt_ctx {
   bool fitted = false;     // the tracks of the loaded batch are fitted
   bool vtx_ready = false;  // pt_find_vertices ran on the loaded batch
   std::vector<int64_t> hit_off;
-  // pinned staging
-  int32_t* h_off = nullptr;
-  BatchHeader* h_hdr = nullptr;
+  // one pinned block: header, offsets and small inputs on the way up; counters and the
+  // results of a small batch (kSmallTracks), which the kernels write, on the way down
+  char* h_stage = nullptr;
+  BatchHeader* h_hdr = nullptr;  // in h_stage
+  int32_t* h_off = nullptr;      // in h_stage
   unsigned long long* h_cnt = nullptr;
+  int64_t* r_off = nullptr;
+  pt_track* r_tracks = nullptr;
+  int32_t* r_hits = nullptr;
+  uint8_t* r_n = nullptr;
   cudaEvent_t staged = nullptr;
   cudaGraphExec_t graph = nullptr;
   // validation staging, allocated on first use
@@ -352,8 +365,32 @@ pt_status check_status(pt_ctx* c) {
   return PT_OK;
 }
 
+// Device memory of the context's own GPU, which its kernels may use in place.
+bool own_device_memory(const pt_ctx* c, const void* p) {
+  cudaPointerAttributes a;
+  if (cudaPointerGetAttributes(&a, p) != cudaSuccess) {
+    cudaGetLastError();
+    return false;
+  }
+  return a.type == cudaMemoryTypeDevice && a.device == c->device;
+}
+
+// Where a whole-batch call wants its results (see BatchHeader).
+struct Results {
+  int32_t* hits = nullptr;
+  uint8_t* n = nullptr;
+  pt_track* tracks = nullptr;
+  int64_t* off = nullptr;
+  int64_t cap = -1;
+};
+
+// Header, offsets and inputs of a batch to the device.  A few copies cost more than they
+// move: one 50-particle event took 30 us to stage in six, so a small batch from the host
+// goes up in one, packed behind the header, and arrays that the caller has on the device
+// are left to the binning pass to copy.
 pt_status stage_inputs(pt_ctx* c, int n_events, const int64_t* off, const float* x,
-                       const float* y, const float* z, const uint8_t* layer, int on_device) {
+                       const float* y, const float* z, const uint8_t* layer, int on_device,
+                       const Results& out = {}) {
   if (n_events < 1) return fail(PT_ERR_INVALID, "n_events must be >= 1");
   if (n_events > c->cap.max_events)
     return fail(PT_ERR_CAPACITY, "max_events = %lld is too small: %d events given",
@@ -367,21 +404,51 @@ pt_status stage_inputs(pt_ctx* c, int n_events, const int64_t* off, const float*
     return fail(PT_ERR_CAPACITY, "max_hits = %lld is too small: %lld hits given",
                 (long long)c->cap.max_hits, (long long)n);
   if (n > 0 && (!x || !y || !z || !layer)) return fail(PT_ERR_INVALID, "hit array is NULL");
-  if (!on_device)
-    for (int64_t i = 0; i < n; ++i)
+  if (!on_device) {
+    uint8_t most = 0;
+    for (int64_t i = 0; i < n; ++i) most = std::max(most, layer[i]);  // vectorises
+    for (int64_t i = 0; most >= kLayers && i < n; ++i)
       if (layer[i] >= kLayers)
         return fail(PT_ERR_INVALID, "layer code %d > 9 at hit %lld", (int)layer[i], (long long)i);
+  }
   // the pinned staging of the previous call must have been consumed
   PT_CUDA(cudaEventSynchronize(c->staged));
-  PT_CUDA(cudaMemsetAsync(&c->B.cnt[CNT_RAW_STATUS], 0, 8, c->stream));
+  BatchHeader& h = *c->h_hdr;
+  h = BatchHeader{};
+  h.n_events = n_events;
+  h.n_hits = (int32_t)n;
+  h.out_hits = out.hits;
+  h.out_n = out.n;
+  h.out_tracks = out.tracks;
+  h.out_off = out.off;
+  h.out_cap = out.cap;
   for (int e = 0; e <= n_events; ++e) c->h_off[e] = (int32_t)off[e];
-  c->h_hdr->n_events = n_events;
-  c->h_hdr->n_hits = (int32_t)n;
-  PT_CUDA(cudaMemcpyAsync(c->B.hit_off, c->h_off, (n_events + 1) * 4, cudaMemcpyHostToDevice,
-                          c->stream));
-  PT_CUDA(cudaMemcpyAsync(c->B.hdr, c->h_hdr, sizeof(BatchHeader), cudaMemcpyHostToDevice,
-                          c->stream));
-  if (n > 0) {
+  const size_t head = kHeaderBytes + (size_t)(n_events + 1) * 4;
+  size_t up = head;
+  bool copies = n > 0;
+  if (n > 0 && !on_device && n <= kSmallHits) {
+    char* p = c->h_stage + head;
+    std::memcpy(p, x, n * 4);
+    std::memcpy(p + n * 4, y, n * 4);
+    std::memcpy(p + n * 8, z, n * 4);
+    std::memcpy(p + n * 12, layer, n);
+    const char* d = (const char*)c->B.hdr + head;
+    h.x = (const float*)d;
+    h.y = h.x + n;
+    h.z = h.y + n;
+    h.layer = (const uint8_t*)(h.z + n);
+    up = head + (size_t)n * 13;
+    copies = false;
+  } else if (n > 0 && on_device && own_device_memory(c, x) && own_device_memory(c, y) &&
+             own_device_memory(c, z) && own_device_memory(c, layer)) {
+    h.x = x;
+    h.y = y;
+    h.z = z;
+    h.layer = layer;
+    copies = false;
+  }
+  PT_CUDA(cudaMemcpyAsync(c->B.hdr, c->h_stage, up, cudaMemcpyHostToDevice, c->stream));
+  if (copies) {
     const cudaMemcpyKind k = on_device ? cudaMemcpyDeviceToDevice : cudaMemcpyHostToDevice;
     PT_CUDA(cudaMemcpyAsync(c->B.in_x, x, n * 4, k, c->stream));
     PT_CUDA(cudaMemcpyAsync(c->B.in_y, y, n * 4, k, c->stream));
@@ -408,7 +475,8 @@ void enqueue_pipeline(pt_ctx* c, cudaStream_t s) {
   if (c->gate_on) launch_gate(c->B, c->P, L, c->gate, s);
   if (c->fishbone_on) launch_fishbone(c->B, c->P, L, s, c->gate_on);
   launch_ntuplets(c->B, c->P, L, s, c->masked());
-  launch_fit(c->B, c->P, L, s);
+  launch_fit(c->B, c->P, L, s, true);
+  cudaMemcpyAsync(c->h_cnt, c->B.cnt, CNT_N * 8, cudaMemcpyDeviceToHost, s);
 }
 
 pt_status ensure_graph(pt_ctx* c) {
@@ -463,8 +531,7 @@ void set_last_error(const char* msg) { g_err = msg; }
 cudaStream_t ctx_stream(pt_ctx* c) { return c->stream; }
 
 pt_status ctx_counters_async(pt_ctx* c, cudaEvent_t done) {
-  DeviceGuard guard(c->device);
-  PT_CUDA(cudaMemcpyAsync(c->h_cnt, c->B.cnt, CNT_N * 8, cudaMemcpyDeviceToHost, c->stream));
+  DeviceGuard guard(c->device);  // the batch's graph ends with the counters' copy
   PT_CUDA(cudaEventRecord(done, c->stream));
   return PT_OK;
 }
@@ -555,10 +622,19 @@ pt_status pt_create(const pt_geometry* geom, const pt_cuts* cuts, const pt_capac
     c->own_ws = true;
   }
   layout(*cap, c->ws, &c->B, &c->gate);
-  if (cudaMallocHost(&c->h_off, (cap->max_events + 1) * 4) != cudaSuccess ||
-      cudaMallocHost(&c->h_hdr, sizeof(BatchHeader)) != cudaSuccess ||
-      cudaMallocHost(&c->h_cnt, CNT_N * 8) != cudaSuccess)
+  const size_t small = (size_t)std::min(cap->max_ntuplets, kSmallTracks);
+  const size_t off_bytes = (size_t)(cap->max_events + 1) * 8;
+  const size_t up_bytes = (stage_bytes(*cap) + 7) / 8 * 8;
+  if (cudaMallocHost(&c->h_stage, up_bytes + CNT_N * 8 + off_bytes +
+                                      small * (sizeof(pt_track) + kMaxHits * 4 + 1)) != cudaSuccess)
     return bail(fail(PT_ERR_NOMEM, "pinned host allocation failed"));
+  c->h_hdr = (BatchHeader*)c->h_stage;
+  c->h_off = (int32_t*)(c->h_stage + kHeaderBytes);
+  c->h_cnt = (unsigned long long*)(c->h_stage + up_bytes);
+  c->r_off = (int64_t*)(c->h_cnt + CNT_N);
+  c->r_tracks = (pt_track*)((char*)c->r_off + off_bytes);
+  c->r_hits = (int32_t*)(c->r_tracks + small);
+  c->r_n = (uint8_t*)(c->r_hits + small * kMaxHits);
   if (cudaEventCreateWithFlags(&c->staged, cudaEventDisableTiming) != cudaSuccess)
     return bail(fail(PT_ERR_CUDA, "cudaEventCreate failed"));
   if (stream) {
@@ -584,9 +660,7 @@ pt_status pt_destroy(pt_ctx* c) {
   if (c->raw_mem) cudaFree(c->raw_mem);
   if (c->bl_mem) cudaFree(c->bl_mem);
   if (c->own_ws && c->ws) cudaFree(c->ws);
-  if (c->h_off) cudaFreeHost(c->h_off);
-  if (c->h_hdr) cudaFreeHost(c->h_hdr);
-  if (c->h_cnt) cudaFreeHost(c->h_cnt);
+  if (c->h_stage) cudaFreeHost(c->h_stage);
   if (c->staged) cudaEventDestroy(c->staged);
   delete c->L.tr;
   if (c->own_stream && c->stream) cudaStreamDestroy(c->stream);
@@ -840,19 +914,19 @@ pt_status pt_load_raw(pt_ctx* c, int n_events, const int64_t* off, const uint64_
   c->R.n_events = n_events;
   c->R.scan_part = c->B.scan_part;
   c->R.cnt = c->B.cnt;
-  PT_CUDA(cudaStreamSynchronize(c->stream));  // the previous batch no longer needs its inputs
   PT_CUDA(cudaMemcpyAsync(c->R.digi_off, off, (size_t)(n_events + 1) * 8, cudaMemcpyHostToDevice,
                           c->stream));
   if (n > 0)
     PT_CUDA(cudaMemcpyAsync(c->R.words, digis, (size_t)n * 8,
                             on_device ? cudaMemcpyDeviceToDevice : cudaMemcpyHostToDevice,
                             c->stream));
+  PT_CUDA(cudaEventRecord(c->staged, c->stream));
   PT_CUDA(cudaMemsetAsync(&c->B.cnt[CNT_RAW_STATUS], 0, 8, c->stream));
   PT_CUDA(launch_raw(c->R, c->B, c->modules, c->n_modules, c->cap.max_hits, c->L, c->stream));
   launch_clear(c->B, c->P, c->L, c->stream);
   launch_bin_hits(c->B, c->P, c->L, c->stream);
   PT_TRY(last_launch());
-  PT_CUDA(cudaStreamSynchronize(c->stream));  // the host offsets and digis may be reused
+  PT_CUDA(cudaEventSynchronize(c->staged));  // the caller's offsets and digis may be reused
   c->n_events = n_events;
   c->n_hits = -1;
   c->hit_off.clear();
@@ -872,10 +946,7 @@ pt_status pt_get_hits(pt_ctx* c, float* x, float* y, float* z, uint8_t* layer,
   PT_TRY(need_loaded(c));
   DeviceGuard guard(c->device);
   PT_TRY(sync_counters(c));
-  BatchHeader hdr{};
-  PT_CUDA(cudaMemcpyAsync(&hdr, c->B.hdr, sizeof(hdr), cudaMemcpyDeviceToHost, c->stream));
-  PT_CUDA(cudaStreamSynchronize(c->stream));
-  const int64_t N = hdr.n_hits;
+  const int64_t N = (int64_t)c->h_cnt[CNT_SCAN_HITS];
   if (n) *n = N;
   if (cap < N)
     return fail(PT_ERR_CAPACITY, "output capacity %lld is too small: %lld hits", (long long)cap,
@@ -884,12 +955,11 @@ pt_status pt_get_hits(pt_ctx* c, float* x, float* y, float* z, uint8_t* layer,
   PT_TRY(copy_out(c, y, c->B.in_y, (size_t)N * 4, 0));
   PT_TRY(copy_out(c, z, c->B.in_z, (size_t)N * 4, 0));
   PT_TRY(copy_out(c, layer, c->B.in_layer, (size_t)N, 0));
-  std::vector<int32_t> off32((size_t)c->n_events + 1);
-  PT_CUDA(cudaMemcpyAsync(off32.data(), c->B.hit_off, off32.size() * 4, cudaMemcpyDeviceToHost,
-                          c->stream));
+  const size_t m = (size_t)c->n_events + 1;  // the stream is idle: h_off is free
+  PT_CUDA(cudaMemcpyAsync(c->h_off, c->B.hit_off, m * 4, cudaMemcpyDeviceToHost, c->stream));
   PT_CUDA(cudaStreamSynchronize(c->stream));
   if (event_offsets)
-    for (size_t e = 0; e < off32.size(); ++e) event_offsets[e] = off32[e];
+    for (size_t e = 0; e < m; ++e) event_offsets[e] = c->h_off[e];
   return PT_OK;
 }
 
@@ -1318,17 +1388,40 @@ pt_status pt_reconstruct_batch(pt_ctx* c, int n_events, const int64_t* hit_offse
   if (!c) return fail(PT_ERR_INVALID, "context is NULL");
   if (!event_offsets) return fail(PT_ERR_INVALID, "event_offsets is NULL");
   DeviceGuard guard(c->device);
-  PT_TRY(stage_inputs(c, n_events, hit_offsets, x, y, z, layer, on_device));
+  // results the kernels write in place: device arrays, or (small batches for the host) the
+  // pinned block; anything else is copied once the counts are known
+  Results out;
+  const bool in_place =
+      out_on_device && own_device_memory(c, event_offsets) &&
+      (!hits_out || own_device_memory(c, hits_out)) &&
+      (!nhits_out || own_device_memory(c, nhits_out)) &&
+      (!tracks_out || own_device_memory(c, tracks_out));
+  if (in_place) {
+    out = {hits_out, nhits_out, tracks_out, event_offsets, cap};
+  } else if (!out_on_device) {
+    out = {c->r_hits, c->r_n, c->r_tracks, c->r_off,
+           std::min({cap, (int64_t)c->cap.max_ntuplets, kSmallTracks})};
+  }
+  PT_TRY(stage_inputs(c, n_events, hit_offsets, x, y, z, layer, on_device, out));
   PT_TRY(ensure_graph(c));
   PT_CUDA(cudaGraphLaunch(c->graph, c->stream));
   c->fitted = true;
   c->links_masked = c->masked();  // the graph's link stage ran in the current form
-  PT_TRY(sync_counters(c));
+  PT_CUDA(cudaStreamSynchronize(c->stream));  // the graph ends with the counters' copy
+  PT_TRY(check_status(c));
   const int64_t S = (int64_t)c->h_cnt[CNT_SV];
   if (n) *n = S;
   if (cap < S)
     return fail(PT_ERR_CAPACITY, "output capacity %lld is too small: %lld ntuplets",
                 (long long)cap, (long long)S);
+  if (S <= out.cap) {
+    if (in_place) return PT_OK;
+    if (hits_out) std::memcpy(hits_out, c->r_hits, (size_t)S * kMaxHits * 4);
+    if (nhits_out) std::memcpy(nhits_out, c->r_n, (size_t)S);
+    if (tracks_out) std::memcpy(tracks_out, c->r_tracks, (size_t)S * sizeof(pt_track));
+    std::memcpy(event_offsets, c->r_off, (size_t)(n_events + 1) * 8);
+    return PT_OK;
+  }
   PT_TRY(copy_out(c, hits_out, c->B.exp_hits, (size_t)S * kMaxHits * 4, out_on_device));
   PT_TRY(copy_out(c, nhits_out, c->B.exp_n, (size_t)S, out_on_device));
   PT_TRY(copy_out(c, tracks_out, c->B.tracks, (size_t)S * sizeof(pt_track), out_on_device));
