@@ -33,9 +33,10 @@
 //
 // The target cell (h1, h2) of a link is found afterwards, one thread per link, in h2's
 // incoming segment from h1's layer (ordered by inner hit): in the warp's own path those
-// dependent loads would hold up the search.  A middle hit with
-// more outgoing cells than the stage holds is handled piece by piece, every incoming
-// group visiting every piece.
+// dependent loads would hold up the search.  A middle hit with more outgoing cells than the
+// stage holds is handled piece by piece, every piece staged once and visited by all of the
+// incoming groups (staged again for each group, the search of 7 gap-pair events, with some
+// 150 outgoing cells a hit, took 693 instead of 492 us).
 #include "ptca_internal.cuh"
 
 namespace ptca {
@@ -46,11 +47,11 @@ constexpr float kTwoPi = 6.28318530717958647692f;
 constexpr float kHalfPi = 1.57079632679489661923f;
 constexpr int kConnWarps = 8;
 constexpr int kConnBlocksPerSm = 4;  // 64 registers per thread
-constexpr int kOut = 128;            // staged outgoing cells of one piece (<= 256)
+constexpr int kOut = 128;            // staged outgoing cells of one piece
 constexpr int kNb = 128;             // slope buckets of a piece (a multiple of 32)
 static_assert(kNb % 32 == 0, "buckets are scanned kNb / 32 per lane");
 constexpr int kQueue = 64;           // window pairs waiting for C1-C3 (power of two)
-static_assert(kOut <= 256 && kOut % 32 == 0, "staged index fits 8 bits");
+static_assert(kOut % 32 == 0, "staged cells are sorted 32 at a time");
 static_assert(kQueue >= 63 && (kQueue & (kQueue - 1)) == 0, "queue holds 31 + 32 entries");
 
 // Azimuthal window of inner hit `hi` (global bin gb, asin_i = asin(kmax*ri/2)) towards
@@ -108,8 +109,8 @@ struct ConnWarp {
   float t[kOut];             // staged outgoing cells: r-z slope
   uint32_t code[kOut];       //   outer hit (sorted index) | slot of the middle hit's layer
                              //   among the outer hit's inner layers << 29
-  uint8_t perm[kOut];        // bucket order -> staged index
   float ts[kOut];            // slopes in bucket order
+  uint32_t cs[kOut];         //   and codes
   uint32_t bstart[kNb + 1];  // first bucket-ordered position of each slope bucket
   float4 qp0[kQueue];        // window pairs: the source's inner hit (x, y, z, r)
   uint4 q[kQueue];           //   source cell, target (outer hit | slot << 29), middle hit,
@@ -120,9 +121,9 @@ struct ConnWarp {
   uint32_t sb[kMaxInner + 1];  //   incoming cells before each segment (the last: all)
   float tmin, scale, m;      // the staged piece: slope origin and scale of the buckets,
                              //   smallest r2 - r1
-  int piece;                 // the staged piece (-1: none)
   unsigned long long chunk_next, chunk_end;  // link slots
   uint32_t used;             //   handed out
+  uint32_t s0, per, dyn0;    // its chunk of sorted hits: first, size; the counter's first one
   float ahead;               //   search_ahead of the warp's hits
 };
 
@@ -227,12 +228,16 @@ __global__ void __launch_bounds__(kConnWarps * 32, kConnBlocksPerSm)
   };
 
   const uint32_t n_warps = gridDim.x * kConnWarps;
-  const uint32_t per = search_chunk(n_sorted, n_warps);
   // chunks of sorted middle hits, the first by the warp's number, the others from a work
-  // counter
-  uint32_t chunk = blockIdx.x * kConnWarps + (threadIdx.x >> 5);
+  // counter (the chunk in shared memory: the kernel's 64 registers are all in use)
+  if (lane == 0) {
+    W.per = search_chunk(n_sorted, n_warps);
+    W.dyn0 = W.per * n_warps;
+    W.s0 = (blockIdx.x * kConnWarps + (threadIdx.x >> 5)) * W.per;
+  }
+  __syncwarp();
   for (;;) {
-    const uint32_t s0 = chunk * per;  // < n_sorted + 2 * per * n_warps < 2^32
+    const uint32_t s0 = W.s0, per = W.per;
     if (s0 >= n_sorted) break;
     // one round of loads finds the hits with incoming cells and outer layers
     uint32_t my_gb = 0;
@@ -254,7 +259,7 @@ __global__ void __launch_bounds__(kConnWarps * 32, kConnBlocksPerSm)
     while (todo) {
       const int src = __ffs(todo) - 1;
       todo &= todo - 1;
-      const uint32_t h1 = s0 + src;
+      const uint32_t h1 = W.s0 + src;
       const uint32_t gb = __shfl_sync(kFull, my_gb, src);
       const int L1 = (gb / (uint32_t)B) % kLayers;
       const float4 p1 = b.hit4[h1];
@@ -280,10 +285,7 @@ __global__ void __launch_bounds__(kConnWarps * 32, kConnBlocksPerSm)
           rg = make_uint4(0u, 0u, 0u, 0u);
         W.rg[lane] = rg;
       }
-      if (lane == 0) {
-        W.ahead = search_ahead(n_sorted, h1 + 1);
-        W.piece = -1;
-      }
+      if (lane == 0) W.ahead = search_ahead(n_sorted, h1 + 1);
       __syncwarp();
       const uint32_t nin = W.sb[kMaxInner];
 
@@ -330,12 +332,9 @@ __global__ void __launch_bounds__(kConnWarps * 32, kConnBlocksPerSm)
             }
           }
         }
-#pragma unroll
-        for (int off = 16; off > 0; off >>= 1) {
-          m = fminf(m, __shfl_xor_sync(kFull, m, off));
-          tlo = fminf(tlo, __shfl_xor_sync(kFull, tlo, off));
-          thi = fmaxf(thi, __shfl_xor_sync(kFull, thi, off));
-        }
+        asm volatile("redux.sync.min.f32 %0, %0, 0xffffffff;" : "+f"(m));
+        asm volatile("redux.sync.min.f32 %0, %0, 0xffffffff;" : "+f"(tlo));
+        asm volatile("redux.sync.max.f32 %0, %0, 0xffffffff;" : "+f"(thi));
         const uint32_t n = cnt > lo_ord ? min(cnt - lo_ord, (uint32_t)kOut) : 0u;
         const float scale = thi - tlo > 1e-6f ? __fdiv_rn((float)kNb, thi - tlo) : 0.0f;
         // counting sort of the staged cells by slope bucket
@@ -377,7 +376,7 @@ __global__ void __launch_bounds__(kConnWarps * 32, kConnBlocksPerSm)
           const uint32_t st = lane + 32 * u;
           if (st < n) {
             const uint32_t sp = W.bstart[key[u]] + rank[u];
-            W.perm[sp] = (uint8_t)st;
+            W.cs[sp] = W.code[st];
             W.ts[sp] = W.t[st];
           }
         }
@@ -385,7 +384,6 @@ __global__ void __launch_bounds__(kConnWarps * 32, kConnBlocksPerSm)
           W.tmin = tlo;
           W.scale = scale;
           W.m = m;
-          W.piece = piece;
         }
         __syncwarp();
         return cnt;
@@ -397,49 +395,58 @@ __global__ void __launch_bounds__(kConnWarps * 32, kConnBlocksPerSm)
         while (i >= W.sb[kin + 1]) ++kin;  // i < W.sb[max_inner] bounds the walk
         return W.so[kin] + (i - W.sb[kin]);
       };
-      // the first incoming group's inner hits are fetched while the outgoing cells are
-      // searched, each later group's while the group before it is processed
-      float4 p0_next = make_float4(0.f, 0.f, 0.f, 0.f);
-      if ((uint32_t)lane < nin) {
-        int kin;
-        const uint32_t c0 = incoming(lane, kin);
-        if (PT_CHECK(b.cnt, c0 < b.cnt[CNT_CELLS], DBG_CON_INCOMING))
-          p0_next = b.hit4[b.cell_in[c0]];
-      }
-      const uint32_t nout = stage_piece(0);
-      if (nout == 0) continue;
-
-      const int npieces = (int)((nout + kOut - 1) / kOut);
-
-      for (uint32_t g0 = 0; g0 < nin; g0 += 32) {
-        // the lane's incoming cell
-        const uint32_t i = g0 + lane;
-        bool valid = i < nin;
-        uint32_t c = 0;
-        int kin = 0;
-        if (valid) {
-          c = incoming(i, kin);
-          valid = PT_CHECK(b.cnt, c < b.cnt[CNT_CELLS], DBG_CON_INCOMING);
-        }
-        const float4 p0 = p0_next;
-        const bool first_b0 = valid && pt.inner[L1][kin] == 0;
-        uint32_t h0_next = 0;
-        const bool valid_next = i + 32 < nin;
-        if (valid_next) {
-          int kn;
-          const uint32_t cn = incoming(i + 32, kn);
-          if (PT_CHECK(b.cnt, cn < b.cnt[CNT_CELLS], DBG_CON_INCOMING)) h0_next = b.cell_in[cn];
-        }
-        const float ta = __fdividef(p1.z - p0.z, p1.w - p0.w);  // the cell's slope dz/dr
-        const float id1 = __fdividef(1.0f, p1.w - p0.w);
-        const float wa = (cuts.rz0 + cuts.rz1 * cuts.cotmax) * id1;
-        const float ua = cuts.rz0 + cuts.rz1 * fabsf(ta);
-        const float shrink = 1.0f - cuts.rz1 * id1;
-
-        bool inited = false;  // the lane's cell had its state set up
+      // Every piece of the outgoing cells is staged once and visited by all incoming groups.
+      // With more than one piece a cell's pairs come up again after some were tested, so
+      // all incoming cells have their state set up first.
+      uint32_t nout = 0;
 #pragma unroll 1
-        for (int piece = 0; piece < npieces; ++piece) {
-          if (W.piece != piece) stage_piece(piece);
+      for (int piece = 0; piece == 0 || (uint32_t)piece * kOut < nout; ++piece) {
+        // the first incoming group's inner hits are fetched while the outgoing cells are
+        // searched, each later group's while the group before it is processed
+        float4 p0_next = make_float4(0.f, 0.f, 0.f, 0.f);
+        if ((uint32_t)lane < nin) {
+          int kin;
+          const uint32_t c0 = incoming(lane, kin);
+          if (PT_CHECK(b.cnt, c0 < b.cnt[CNT_CELLS], DBG_CON_INCOMING))
+            p0_next = b.hit4[b.cell_in[c0]];
+        }
+        nout = stage_piece(piece);
+        if (nout == 0) break;
+        if (piece == 0 && nout > (uint32_t)kOut) {
+          for (uint32_t i = lane; i < nin; i += 32) {
+            int kin;
+            const uint32_t c = incoming(i, kin);
+            if (PT_CHECK(b.cnt, c < b.cnt[CNT_CELLS], DBG_CON_INCOMING))
+              *(uint2*)&b.cell[c] = make_uint2(kHole, 0u);
+          }
+        }
+#pragma unroll 1
+        for (uint32_t g0 = 0; g0 < nin; g0 += 32) {
+          // the lane's incoming cell
+          const uint32_t i = g0 + lane;
+          bool valid = i < nin;
+          uint32_t c = 0;
+          int kin = 0;
+          if (valid) {
+            c = incoming(i, kin);
+            valid = PT_CHECK(b.cnt, c < b.cnt[CNT_CELLS], DBG_CON_INCOMING);
+          }
+          const float4 p0 = p0_next;
+          const bool first_b0 = valid && pt.inner[L1][kin] == 0;
+          uint32_t h0_next = 0;
+          const bool valid_next = i + 32 < nin;
+          if (valid_next) {
+            int kn;
+            const uint32_t cn = incoming(i + 32, kn);
+            if (PT_CHECK(b.cnt, cn < b.cnt[CNT_CELLS], DBG_CON_INCOMING)) h0_next = b.cell_in[cn];
+          }
+          const float ta = __fdividef(p1.z - p0.z, p1.w - p0.w);  // the cell's slope dz/dr
+          const float id1 = __fdividef(1.0f, p1.w - p0.w);
+          const float wa = (cuts.rz0 + cuts.rz1 * cuts.cotmax) * id1;
+          const float ua = cuts.rz0 + cuts.rz1 * fabsf(ta);
+          const float shrink = 1.0f - cuts.rz1 * id1;
+
+          bool inited = nout > (uint32_t)kOut;  // the lane's cell had its state set up
           const float m = W.m, tmin = W.tmin, scale = W.scale;
           float w = 0.0f;
           uint32_t pos = 0, pend = 0;
@@ -464,8 +471,7 @@ __global__ void __launch_bounds__(kConnWarps * 32, kConnBlocksPerSm)
               if (pass) {
                 // the target cell, named by its outer hit and the slot of h1's layer
                 // among that hit's inner layers until k_link_targets finds it
-                const uint32_t st = W.perm[pos];
-                code = W.code[st];
+                code = W.cs[pos];
                 if (!inited) {
                   // before any of its pairs is tested: no links, no flags
                   *(uint2*)&b.cell[c] = make_uint2(kHole, 0u);
@@ -484,12 +490,17 @@ __global__ void __launch_bounds__(kConnWarps * 32, kConnBlocksPerSm)
             qtail += __popc(bal);
             if (qtail - qhead >= 32u) process(32u);
           }
+          if (valid_next) p0_next = b.hit4[h0_next];
         }
-        if (valid_next) p0_next = b.hit4[h0_next];
       }
     }
-    if (lane == 0) chunk = n_warps + (uint32_t)atomicAdd(&b.cnt[CNT_LNK_WORK], 1ull);
-    chunk = __shfl_sync(kFull, chunk, 0);
+    __syncwarp();
+    if (lane == 0) {
+      const uint32_t next = search_chunk(n_sorted - W.s0, n_warps);
+      W.per = next;
+      W.s0 = W.dyn0 + (uint32_t)atomicAdd(&b.cnt[CNT_LNK_WORK], (unsigned long long)next);
+    }
+    __syncwarp();
   }
   while (qtail != qhead) process(min(32u, qtail - qhead));
   __syncwarp();

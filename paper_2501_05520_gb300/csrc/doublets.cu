@@ -100,9 +100,10 @@ __global__ void __launch_bounds__(kWarpsPerBlock * 32, 5)
   WarpChunk ch;
 
   const uint32_t n_warps = gridDim.x * kWarpsPerBlock;
-  const uint32_t per = search_chunk(n_sorted, n_warps);
-  for (uint32_t chunk = blockIdx.x * kWarpsPerBlock + wib;;) {
-    const uint32_t s0 = chunk * per;  // < n_sorted + 2 * per * n_warps < 2^32
+  for (uint32_t s0 = 0;;) {
+    const uint32_t per = search_chunk(n_sorted - s0, n_warps);
+    if (lane == 0) s0 = (uint32_t)atomicAdd(&b.cnt[CNT_DBL_WORK], (unsigned long long)per);
+    s0 = __shfl_sync(kFull, s0, 0);
     if (s0 >= n_sorted) break;
     const uint32_t nh = min(per, n_sorted - s0);
     __syncwarp();
@@ -197,8 +198,6 @@ __global__ void __launch_bounds__(kWarpsPerBlock * 32, 5)
         __syncwarp();
       }
     }
-    if (lane == 0) chunk = n_warps + (uint32_t)atomicAdd(&b.cnt[CNT_DBL_WORK], 1ull);
-    chunk = __shfl_sync(kFull, chunk, 0);
   }
   if (lane == 0 && ch.total) atomicAdd(&b.cnt[CNT_CELLS_USED], (unsigned long long)ch.total);
 }

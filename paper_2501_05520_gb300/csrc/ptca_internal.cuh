@@ -481,14 +481,18 @@ __device__ __forceinline__ bool rz_box_reachable(const pt_cuts& c, float r, floa
 
 // Doublet cuts D0..D4 on (x, y, z, r) of the inner and outer hit, in the library's
 // fixed evaluation order (see pt_cuts in pt_ca.h).
+// The four cheap cuts are all evaluated before one branch skips the square root: leaving at
+// each of them took 1463 instead of 1432 us in the doublet search of 64 pileup-200 events,
+// no branch at all 3 % longer than that in the link search.
 __device__ __forceinline__ bool doublet_pass(const pt_cuts& c, float4 hi, float4 ho) {
   const float dx = fsub(ho.x, hi.x), dy = fsub(ho.y, hi.y);
   const float dr = fsub(ho.w, hi.w), dz = fsub(ho.z, hi.z);
-  if (!(dr > 0.0f)) return false;
-  if (!(fadd(fmul(hi.x, ho.x), fmul(hi.y, ho.y)) > 0.0f)) return false;
-  if (!(fabsf(fsub(fmul(hi.z, dr), fmul(hi.w, dz))) <= fmul(c.z0max, dr))) return false;
-  if (!(fabsf(dz) <= fmul(c.cotmax, dr))) return false;
+  const bool d0 = dr > 0.0f;
+  const bool d1 = fadd(fmul(hi.x, ho.x), fmul(hi.y, ho.y)) > 0.0f;
+  const bool d3 = fabsf(fsub(fmul(hi.z, dr), fmul(hi.w, dz))) <= fmul(c.z0max, dr);
+  const bool d4 = fabsf(dz) <= fmul(c.cotmax, dr);
   const float l2 = fmul(fabsf(fsub(fmul(hi.x, ho.y), fmul(hi.y, ho.x))), 2.0f);
+  if (!(d0 & d1 & d3 & d4)) return false;
   const float r2 = fmul(c.kmax, fmul(fmul(hi.w, ho.w), fsqrt(fadd(fmul(dx, dx), fmul(dy, dy)))));
   return l2 <= r2;
 }
@@ -618,16 +622,18 @@ __device__ __forceinline__ unsigned warp_incl_scan(unsigned v) {
 
 constexpr uint32_t kHole = 0xffffffffu;  // marks a reserved but unused slot
 
-// Sorted hits that a warp of the two searches takes at once, of n_sorted hits over `warps`
-// warps.  A search warp handles its hits one after the other, so large chunks leave most
-// of the GPU idle on a single event (41k hits in chunks of 32 keep 1281 of 6080 warps
-// busy), and uneven hits leave the last warps of a batch running alone.  The chunk gives
-// every warp 16, at most 8 hits.  Doublet / link search in us with 32, 16, 8, 4 and 2 hits
-// at most: 64 pileup-200 events 1719 / 3576, 1631 / 3358, 1607 / 3315, 1661 / 3382,
-// 1854 / 3655; and for 2, 4, 8, 16 and 32 chunks per warp, 7 gap-pair events (217k hits)
-// 320 / 1498, 277 / 1096, 264 / 883, 269 / 753, 304 / 747.
-__device__ __forceinline__ uint32_t search_chunk(uint32_t n_sorted, uint32_t warps) {
-  return min(8u, max(1u, n_sorted / (16u * warps)));
+// Sorted hits that a warp of the two searches takes next, of `left` not yet taken, with
+// `warps` warps.  A search warp handles its hits one after the other, so large chunks leave
+// most of the GPU idle on a single event (41k hits in chunks of 32 keep 1281 of 6080 warps
+// busy), and uneven hits leave the last warps of a batch running alone; small ones pay the
+// chunk's set-up, which is lane-parallel over its hits, more often.  So a chunk is an eighth
+// of an even share of what is left, 1 to 32 hits.  Doublet / link search in us, with this
+// (and a quarter), with 8 hits at most of a fixed sixteenth, and with 32 always: 64
+// pileup-200 events 1432 / 3082 (1467 / 3529), 1607 / 3315, 1656 / 3367; 7 gap-pair events
+// 260 / 492 (252 / 1071), 269 / 747, 392 / 1878; one pileup-200 event 77 / 82, 75 / 83,
+// 342 / 440.
+__device__ __forceinline__ uint32_t search_chunk(uint32_t left, uint32_t warps) {
+  return min(32u, max(1u, left / (8u * warps)));
 }
 
 // How much a search warp still has to do, as half of the hits after `done` over the hits
