@@ -562,16 +562,16 @@ __device__ __forceinline__ uint32_t find_inner(const Buffers& b, uint32_t lo, ui
 // completed for the ntuplet walk.  The target has links of its own when the list head in
 // its state names a link that starts from it: a cell without links may hold anything
 // there, but no link then names it as its source.  Such a leaf gets its state here, named
-// by whichever of its in-links writes last.  The cleaning keys start here too.  Plain form: the flag of the target's incoming link is set (a leaf needs
+// by whichever of its in-links writes last.  Plain form: the flag of the target's incoming link is set (a leaf needs
 // none: only cells with links can be roots).  Gated form: the link's bf16 feature row for
 // the gate's MLP is computed, one thread per link with every lane busy, from the three
 // hits (mostly still in L2).  A target can be missing only when the doublet stage ran out
 // of cell slots (its status bit is set then); the link then points back to its source, a
 // valid cell, so that the later stages stay within their arrays.
 //
-// Bound by its random sectors.  64 pileup-200 events (5.3M links): 0.32 ms, against 0.27
-// when it left the walk's other fields and the cleaning keys to the stages that now read
-// or reduce them in one sector (A4 to A6 1.00 against 1.62 ms).
+// Bound by its random sectors.  64 pileup-200 events (5.3M links): 0.30 ms, against 0.27
+// when it left the walk's other fields to the search, which now reads a link in one sector
+// (A4 to A6 0.84 against 1.62 ms).
 template <bool GATE>
 __global__ void k_link_targets(Buffers b, pt_cuts cuts, int32_t B, int max_inner,
                                uint64_t cap_links) {
@@ -583,7 +583,6 @@ __global__ void k_link_targets(Buffers b, pt_cuts cuts, int32_t B, int max_inner
     const uint32_t a = hi.x, t = hi.y, h1 = hi.z;
     if (a == kHole) continue;
     const uint32_t next = b.link[l].next;
-    *(uint4*)&b.link_best[l] = make_uint4(~0u, ~0u, ~0u, ~0u);
     uint2 sg = b.seg[(uint64_t)(t & 0x1fffffffu) * max_inner + (t >> 29)];
     if (!PT_CHECK(b.cnt, (uint64_t)sg.x + sg.y <= b.cnt[CNT_CELLS], DBG_TGT_SEGMENT))
       sg = make_uint2(0u, 0u);

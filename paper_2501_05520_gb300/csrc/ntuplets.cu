@@ -16,8 +16,7 @@
 //     one of its cells, and a triplet then dies if it shares a hit with a surviving ntuplet
 //     of >= 4 hits.  The key (6 - nhits, q bits, ntuplet) packed in 64 bits orders ntuplets
 //     that way except where two have the same hit count and q, and it needs no sorted
-//     position, so the search itself reduces it into the cells (atomicMin) as it writes a
-//     path.  An ntuplet that finds another one with its own hit count and q in a cell
+//     position.  One pass reduces the keys into the cells (atomicMin).  An ntuplet that finds another one with its own hit count and q in a cell
 //     compares the tuples and takes the cell if its own is smaller.
 // A6  canonical order: events in order, hit tuples ascending.  Only the survivors are
 //     ordered (0.67M of 4.6M ntuplets on 64 pileup-200 events): they are counted and listed
@@ -29,7 +28,7 @@
 // counting sort on the first hit, then each bucket's few entries by insertion), the sorted
 // position stands in the key for the first hit (so that keys never tie), and the survivors
 // are compacted in that order.  Both give the same ntuplets in the same order.  A4 to A6
-// on 64 pileup-200 events: 1.00 ms, against 1.62 ms when the graph ran the separate steps.
+// on 64 pileup-200 events: 0.84 ms, against 1.62 ms when the graph ran the separate steps.
 #include "ptca_internal.cuh"
 
 namespace ptca {
@@ -73,9 +72,7 @@ __device__ __forceinline__ unsigned long long* best_of(const Buffers& b, uint32_
 }
 
 // Writes ntuplet t (hits g[0..5], batch indices, -1 padded; cells c[0..4], link slots,
-// kHole padded).  CLEAN: reduces its key into its cells; otherwise the cells' keys are
-// reset for the steps that follow.
-template <bool CLEAN>
+// kHole padded) and resets its cells' keys for the cleaning.
 __device__ __forceinline__ void write_ntuplet(const Buffers& b, uint64_t t, uint32_t n, float q,
                                               bool last_is_source, const int32_t (&g)[kMaxHits],
                                               const uint32_t (&c)[kMaxCellsPerNt]) {
@@ -86,13 +83,10 @@ __device__ __forceinline__ void write_ntuplet(const Buffers& b, uint64_t t, uint
   for (int k = 0; k < kMaxCellsPerNt; ++k) b.nt_cells[t * kMaxCellsPerNt + k] = c[k];
   b.nt_n[t] = (uint8_t)n;
   b.nt_q[t] = last_is_source ? -q : q;
-  const unsigned long long key = dedup_key(n, q, (uint32_t)t);
 #pragma unroll
   for (int k = 0; k < kMaxCellsPerNt; ++k) {
     if ((uint32_t)k + 1 >= n) break;
-    unsigned long long* p = best_of(b, c[k], k, n, last_is_source);
-    if (CLEAN) atomicMin(p, key);
-    else *p = ~0ull;
+    *best_of(b, c[k], k, n, last_is_source) = ~0ull;
   }
 }
 
@@ -106,7 +100,7 @@ __device__ __forceinline__ void write_ntuplet(const Buffers& b, uint64_t t, uint
 // indices (perm) are looked up when a path is written (kEmit) or when the warp copies its
 // buffer out (kBuffer).
 constexpr uint32_t kLastIsSource = 1u << 8;  // beside an entry's hit count in the buffer
-template <int MODE, bool GATED, bool CLEAN>
+template <int MODE, bool GATED>
 __device__ uint32_t walk(const Buffers& b, uint32_t l0, unsigned long long t0, uint64_t cap_nt,
                          NtWarp* W) {
   uint32_t path[kMaxCellsPerNt];  // list head of each cell
@@ -157,7 +151,7 @@ __device__ uint32_t walk(const Buffers& b, uint32_t l0, unsigned long long t0, u
                    : last_is_source ? last : b.cell[last].head;
             g[k + 1] = k > depth ? -1 : (int32_t)b.perm[k < depth ? gh[k] : lo.w];
           }
-          write_ntuplet<CLEAN>(b, t, (uint32_t)(depth + 2), q, last_is_source, g, c);
+          write_ntuplet(b, t, (uint32_t)(depth + 2), q, last_is_source, g, c);
         }
       } else {
         const uint32_t e = atomicAdd(&W->cnt, 1u);
@@ -192,12 +186,12 @@ __device__ uint32_t walk(const Buffers& b, uint32_t l0, unsigned long long t0, u
 // then reserves them and the warp copies them out.  If a batch finds more than the buffer
 // holds, it is walked again and written directly.
 //
-// Bound by the latency of its random reads.  64 pileup-200 events (4.6M ntuplets): 0.72 ms
-// with the cleaning keys reduced on the way, against 0.68 + 0.28 ms for the search and a
-// key pass of its own.  Two other places for the keys took longer here: among all cells
-// (2.6 GB, every atomic a DRAM sector) 1.07 ms, and there with the atomics' results taken
-// back (to see equal keys meet) 1.11 ms.
-template <bool GATED, bool CLEAN>
+// Bound by the latency of its random reads.  64 pileup-200 events (4.6M ntuplets): 0.50 ms
+// (0.40 traced), against 0.68 when a step read four arrays.  Reducing the cleaning keys here as well holds
+// up the walks behind the atomics: 0.75 ms with the keys in link space (0.07 for them in a
+// pass of their own), 1.07 with the keys among all cells, 1.11 if their results are waited
+// for.
+template <bool GATED>
 __global__ void __launch_bounds__(kNtWarps * 32, kNtBlocksPerSm)
     k_find_ntuplets(Buffers b, uint64_t cap_links, uint64_t cap_nt) {
   pdl_wait();
@@ -228,7 +222,7 @@ __global__ void __launch_bounds__(kNtWarps * 32, kNtBlocksPerSm)
       const uint32_t r = (uint32_t)lane < take ? W.roots[lane] : kHole;
       if (lane == 0) W.cnt = 0;
       __syncwarp();
-      const uint32_t n = r != kHole ? walk<kBuffer, GATED, CLEAN>(b, r, 0, cap_nt, &W) : 0u;
+      const uint32_t n = r != kHole ? walk<kBuffer, GATED>(b, r, 0, cap_nt, &W) : 0u;
       __syncwarp();
       const uint32_t tot = W.cnt;
       // the roots not taken move to the front of the queue
@@ -262,12 +256,12 @@ __global__ void __launch_bounds__(kNtWarps * 32, kNtBlocksPerSm)
               for (int k = 1; k < kMaxCellsPerNt; ++k)
                 if ((uint32_t)k + 2 == n) c[k] = b.cell[c[k]].head;
             }
-            write_ntuplet<CLEAN>(b, t, n, W.q[e], last_is_source, g, c);
+            write_ntuplet(b, t, n, W.q[e], last_is_source, g, c);
           }
         }
       } else {
         const uint32_t inc = warp_incl_scan(n);
-        if (n) walk<kEmit, GATED, CLEAN>(b, r, base + inc - n, cap_nt, &W);
+        if (n) walk<kEmit, GATED>(b, r, base + inc - n, cap_nt, &W);
       }
     }
   }
@@ -297,6 +291,27 @@ __device__ __noinline__ void take_tied_cell(const Buffers& b, uint32_t t, unsign
     cur = old;
   }
   b.cnt[CNT_NT_TIES] = 1;
+}
+
+// Reduces every ntuplet's key into its cells; `rank` NULL: the key's id is the ntuplet.
+__global__ void k_dedup_min(Buffers b, const uint32_t* rank, uint64_t cap_nt) {
+  pdl_wait();
+  const uint64_t T = min(b.cnt[CNT_NT], (unsigned long long)cap_nt);
+  const uint64_t stride = (uint64_t)gridDim.x * blockDim.x;
+  for (uint64_t t = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x; t < T; t += stride) {
+    const float sq = b.nt_q[t];
+    const bool last_is_source = (__float_as_uint(sq) >> 31) != 0;
+    uint32_t c[kMaxCellsPerNt], n = 1;
+#pragma unroll
+    for (int k = 0; k < kMaxCellsPerNt; ++k) {
+      c[k] = b.nt_cells[t * kMaxCellsPerNt + k];
+      n += c[k] != kHole;
+    }
+    const unsigned long long key = dedup_key(n, fabsf(sq), rank ? rank[t] : (uint32_t)t);
+#pragma unroll
+    for (int k = 0; k < kMaxCellsPerNt; ++k)
+      if (c[k] != kHole) atomicMin(best_of(b, c[k], k, n, last_is_source), key);
+  }
 }
 
 // Ntuplets that no cell ranks behind another hit count or q go to best_list (one
@@ -485,19 +500,6 @@ __global__ void k_bucket_sort(Buffers b, StageSort w) {
   }
 }
 
-__global__ void k_dedup_min(Buffers b, StageSort w) {
-  const uint64_t T = b.cnt[CNT_SCAN_NT];
-  const uint64_t stride = (uint64_t)gridDim.x * blockDim.x;
-  for (uint64_t t = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x; t < T; t += stride) {
-    const uint32_t n = b.nt_n[t];
-    const float sq = b.nt_q[t];
-    const bool last_is_source = (__float_as_uint(sq) >> 31) != 0;
-    const unsigned long long key = dedup_key(n, fabsf(sq), w.rank[t]);
-    for (uint32_t k = 0; k + 1 < n; ++k)
-      atomicMin(best_of(b, b.nt_cells[t * kMaxCellsPerNt + k], k, n, last_is_source), key);
-  }
-}
-
 __global__ void k_dedup_alive(Buffers b, StageSort w) {
   const uint64_t T = b.cnt[CNT_SCAN_NT];
   const uint64_t stride = (uint64_t)gridDim.x * blockDim.x;
@@ -548,24 +550,24 @@ __global__ void k_event_offsets(Buffers b) {
 
 }  // namespace
 
-// The search: in the whole-batch graph (CLEAN) it also reduces the cleaning keys.
-template <bool CLEAN>
 static void launch_search(const Buffers& b, const Params& p, const Launch& l, cudaStream_t s,
                           bool gated) {
   const uint64_t cap_links = (uint64_t)p.max_links, cap_nt = (uint64_t)p.max_ntuplets;
   const int grid = l.sms * kNtBlocksPerSm, block = kNtWarps * 32;
   if (gated)
     PT_TRACE(l, s, "k_find_ntuplets",
-             launch_pdl(k_find_ntuplets<true, CLEAN>, grid, block, 0, s, b, cap_links, cap_nt));
+             launch_pdl(k_find_ntuplets<true>, grid, block, 0, s, b, cap_links, cap_nt));
   else
     PT_TRACE(l, s, "k_find_ntuplets",
-             launch_pdl(k_find_ntuplets<false, CLEAN>, grid, block, 0, s, b, cap_links, cap_nt));
+             launch_pdl(k_find_ntuplets<false>, grid, block, 0, s, b, cap_links, cap_nt));
 }
 
 void launch_ntuplets(const Buffers& b, const Params& p, const Launch& l, cudaStream_t s,
                      bool gated) {
-  launch_search<true>(b, p, l, s, gated);
-  launch_pdl(k_dedup_best, l.grid, 256, 0, s, b, (uint64_t)p.max_ntuplets);
+  const uint64_t cap_nt = (uint64_t)p.max_ntuplets;
+  launch_search(b, p, l, s, gated);
+  launch_pdl(k_dedup_min, l.grid, 256, 0, s, b, nullptr, cap_nt);
+  launch_pdl(k_dedup_best, l.grid, 256, 0, s, b, cap_nt);
   launch_pdl(k_used_hits, l.grid, 256, 0, s, b);
   launch_pdl(k_survivors, l.grid, 256, 0, s, b);
   launch_scan(b.sv_cnt, b.sv_start, &b.cnt[CNT_SCAN_HITS], b.scan_part, s);
@@ -576,12 +578,12 @@ void launch_ntuplet_steps(const Buffers& b, const Params& p, const Launch& l, cu
                           bool gated) {
   const uint64_t cap_nt = (uint64_t)p.max_ntuplets;
   const StageSort w = stage_sort(b, cap_nt);
-  launch_search<false>(b, p, l, s, gated);
+  launch_search(b, p, l, s, gated);
   PT_TRACE(l, s, "k_bucket_count", k_bucket_count<<<l.grid, 256, 0, s>>>(b, w, cap_nt));
   PT_TRACE(l, s, "scan", launch_scan(w.cnt, w.start, &b.cnt[CNT_SCAN_HITS], b.scan_part, s));
   PT_TRACE(l, s, "k_bucket_scatter", k_bucket_scatter<<<l.grid, 256, 0, s>>>(b, w));
   PT_TRACE(l, s, "k_bucket_sort", k_bucket_sort<<<l.grid, 256, 0, s>>>(b, w));
-  PT_TRACE(l, s, "k_dedup_min", k_dedup_min<<<l.grid, 256, 0, s>>>(b, w));
+  PT_TRACE(l, s, "k_dedup_min", k_dedup_min<<<l.grid, 256, 0, s>>>(b, w.rank, cap_nt));
   PT_TRACE(l, s, "k_dedup_alive", k_dedup_alive<<<l.grid, 256, 0, s>>>(b, w));
   PT_TRACE(l, s, "k_dedup_triplets", k_dedup_triplets<<<l.grid, 256, 0, s>>>(b, w));
   PT_TRACE(l, s, "scan", launch_scan(w.alive, w.alive_scan, &b.cnt[CNT_SCAN_NT], b.scan_part, s));

@@ -383,9 +383,9 @@ void launch_fishbone(const Buffers& b, const Params& p, const Launch& l, cudaStr
 // Debug build: records a failure of bounds check `site` as a failing check does.
 cudaError_t launch_debug_inject(const Buffers& b, unsigned site, cudaStream_t s);
 // Ntuplet search, cleaning and order; gated: the search follows the keep mask.  The first
-// form is the whole-batch graph's (the cells' cleaning keys and the lists must be as the
-// link stage and launch_clear leave them; the ntuplets go to the export staging too), the
-// second the stage call's, which may run again on the same links.
+// form is the whole-batch graph's (the survivors' lists must be as launch_clear leaves
+// them; the ntuplets also go out), the second the stage call's, which may run again on the
+// same links.
 void launch_ntuplets(const Buffers& b, const Params& p, const Launch& l, cudaStream_t s,
                      bool gated);
 void launch_ntuplet_steps(const Buffers& b, const Params& p, const Launch& l, cudaStream_t s,
