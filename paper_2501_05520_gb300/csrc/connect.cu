@@ -50,57 +50,53 @@ constexpr int kConnBlocksPerSm = 4;  // 64 registers per thread
 constexpr int kOut = 128;            // staged outgoing cells of one piece
 constexpr int kNb = 128;             // slope buckets of a piece (a multiple of 32)
 static_assert(kNb % 32 == 0, "buckets are scanned kNb / 32 per lane");
+constexpr int kGroup = 8;            // middle hits whose windows are found at once
 constexpr int kQueue = 64;           // window pairs waiting for C1-C3 (power of two)
 static_assert(kOut % 32 == 0, "staged cells are sorted 32 at a time");
 static_assert(kQueue >= 63 && (kQueue & (kQueue - 1)) == 0, "queue holds 31 + 32 entries");
 
-// Azimuthal window of inner hit `hi` (global bin gb, asin_i = asin(kmax*ri/2)) towards
-// outer slot k, the doublet search's window from the inner side: the outer layer's
-// asin(kmax*ro_max/2) - asin_i (+1e-4 rad, +1 bin); up to two ranges [r.x, r.y) and
-// [r.z, r.w) of the sorted hits; empty where the slot is unused, the outer layer ends
-// inside the inner hit's radius, or none of its r-z extent can pass D2 and D3 with the
-// inner hit.
-__device__ __forceinline__ uint4 forward_window(const Buffers& b, const pt_cuts& cuts,
+// Azimuthal window of inner hit `hi` (global bin gb) towards outer slot k, the doublet
+// search's window from the inner side: the outer layer's asin(kmax*ro_max/2) less
+// asin(kmax*ri/2) (+1e-4 rad, +1 bin).  It is the range [x, y) of the sorted hits, or, with
+// kWindowWraps in x, from x to the outer layer's end and from its start to y; y may carry
+// kWindowExact (window_flag).  Empty where the slot is unused, the outer layer ends inside
+// the inner hit's radius, or none of its r-z extent can pass D2 and D3 with the inner hit.
+constexpr uint32_t kWindowWraps = 0x80000000u;
+__device__ __forceinline__ uint2 forward_window(const Buffers& b, const pt_cuts& cuts,
                                                 const PairTable& pt, int32_t B,
-                                                float bins_per_rad, uint32_t gb, float4 hi,
-                                                float asin_i, int k) {
+                                                float bins_per_rad, uint32_t gb, float4 hi, int k) {
   const int el = gb / B;  // event*10 + layer
   const int e = el / kLayers, L = el - e * kLayers;
   const int bin = gb - el * B;
-  uint4 r = make_uint4(0u, 0u, 0u, 0u);
-  if (k >= pt.n_outer[L]) return r;
+  uint2 r = make_uint2(0u, 0u);
   const int Lo = pt.outer[L][k];
   const float ro_max = __uint_as_float(b.layer_rmax[e * kLayers + Lo]);
+  const float ro_min = __uint_as_float(b.layer_rmin[e * kLayers + Lo]);
   if (!(ro_max > hi.w)) return r;
-  if (!rz_box_reachable(cuts, hi.w, hi.z, __uint_as_float(b.layer_rmin[e * kLayers + Lo]), ro_max,
+  if (!rz_box_reachable(cuts, hi.w, hi.z, ro_min, ro_max,
                         float_from_order_key(b.layer_zmin[e * kLayers + Lo]),
                         float_from_order_key(b.layer_zmax[e * kLayers + Lo]), true))
     return r;
   const float asin_o = b.layer_asin[e * kLayers + Lo];
   float win = kHalfPi + 1e-3f;
-  if (asin_o != __int_as_float(0x7f800000)) win = fminf(asin_o - asin_i + 1e-4f, win);
+  if (asin_o != __int_as_float(0x7f800000))
+    win = fminf(asin_o - asinf(0.5f * cuts.kmax * hi.w) + 1e-4f, win);
   const int w = (int)ceilf(win * bins_per_rad) + 1;
   const uint32_t base = (uint32_t)(e * kLayers + Lo) * (uint32_t)B;
+  int lo = bin - w, hb = bin + w + 1;
+  uint32_t wraps = 0u;
   if (2 * w + 1 >= B) {
-    r.x = b.bin_start[base];
-    r.y = b.bin_start[base + B];
-  } else {
-    const int lo = bin - w, hb = bin + w;
-    if (lo < 0) {
-      r.x = b.bin_start[base + B + lo];
-      r.y = b.bin_start[base + B];
-      r.z = b.bin_start[base];
-      r.w = b.bin_start[base + hb + 1];
-    } else if (hb >= B) {
-      r.x = b.bin_start[base + lo];
-      r.y = b.bin_start[base + B];
-      r.z = b.bin_start[base];
-      r.w = b.bin_start[base + hb - B + 1];
-    } else {
-      r.x = b.bin_start[base + lo];
-      r.y = b.bin_start[base + hb + 1];
-    }
+    lo = 0;
+    hb = B;
+  } else if (lo < 0) {
+    lo += B;
+    wraps = kWindowWraps;
+  } else if (hb > B) {
+    hb -= B;
+    wraps = kWindowWraps;
   }
+  r.x = b.bin_start[base + lo] | wraps;
+  r.y = b.bin_start[base + hb] | window_flag(cuts, w, bins_per_rad, hi.w, ro_min, ro_max);
   return r;
 }
 
@@ -115,9 +111,8 @@ struct ConnWarp {
   float4 qp0[kQueue];        // window pairs: the source's inner hit (x, y, z, r)
   uint4 q[kQueue];           //   source cell, target (outer hit | slot << 29), middle hit,
                              //   inner hit on layer 0
-  uint4 rg[kMaxOuter];       // middle hit: its forward windows, one per outer slot
-  uint32_t so[kMaxInner];    //   its incoming segments: first cell
-  uint32_t sc[kMaxInner];    //   and number of cells
+  uint2 rg[kGroup][kMaxOuter];  // forward windows of a group of middle hits, by outer slot
+  uint32_t so[kMaxInner];    // middle hit: its incoming segments: first cell
   uint32_t sb[kMaxInner + 1];  //   incoming cells before each segment (the last: all)
   float tmin, scale, m;      // the staged piece: slope origin and scale of the buckets,
                              //   smallest r2 - r1
@@ -256,34 +251,47 @@ __global__ void __launch_bounds__(kConnWarps * 32, kConnBlocksPerSm)
       }
     }
     unsigned todo = __ballot_sync(kFull, work);
+    uint32_t group = 0xffffffffu;
     while (todo) {
       const int src = __ffs(todo) - 1;
-      todo &= todo - 1;
       const uint32_t h1 = W.s0 + src;
       const uint32_t gb = __shfl_sync(kFull, my_gb, src);
       const int L1 = (gb / (uint32_t)B) % kLayers;
       const float4 p1 = b.hit4[h1];
+      // h1's incoming segments, one slot per lane, and the cells before each
+      const uint2 sgl = lane < pt.n_inner[L1] ? b.seg[(uint64_t)h1 * pt.max_inner + lane]
+                                              : make_uint2(0u, 0u);
+      if (h1 / kGroup != group) {
+        // the windows of the group's hits that are in the chunk and have work, lanes over
+        // hits and outer slots (hit by hit, a few lanes busy, they made the call on 64
+        // pileup-200 events 170 us longer; more hits a group would cost the L1 its size)
+        group = h1 / kGroup;
+        const uint32_t h = group * kGroup + lane % kGroup;
+        const uint32_t j = h - W.s0;
+        const uint32_t hgb = __shfl_sync(kFull, my_gb, j & 31);
+        __syncwarp();
+        if (j < 32u && (todo >> j & 1u)) {
+          const float4 p = b.hit4[h];
+          const int n = pt.n_outer[(hgb / (uint32_t)B) % kLayers];
+          for (int k = lane / kGroup; k < n; k += 32 / kGroup) {
+            uint2 rg = forward_window(b, cuts, pt, B, bins_per_rad, hgb, p, k);
+            const uint32_t rx = rg.x & ~kWindowWraps, ry = rg.y & ~kWindowExact;
+            if (!PT_CHECK(b.cnt, (rx <= ry || (rg.x & kWindowWraps)) && rx <= n_sorted &&
+                                     ry <= n_sorted, DBG_CON_WINDOW))
+              rg = make_uint2(0u, 0u);
+            W.rg[lane % kGroup][k] = rg;
+          }
+        }
+      }
+      todo &= todo - 1;
       __syncwarp();
       {
-        // h1's incoming segments, one slot per lane, and the cells before each
-        const uint2 sgl = lane < pt.n_inner[L1] ? b.seg[(uint64_t)h1 * pt.max_inner + lane]
-                                              : make_uint2(0u, 0u);
         const uint32_t inc = warp_incl_scan(sgl.y);
         if (lane < kMaxInner) {
           W.so[lane] = sgl.x;
-          W.sc[lane] = sgl.y;
           W.sb[lane] = inc - sgl.y;
         }
         if (lane == kMaxInner) W.sb[kMaxInner] = inc;
-      }
-      // forward windows, one outer slot per lane
-      if (lane < kMaxOuter) {
-        uint4 rg = forward_window(b, cuts, pt, B, bins_per_rad, gb, p1,
-                                  asinf(0.5f * cuts.kmax * p1.w), lane);
-        if (!PT_CHECK(b.cnt, rg.x <= rg.y && rg.y <= n_sorted && rg.z <= rg.w && rg.w <= n_sorted,
-                      DBG_CON_WINDOW))
-          rg = make_uint4(0u, 0u, 0u, 0u);
-        W.rg[lane] = rg;
       }
       if (lane == 0) W.ahead = search_ahead(n_sorted, h1 + 1);
       __syncwarp();
@@ -296,11 +304,19 @@ __global__ void __launch_bounds__(kConnWarps * 32, kConnBlocksPerSm)
         const uint32_t lo_ord = (uint32_t)piece * kOut;
         uint32_t cnt = 0;
         float m = __int_as_float(0x7f800000), tlo = m, thi = -m;
+        const float half_k = 0.5f * cuts.kmax * p1.w;
         for (int k = 0; k < pt.n_outer[L1]; ++k) {
           const uint8_t j2 = (uint8_t)pt.slot[pt.outer[L1][k]][L1];
-          for (int part = 0; part < 2; ++part) {
-            const uint4 rk = W.rg[k];
-            const uint32_t beg = part ? rk.z : rk.x, end = part ? rk.w : rk.y;
+          const uint2 rk = W.rg[h1 % kGroup][k];
+          const float tiny = window_tiny(rk.y);
+          uint32_t beg = rk.x & ~kWindowWraps, end = rk.y & ~kWindowExact;
+          uint32_t first = 0;  // the outer layer's bins, where the window wraps
+          bool wraps = rk.x & kWindowWraps;
+          if (wraps) {
+            first = (b.hbin[h1] / (kLayers * B) * kLayers + pt.outer[L1][k]) * B;
+            end = b.bin_start[first + B];
+          }
+          for (;;) {
             // two candidates per lane in flight: both loads are issued before either test
             for (uint32_t o0 = beg; o0 < end; o0 += 64) {
               float4 hv[2];
@@ -313,7 +329,7 @@ __global__ void __launch_bounds__(kConnWarps * 32, kConnBlocksPerSm)
               for (int u = 0; u < 2; ++u) {
                 const uint32_t o = o0 + 32 * u + lane;
                 const float4 ho = hv[u];
-                const bool pass = o < end && doublet_pass(cuts, p1, ho);
+                const bool pass = doublet_quick(cuts, o < end, p1, ho, half_k, ho.w, tiny);
                 const unsigned bal = __ballot_sync(kFull, pass);
                 if (pass) {
                   const uint32_t pos = cnt + __popc(bal & lt_mask);
@@ -330,6 +346,10 @@ __global__ void __launch_bounds__(kConnWarps * 32, kConnBlocksPerSm)
                 cnt += __popc(bal);
               }
             }
+            if (!wraps) break;
+            wraps = false;
+            beg = b.bin_start[first];
+            end = rk.y & ~kWindowExact;
           }
         }
         asm volatile("redux.sync.min.f32 %0, %0, 0xffffffff;" : "+f"(m));

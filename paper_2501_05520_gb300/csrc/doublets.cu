@@ -77,6 +77,8 @@ __device__ __forceinline__ uint4 reverse_window(const Buffers& b, const pt_cuts&
       r.y = b.bin_start[base + hb + 1];
     }
   }
+  r.w |= window_flag(cuts, w, bins_per_rad, ho.w, ri_min,
+                     __uint_as_float(b.layer_rmax[e * kLayers + Li]));
   return r;
 }
 
@@ -118,7 +120,8 @@ __global__ void __launch_bounds__(kWarpsPerBlock * 32, 5)
       st_nin[wib][lane] = (uint8_t)nin;
       for (int k = 0; k < nin; ++k) {
         uint4 rg = reverse_window(b, cuts, pt, B, bins_per_rad, gb, ho, asin_o, k);
-        if (!PT_CHECK(b.cnt, rg.x <= rg.y && rg.y <= n_sorted && rg.z <= rg.w && rg.w <= n_sorted,
+        const uint32_t rw = rg.w & ~kWindowExact;
+        if (!PT_CHECK(b.cnt, rg.x <= rg.y && rg.y <= n_sorted && rg.z <= rw && rw <= n_sorted,
                       DBG_DBL_WINDOW))
           rg = make_uint4(0u, 0u, 0u, 0u);
         st_rng[wib][lane][k] = rg;
@@ -130,12 +133,15 @@ __global__ void __launch_bounds__(kWarpsPerBlock * 32, 5)
       const uint32_t s = s0 + j;
       const float4 ho = st_hit[wib][j];
       const int nin = st_nin[wib][j];
+      const float half_k = 0.5f * cuts.kmax * ho.w;
       // the slots the hit's layer does not use are written empty, so readers need not
       // know the hit's layer
       if (lane >= nin && lane < pt.max_inner)
         b.seg[(uint64_t)s * pt.max_inner + lane] = make_uint2(0u, 0u);
       for (int k = 0; k < nin; ++k) {
-        const uint4 rg = st_rng[wib][j][k];
+        uint4 rg = st_rng[wib][j][k];
+        const float tiny = window_tiny(rg.w);
+        rg.w &= ~kWindowExact;
         uint32_t cnt = 0;
         // pass 1: test, stage up to kStage passing hits, count all; two candidates per
         // lane in flight (both loads issued before either test)
@@ -151,7 +157,8 @@ __global__ void __launch_bounds__(kWarpsPerBlock * 32, 5)
 #pragma unroll
             for (int u = 0; u < 2; ++u) {
               const uint32_t i = i0 + 32 * u + lane;
-              const bool pass = i < end && doublet_pass(cuts, hv[u], ho);
+              const bool pass =
+                  doublet_quick(cuts, i < end, hv[u], ho, half_k, hv[u].w, tiny);
               const unsigned bal = __ballot_sync(kFull, pass);
               if (pass) {
                 const uint32_t pos = cnt + __popc(bal & lt_mask);
