@@ -55,19 +55,19 @@ constexpr int kQueue = 64;           // window pairs waiting for C1-C3 (power of
 static_assert(kOut % 32 == 0, "staged cells are sorted 32 at a time");
 static_assert(kQueue >= 63 && (kQueue & (kQueue - 1)) == 0, "queue holds 31 + 32 entries");
 
-// Azimuthal window of inner hit `hi` (global bin gb) towards outer slot k, the doublet
+// Azimuthal window of inner hit `hi` (global bin gb, azimuth phi) towards outer slot k, the doublet
 // search's window from the inner side: the outer layer's asin(kmax*ro_max/2) less
-// asin(kmax*ri/2) (+1e-4 rad, +1 bin).  It is the range [x, y) of the sorted hits, or, with
+// asin(kmax*ri/2) (+1e-4 rad).  It is the range [x, y) of the sorted hits, or, with
 // kWindowWraps in x, from x to the outer layer's end and from its start to y; y may carry
 // kWindowExact (window_flag).  Empty where the slot is unused, the outer layer ends inside
 // the inner hit's radius, or none of its r-z extent can pass D2 and D3 with the inner hit.
 constexpr uint32_t kWindowWraps = 0x80000000u;
 __device__ __forceinline__ uint2 forward_window(const Buffers& b, const pt_cuts& cuts,
                                                 const PairTable& pt, int32_t B,
-                                                float bins_per_rad, uint32_t gb, float4 hi, int k) {
+                                                float bins_per_rad, uint32_t gb, float4 hi,
+                                                float phi, int k) {
   const int el = gb / B;  // event*10 + layer
   const int e = el / kLayers, L = el - e * kLayers;
-  const int bin = gb - el * B;
   uint2 r = make_uint2(0u, 0u);
   const int Lo = pt.outer[L][k];
   const float ro_max = __uint_as_float(b.layer_rmax[e * kLayers + Lo]);
@@ -81,22 +81,12 @@ __device__ __forceinline__ uint2 forward_window(const Buffers& b, const pt_cuts&
   float win = kHalfPi + 1e-3f;
   if (asin_o != __int_as_float(0x7f800000))
     win = fminf(asin_o - asinf(0.5f * cuts.kmax * hi.w) + 1e-4f, win);
-  const int w = (int)ceilf(win * bins_per_rad) + 1;
   const uint32_t base = (uint32_t)(e * kLayers + Lo) * (uint32_t)B;
-  int lo = bin - w, hb = bin + w + 1;
-  uint32_t wraps = 0u;
-  if (2 * w + 1 >= B) {
-    lo = 0;
-    hb = B;
-  } else if (lo < 0) {
-    lo += B;
-    wraps = kWindowWraps;
-  } else if (hb > B) {
-    hb -= B;
-    wraps = kWindowWraps;
-  }
-  r.x = b.bin_start[base + lo] | wraps;
-  r.y = b.bin_start[base + hb] | window_flag(cuts, w, bins_per_rad, hi.w, ro_min, ro_max);
+  const int2 w = window_bins(phi, win, bins_per_rad, B);
+  const uint32_t wraps = w.x < 0 || w.y > B ? kWindowWraps : 0u;
+  r.x = b.bin_start[base + (w.x < 0 ? w.x + B : w.x)] | wraps;
+  r.y = b.bin_start[base + (w.y > B ? w.y - B : w.y)] |
+        window_flag(cuts, win, bins_per_rad, hi.w, ro_min, ro_max);
   return r;
 }
 
@@ -272,9 +262,10 @@ __global__ void __launch_bounds__(kConnWarps * 32, kConnBlocksPerSm)
         __syncwarp();
         if (j < 32u && (todo >> j & 1u)) {
           const float4 p = b.hit4[h];
+          const float phi = azimuth(p);
           const int n = pt.n_outer[(hgb / (uint32_t)B) % kLayers];
           for (int k = lane / kGroup; k < n; k += 32 / kGroup) {
-            uint2 rg = forward_window(b, cuts, pt, B, bins_per_rad, hgb, p, k);
+            uint2 rg = forward_window(b, cuts, pt, B, bins_per_rad, hgb, p, phi, k);
             const uint32_t rx = rg.x & ~kWindowWraps, ry = rg.y & ~kWindowExact;
             if (!PT_CHECK(b.cnt, (rx <= ry || (rg.x & kWindowWraps)) && rx <= n_sorted &&
                                      ry <= n_sorted, DBG_CON_WINDOW))

@@ -13,7 +13,7 @@
 // asin(kmax*ro/2) - asin(kmax*ri/2) between radii ri < ro (and every radius of this
 // detector lies on the first half of such a circle, which D1 keeps), so with ri bounded
 // below by the smallest radius seen on the inner layer in this event the window is
-// asin(kmax*ro/2) - asin(kmax*ri_min/2), plus a safety margin and one bin each side.
+// asin(kmax*ro/2) - asin(kmax*ri_min/2), plus a safety margin, either side of the hit.
 // It is one contiguous range of the sorted hits, or two when it wraps, taken in
 // increasing index order.  Lanes stride over it, test the exact float32 cuts and stage
 // the passing inner hits in shared memory; the segment is then appended with one
@@ -31,18 +31,17 @@ constexpr float kTwoPi = 6.28318530717958647692f;
 constexpr float kHalfPi = 1.57079632679489661923f;
 constexpr int kWarpsPerBlock = 8;
 
-// Azimuthal window of outer hit `ho` (global bin gb, asin_o = asin(kmax*ro/2), +inf where
-// kmax*ro/2 >= 0.7) towards inner slot k: up to two ranges [r.x, r.y) and [r.z, r.w) of
-// the sorted hits, the first below the second; empty where the slot is unused, the
-// inner layer has no hit inside the outer hit's radius, or none of its r-z extent can
-// pass D2 and D3 with the outer hit.
+// Azimuthal window of outer hit `ho` (global bin gb, azimuth phi, asin_o = asin(kmax*ro/2),
+// +inf where kmax*ro/2 >= 0.7) towards inner slot k: up to two ranges [r.x, r.y) and
+// [r.z, r.w) of the sorted hits, the first below the second, r.w with kWindowExact or
+// without; empty where the slot is unused, the inner layer has no hit inside the outer hit's
+// radius, or none of its r-z extent can pass D2 and D3 with the outer hit.
 __device__ __forceinline__ uint4 reverse_window(const Buffers& b, const pt_cuts& cuts,
                                                 const PairTable& pt, int32_t B,
                                                 float bins_per_rad, uint32_t gb, float4 ho,
-                                                float asin_o, int k) {
+                                                float asin_o, float phi, int k) {
   const int el = gb / B;  // event*10 + layer
   const int e = el / kLayers, L = el - e * kLayers;
-  const int bin = gb - el * B;
   uint4 r = make_uint4(0u, 0u, 0u, 0u);
   if (k >= pt.n_inner[L]) return r;
   const int Li = pt.inner[L][k];
@@ -55,29 +54,23 @@ __device__ __forceinline__ uint4 reverse_window(const Buffers& b, const pt_cuts&
   float win = kHalfPi + 1e-3f;     // where the curvature bound is void, D1's
   if (asin_o != __int_as_float(0x7f800000))
     win = fminf(asin_o - b.layer_asin_lo[e * kLayers + Li] + 1e-4f, win);
-  const int w = (int)ceilf(win * bins_per_rad) + 1;
   const uint32_t base = (uint32_t)(e * kLayers + Li) * (uint32_t)B;
-  if (2 * w + 1 >= B) {
+  const int2 w = window_bins(phi, win, bins_per_rad, B);
+  if (w.x < 0) {
     r.x = b.bin_start[base];
-    r.y = b.bin_start[base + B];
+    r.y = b.bin_start[base + w.y];
+    r.z = b.bin_start[base + B + w.x];
+    r.w = b.bin_start[base + B];
+  } else if (w.y > B) {
+    r.x = b.bin_start[base];
+    r.y = b.bin_start[base + w.y - B];
+    r.z = b.bin_start[base + w.x];
+    r.w = b.bin_start[base + B];
   } else {
-    const int lo = bin - w, hb = bin + w;
-    if (lo < 0) {
-      r.x = b.bin_start[base];
-      r.y = b.bin_start[base + hb + 1];
-      r.z = b.bin_start[base + B + lo];
-      r.w = b.bin_start[base + B];
-    } else if (hb >= B) {
-      r.x = b.bin_start[base];
-      r.y = b.bin_start[base + hb - B + 1];
-      r.z = b.bin_start[base + lo];
-      r.w = b.bin_start[base + B];
-    } else {
-      r.x = b.bin_start[base + lo];
-      r.y = b.bin_start[base + hb + 1];
-    }
+    r.x = b.bin_start[base + w.x];
+    r.y = b.bin_start[base + w.y];
   }
-  r.w |= window_flag(cuts, w, bins_per_rad, ho.w, ri_min,
+  r.w |= window_flag(cuts, win, bins_per_rad, ho.w, ri_min,
                      __uint_as_float(b.layer_rmax[e * kLayers + Li]));
   return r;
 }
@@ -115,11 +108,12 @@ __global__ void __launch_bounds__(kWarpsPerBlock * 32, 5)
       const float4 ho = b.hit4[s];
       const float a = 0.5f * cuts.kmax * ho.w;
       const float asin_o = a >= 0.7f ? __int_as_float(0x7f800000) : asinf(a);
+      const float phi = azimuth(ho);
       st_hit[wib][lane] = ho;
       const int nin = pt.n_inner[(gb / (uint32_t)B) % kLayers];
       st_nin[wib][lane] = (uint8_t)nin;
       for (int k = 0; k < nin; ++k) {
-        uint4 rg = reverse_window(b, cuts, pt, B, bins_per_rad, gb, ho, asin_o, k);
+        uint4 rg = reverse_window(b, cuts, pt, B, bins_per_rad, gb, ho, asin_o, phi, k);
         const uint32_t rw = rg.w & ~kWindowExact;
         if (!PT_CHECK(b.cnt, rg.x <= rg.y && rg.y <= n_sorted && rg.z <= rw && rw <= n_sorted,
                       DBG_DBL_WINDOW))

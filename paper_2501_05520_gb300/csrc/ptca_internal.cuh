@@ -512,12 +512,33 @@ constexpr uint32_t kWindowExact = 0x80000000u;  // a window's flag, in its last 
 __device__ __forceinline__ float window_tiny(uint32_t flagged) {
   return flagged & kWindowExact ? __int_as_float(0x7f800000) : 1e-20f;
 }
-// The flag of a window of +-w bins between a hit of radius r and hits of radii [rlo, rhi].
-__device__ __forceinline__ uint32_t window_flag(const pt_cuts& c, int w, float bins_per_rad,
+// The flag of a window of +-win (and the bins that it cuts) between a hit of radius r and hits
+// of radii [rlo, rhi].
+__device__ __forceinline__ uint32_t window_flag(const pt_cuts& c, float win, float bins_per_rad,
                                                 float r, float rlo, float rhi) {
-  const bool implied = (float)(w + 1) < kHalfPlane * bins_per_rad && fminf(r, rlo) > 1e-9f &&
+  const bool implied = (win - kHalfPlane) * bins_per_rad < -1.0f && fminf(r, rlo) > 1e-9f &&
                        r < 1e9f && rhi < 1e9f && c.kmax >= 0.0f;
   return implied ? 0u : kWindowExact;
+}
+
+// Azimuth of a hit from 0, and the bins [lo, hi) that the range phi -+ win touches: lo < 0 or
+// hi > B where it wraps, 0 and B where it covers them all.  win has room (1e-4 rad) for the
+// rounding of the azimuths and of their bins.  Around the hit's bin instead of its azimuth the
+// range had to have two bins more at either end, half of them beyond need: a hit of a pileup-200
+// event has 151 doublet and 170 link candidates with 256 bins (237 and 244 then), 138 and 158
+// with 512 (181 and 197), 128 and 150 with 2048 (139 and 160).
+__device__ __forceinline__ float azimuth(float4 h) {  // from 0
+  return atan2f(h.y, h.x) + 3.14159265358979323846f;
+}
+__device__ __forceinline__ int2 window_bins(float phi, float win, float bins_per_rad, int32_t B) {
+  win = fmaxf(win, 0.0f);
+  int lo = min((int)floorf((phi - win) * bins_per_rad), B - 1);
+  int hi = (int)floorf((phi + win) * bins_per_rad) + 1;
+  if (hi - lo >= B) {
+    lo = 0;
+    hi = B;
+  }
+  return make_int2(lo, hi);
 }
 __device__ __forceinline__ bool doublet_quick(const pt_cuts& c, bool in, float4 hi, float4 ho,
                                               float half_k, float r, float tiny) {
