@@ -39,18 +39,21 @@ enum : int {
   CNT_SCORE_STATUS = 9,  // status bits of the standalone gate scoring (pt_gate_score)
   CNT_CELLS_USED = 10,  // cells written (CNT_CELLS counts reserved slots incl. holes)
   CNT_LINKS_USED = 11,  // links written (CNT_LINKS counts reserved slots incl. holes)
-  CNT_DBL_WORK = 12,    // doublet search: next chunk of sorted hits
   CNT_VTX = 14,         // vertices of the batch
   CNT_RAW_STATUS = 15,  // raw input: status bits (RAW_*), not reset by the chain
   CNT_RAW_DIGIS = 16,   // raw input: digis of the batch (size of the run-flag scan)
   CNT_RAW_RUNS = 17,    // raw input: module runs (size of the hit-count scan)
   CNT_RAW_HITS = 18,    // raw input: hits made from the digis
   CNT_RAW_BIG = 19,     // raw input: long module runs listed for the block-per-run launch
-  CNT_LNK_WORK = 20,    // link search: next chunk of sorted middle hits
   CNT_NT_BEST = 21,     // ntuplets on best_list
   CNT_DEBUG_SITE = 22,  // debug build: the first failing bounds check (DebugSite)
   CNT_NT_TIES = 23,     // nonzero: ntuplets of the same hit count and q met in a cell
-  CNT_N = 24
+  // The searches' work counters, each in a 128-byte line of its own: a warp adds to one for
+  // nearly every hit of a single event, and to CNT_CELLS or CNT_LINKS meanwhile (one gated
+  // pileup-200 event 345 us with all of them in one line, 330 so).
+  CNT_DBL_WORK = 32,    // doublet search: next chunk of sorted hits
+  CNT_LNK_WORK = 48,    // link search: next chunk of sorted middle hits
+  CNT_N = 64
 };
 // raw-input status bits (cnt[CNT_RAW_STATUS])
 enum : unsigned long long {
