@@ -23,7 +23,7 @@
 // slope is a monotone function of it, evaluated the same way for the staged slopes and
 // for the window's ends, which are moved out by a further 0.1 % + 1e-5 so that rounding
 // of t_a -+ w cannot exclude a bucket); the staged cells there that fall inside the
-// window are queued as (source cell, target) pairs.  A queued pair carries all it needs,
+// window are queued as (source cell, target) pairs.  A queued pair names its three hits,
 // so the queue runs on across incoming groups and middle hits, and C1, C2 and C3 are
 // tested only once 32 pairs are waiting, all lanes busy (about six pairs fall in the
 // windows of a group of 32 incoming cells).  A link takes the next slot of the warp's
@@ -90,6 +90,8 @@ __device__ __forceinline__ uint2 forward_window(const Buffers& b, const pt_cuts&
   return r;
 }
 
+constexpr uint32_t kOnLayer0 = 0x80000000u;
+
 // Per-warp shared state.
 struct ConnWarp {
   float t[kOut];             // staged outgoing cells: r-z slope
@@ -98,9 +100,8 @@ struct ConnWarp {
   float ts[kOut];            // slopes in bucket order
   uint32_t cs[kOut];         //   and codes
   uint32_t bstart[kNb + 1];  // first bucket-ordered position of each slope bucket
-  float4 qp0[kQueue];        // window pairs: the source's inner hit (x, y, z, r)
-  uint4 q[kQueue];           //   source cell, target (outer hit | slot << 29), middle hit,
-                             //   inner hit on layer 0
+  uint4 q[kQueue];           // window pairs: source cell, target (outer hit | slot << 29),
+                             //   middle hit, inner hit (with kOnLayer0 or without)
   uint2 rg[kGroup][kMaxOuter];  // forward windows of a group of middle hits, by outer slot
   uint32_t so[kMaxInner];    // middle hit: its incoming segments: first cell
   uint32_t sb[kMaxInner + 1];  //   incoming cells before each segment (the last: all)
@@ -168,29 +169,24 @@ __global__ void __launch_bounds__(kConnWarps * 32, kConnBlocksPerSm)
     hi = min(hi, (unsigned long long)cap_links);
     for (unsigned long long i = lo + lane; i < hi; i += 32) b.link[i].src = kHole;
   };
-  // C1, C2 and C3 on nt queued pairs, one per lane, all of them carrying what they need
-  // (the source cell and the target's outer hit and slot), so that pairs of different
-  // incoming groups and middle hits share one pass; a link is appended to its source's
-  // out-link list.
+  // C1, C2 and C3 on nt queued pairs, one per lane, each with its hits, its source cell and
+  // its target's slot, so that pairs of different incoming groups and middle hits share one
+  // pass; a link is appended to its source's out-link list.
   uint32_t qhead = 0, qtail = 0;  // warp-uniform queue positions
   auto process = [&](uint32_t nt) {
     __syncwarp();
     const bool v = (uint32_t)lane < nt;
     const uint32_t qi = (qhead + lane) & (kQueue - 1);
     uint4 e = make_uint4(0u, 0u, 0u, 0u);
-    float4 q0 = make_float4(0.f, 0.f, 0.f, 0.f);
-    if (v) {
-      e = W.q[qi];
-      q0 = W.qp0[qi];
-    }
+    if (v) e = W.q[qi];
     qhead += nt;
     __syncwarp();
     bool ok = false;
     float q = 0.0f;
     const uint32_t src = e.x;
     if (v) {
-      const float4 q1 = b.hit4[e.z], q2 = b.hit4[e.y & 0x1fffffffu];
-      ok = link_c1(cuts, q0, q1, q2) && link_c23(cuts, q0, e.w != 0, q1, q2, q);
+      const float4 q0 = b.hit4[e.w & ~kOnLayer0], q1 = b.hit4[e.z], q2 = b.hit4[e.y & 0x1fffffffu];
+      ok = link_c1(cuts, q0, q1, q2) && link_c23(cuts, q0, e.w >> 31, q1, q2, q);
     }
     const unsigned pm = __ballot_sync(kFull, ok);
     const uint32_t n = __popc(pm);
@@ -279,7 +275,7 @@ __global__ void __launch_bounds__(kConnWarps * 32, kConnBlocksPerSm)
       {
         const uint32_t inc = warp_incl_scan(sgl.y);
         if (lane < kMaxInner) {
-          W.so[lane] = sgl.x;
+          W.so[lane] = sgl.x - (inc - sgl.y);
           W.sb[lane] = inc - sgl.y;
         }
         if (lane == kMaxInner) W.sb[kMaxInner] = inc;
@@ -288,6 +284,8 @@ __global__ void __launch_bounds__(kConnWarps * 32, kConnBlocksPerSm)
       __syncwarp();
       const uint32_t nin = W.sb[kMaxInner];
 
+      uint32_t h0a = 0, h0b = 0;
+      float4 p0n = make_float4(0.f, 0.f, 0.f, 0.f);
       // Stages piece `piece` (the passing outgoing cells of ordinal [piece*kOut,
       // (piece+1)*kOut) in search order) and orders it by slope; returns the number of
       // outgoing cells of h1.
@@ -343,6 +341,7 @@ __global__ void __launch_bounds__(kConnWarps * 32, kConnBlocksPerSm)
             end = rk.y & ~kWindowExact;
           }
         }
+        if ((uint32_t)lane < nin) p0n = b.hit4[h0a];
         asm volatile("redux.sync.min.f32 %0, %0, 0xffffffff;" : "+f"(m));
         asm volatile("redux.sync.min.f32 %0, %0, 0xffffffff;" : "+f"(tlo));
         asm volatile("redux.sync.max.f32 %0, %0, 0xffffffff;" : "+f"(thi));
@@ -404,7 +403,13 @@ __global__ void __launch_bounds__(kConnWarps * 32, kConnBlocksPerSm)
       auto incoming = [&](uint32_t i, int& kin) -> uint32_t {
         kin = 0;
         while (i >= W.sb[kin + 1]) ++kin;  // i < W.sb[max_inner] bounds the walk
-        return W.so[kin] + (i - W.sb[kin]);
+        return W.so[kin] + i;
+      };
+      auto inner_hit = [&](uint32_t i) -> uint32_t {
+        int kin;
+        if (i >= nin) return 0u;
+        const uint32_t c = incoming(i, kin);
+        return PT_CHECK(b.cnt, c < b.cnt[CNT_CELLS], DBG_CON_INCOMING) ? b.cell_in[c] : 0u;
       };
       // Every piece of the outgoing cells is staged once and visited by all incoming groups.
       // With more than one piece a cell's pairs come up again after some were tested, so
@@ -412,15 +417,14 @@ __global__ void __launch_bounds__(kConnWarps * 32, kConnBlocksPerSm)
       uint32_t nout = 0;
 #pragma unroll 1
       for (int piece = 0; piece == 0 || (uint32_t)piece * kOut < nout; ++piece) {
-        // the first incoming group's inner hits are fetched while the outgoing cells are
-        // searched, each later group's while the group before it is processed
-        float4 p0_next = make_float4(0.f, 0.f, 0.f, 0.f);
-        if ((uint32_t)lane < nin) {
-          int kin;
-          const uint32_t c0 = incoming(lane, kin);
-          if (PT_CHECK(b.cnt, c0 < b.cnt[CNT_CELLS], DBG_CON_INCOMING))
-            p0_next = b.hit4[b.cell_in[c0]];
-        }
+        // Inner hits of the lane's cells: the first two groups' indices are fetched while the
+        // outgoing cells are searched, the first group's coordinates while they are sorted;
+        // each group then fetches the next one's coordinates and the indices of the one
+        // after that, and a queued pair names its inner hit instead of carrying it.  With
+        // the first group's two dependent loads ahead of the search, and the pairs' inner
+        // hits in shared memory, 64 pileup-200 events took 5700 instead of 5490 us.
+        h0a = inner_hit(lane);
+        h0b = inner_hit(lane + 32);
         nout = stage_piece(piece);
         if (nout == 0) break;
         if (piece == 0 && nout > (uint32_t)kOut) {
@@ -442,15 +446,11 @@ __global__ void __launch_bounds__(kConnWarps * 32, kConnBlocksPerSm)
             c = incoming(i, kin);
             valid = PT_CHECK(b.cnt, c < b.cnt[CNT_CELLS], DBG_CON_INCOMING);
           }
-          const float4 p0 = p0_next;
-          const bool first_b0 = valid && pt.inner[L1][kin] == 0;
-          uint32_t h0_next = 0;
-          const bool valid_next = i + 32 < nin;
-          if (valid_next) {
-            int kn;
-            const uint32_t cn = incoming(i + 32, kn);
-            if (PT_CHECK(b.cnt, cn < b.cnt[CNT_CELLS], DBG_CON_INCOMING)) h0_next = b.cell_in[cn];
-          }
+          const float4 p0 = p0n;
+          const uint32_t h0 = h0a | (valid && pt.inner[L1][kin] == 0 ? kOnLayer0 : 0u);
+          h0a = h0b;
+          if (i + 32 < nin) p0n = b.hit4[h0a];
+          h0b = inner_hit(i + 64);
           const float ta = __fdividef(p1.z - p0.z, p1.w - p0.w);  // the cell's slope dz/dr
           const float id1 = __fdividef(1.0f, p1.w - p0.w);
           const float wa = (cuts.rz0 + cuts.rz1 * cuts.cotmax) * id1;
@@ -495,13 +495,11 @@ __global__ void __launch_bounds__(kConnWarps * 32, kConnBlocksPerSm)
             (void)PT_CHECK(b.cnt, qtail + __popc(bal) - qhead <= (uint32_t)kQueue, DBG_CON_QUEUE);
             if (pass) {
               const uint32_t qi = (qtail + __popc(bal & lt_mask)) & (kQueue - 1);
-              W.q[qi] = make_uint4(c, code, h1, first_b0 ? 1u : 0u);
-              W.qp0[qi] = p0;
+              W.q[qi] = make_uint4(c, code, h1, h0);
             }
             qtail += __popc(bal);
             if (qtail - qhead >= 32u) process(32u);
           }
-          if (valid_next) p0_next = b.hit4[h0_next];
         }
       }
     }
