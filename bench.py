@@ -106,18 +106,18 @@ CALL_STAGES = {"load": ("A1",), "doublets": ("A2",), "connect": ("A3",),
 def kernel_layout_bytes(kernel: str, c: dict) -> int | None:
     N, C, Lk, T = c["hits"], c["cells"], c["links"], c["candidates"]
     return {
-        # hit (x,y,z,r) and bin 20 N; incoming segments 24 N; cells (inner, outer) 8 C and
-        # their two link flags 2 C
-        "k_doublets": 20 * N + 24 * N + 10 * C,
+        # hit (x,y,z,r) and bin 20 N; incoming segments 24 N; cells (inner hit) 4 C
+        "k_doublets": 20 * N + 24 * N + 4 * C,
         # hit and bin 20 N, incoming segments 24 N; inner hit of each incoming cell 4 C;
-        # links (source, target, quality, next) 16 Lk, list heads and out flags <= 5 Lk
-        "k_connect": 44 * N + 4 * C + 21 * Lk,
-        # link source and target 8 Lk (read), the source's outer hit and the target's
-        # segment 12 Lk, target (write) and in flag 5 Lk
-        "k_link_targets": 25 * Lk,
-        # link sources (root search) 4 Lk, roots' flags and lists <= 10 Lk, link targets
-        # and qualities 8 Lk; candidates (6 hits, 5 cells, n, q) 49 T
-        "k_find_ntuplets": 22 * Lk + 49 * T,
+        # links (source, target code, middle hit, quality, next) 20 Lk, their sources' states
+        # <= 8 Lk
+        "k_connect": 44 * N + 4 * C + 28 * Lk,
+        # the search's part of a link 20 Lk, the target's segment 8 Lk, state 8 Lk and its
+        # list's first link 4 Lk; the rest of the record 16 Lk
+        "k_link_targets": 56 * Lk,
+        # link records 32 Lk, their sources' states 8 Lk; candidates (6 hits, 5 cells, n, q)
+        # 49 T and their hits' input indices 24 T
+        "k_find_ntuplets": 40 * Lk + 73 * T,
     }.get(kernel)
 
 
@@ -774,8 +774,9 @@ def run_ours(args):
             trace = ctx.pt_get_trace()
             ctx.pt_set_tracing(False)
             kernels[form] = {k: round(ms / n, 4) for k, (ms, n) in trace.items()}
+            # a scan is two launches, the binning's one
             launches[form] = sum(n * (2 if k == "scan" else 1)
-                                 for k, (_, n) in trace.items()) // TRACE_STEPS
+                                 for k, (_, n) in trace.items()) // TRACE_STEPS - 1
         total_s = max_over_ranks(sum(step_ms) / 1000.0, dist, dev)
         # end to end through the public call: pinned host in, host out; E2E_THREADS host
         # threads, each with its own context and stream, so one batch's copies overlap the

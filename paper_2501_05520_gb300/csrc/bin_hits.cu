@@ -19,6 +19,7 @@ __global__ void k_clear(Buffers b, int32_t phi_bins) {
   const int stride = gridDim.x * blockDim.x;
   const int t0 = blockIdx.x * blockDim.x + threadIdx.x;
   for (int i = t0; i <= nb; i += stride) b.bin_cnt[i] = 0;
+  for (int i = t0; i < kScanBlocks; i += stride) b.scan_part[i] = 0;
   for (int i = t0; i < E * kLayers; i += stride) {
     b.layer_rmax[i] = 0u;
     b.layer_rmin[i] = 0x7f800000u;  // +inf
@@ -71,12 +72,17 @@ struct LayerRange {
 // ranges are gathered in shared memory and go to the global arrays once per event and block
 // (a warp's hits lie on some ten layers, and four global atomics for each of them were most
 // of the kernel: 64 pileup-200 events 93 us, now 38), and the event of a tile is
-// looked up once where all its hits share it.
+// looked up once where all its hits share it.  The sums that the scan of the counts starts
+// from, one per share of the bins, come from here as well, counted in shared memory, which
+// saves the scan its first pass and launch.
 constexpr int kCountThreads = 256;
 __global__ void __launch_bounds__(kCountThreads) k_bin_count(Buffers b, int32_t B) {
   pdl_sync();
   __shared__ LayerRange s_range[kLayers];
+  __shared__ uint32_t s_share[kScanBlocks];
   const int E = b.hdr->n_events, N = b.hdr->n_hits;
+  const uint32_t share = (uint32_t)scan_share((uint64_t)E * kLayers * B);
+  for (int i = threadIdx.x; i < kScanBlocks; i += kCountThreads) s_share[i] = 0;
   const float scale = (float)B / (2.0f * kPi);
   const bool copy = b.hdr->x != nullptr;
   const float* X = copy ? b.hdr->x : b.in_x;
@@ -138,6 +144,7 @@ __global__ void __launch_bounds__(kCountThreads) k_bin_count(Buffers b, int32_t 
     const uint32_t gb = key * (uint32_t)B + (uint32_t)bin;
     b.in_bin[g] = gb;
     b.in_rank[g] = atomicAdd(&b.bin_cnt[gb], 1u);
+    atomicAdd(&s_share[gb / share], 1u);
     // r >= 0, so the integer order of the bit patterns is the float order
     if (e == e_now) {
       // most hits lie inside the range gathered so far
@@ -155,6 +162,8 @@ __global__ void __launch_bounds__(kCountThreads) k_bin_count(Buffers b, int32_t 
     }
   }
   flush(e_now);
+  for (int i = threadIdx.x; i < kScanBlocks; i += kCountThreads)
+    if (s_share[i]) atomicAdd(&b.scan_part[i], s_share[i]);
 }
 
 __global__ void k_bin_scatter(Buffers b, float kmax) {
@@ -202,10 +211,8 @@ __device__ __forceinline__ uint32_t block_excl_scan(uint32_t v, uint32_t* warp_s
   return r;
 }
 
-// A block's share of n entries, a multiple of four so that aligned arrays are read four at a
-// time.
 __device__ __forceinline__ void chunk_of(uint64_t n, uint64_t* lo, uint64_t* hi) {
-  const uint64_t per = ((n + gridDim.x - 1) / gridDim.x + 3) & ~3ull;
+  const uint64_t per = scan_share(n);
   *lo = min(n, per * blockIdx.x);
   *hi = min(n, *lo + per);
 }
@@ -277,6 +284,11 @@ __global__ void __launch_bounds__(kScanThreads) k_scan_final(const uint32_t* in,
 void launch_scan(const uint32_t* in, uint32_t* out, const unsigned long long* n_dev,
                  uint32_t* part, cudaStream_t s) {
   launch_pdl(k_scan_partial, kScanBlocks, kScanThreads, 0, s, in, part, n_dev);
+  launch_scan_counted(in, out, n_dev, part, s);
+}
+
+void launch_scan_counted(const uint32_t* in, uint32_t* out, const unsigned long long* n_dev,
+                         const uint32_t* part, cudaStream_t s) {
   launch_pdl(k_scan_final, kScanBlocks, kScanThreads, 0, s, in, out, part, n_dev);
 }
 
@@ -286,7 +298,8 @@ void launch_clear(const Buffers& b, const Params& p, const Launch& l, cudaStream
 
 void launch_bin_hits(const Buffers& b, const Params& p, const Launch& l, cudaStream_t s) {
   PT_TRACE(l, s, "k_bin_count", launch_pdl(k_bin_count, l.grid, kCountThreads, 0, s, b, p.phi_bins));
-  PT_TRACE(l, s, "scan", launch_scan(b.bin_cnt, b.bin_start, &b.cnt[CNT_SCAN_BINS], b.scan_part, s));
+  PT_TRACE(l, s, "scan", launch_scan_counted(b.bin_cnt, b.bin_start, &b.cnt[CNT_SCAN_BINS],
+                                           b.scan_part, s));
   PT_TRACE(l, s, "k_bin_scatter", launch_pdl(k_bin_scatter, l.grid, 256, 0, s, b, p.cuts.kmax));
 }
 

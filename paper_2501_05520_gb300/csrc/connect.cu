@@ -250,7 +250,7 @@ __global__ void __launch_bounds__(kConnWarps * 32, kConnBlocksPerSm)
       if (h1 / kGroup != group) {
         // the windows of the group's hits that are in the chunk and have work, lanes over
         // hits and outer slots (hit by hit, a few lanes busy, they made the call on 64
-        // pileup-200 events 170 us longer; more hits a group would cost the L1 its size)
+        // pileup-200 events 170 us longer; groups of 16 or 32 gain nothing more)
         group = h1 / kGroup;
         const uint32_t h = group * kGroup + lane % kGroup;
         const uint32_t j = h - W.s0;
@@ -578,9 +578,9 @@ __device__ __forceinline__ uint32_t find_inner(const Buffers& b, uint32_t lo, ui
 // of cell slots (its status bit is set then); the link then points back to its source, a
 // valid cell, so that the later stages stay within their arrays.
 //
-// Bound by its random sectors.  64 pileup-200 events (5.3M links): 0.30 ms, against 0.27
+// Bound by its random sectors.  64 pileup-200 events (5.3M links): 0.34 ms, against 0.27
 // when it left the walk's other fields to the search, which now reads a link in one sector
-// (A4 to A6 0.84 against 1.62 ms).
+// (A4 to A6 0.73 against 1.62 ms).
 template <bool GATE>
 __global__ void k_link_targets(Buffers b, pt_cuts cuts, int32_t B, int max_inner,
                                uint64_t cap_links) {

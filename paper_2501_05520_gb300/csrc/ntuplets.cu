@@ -28,7 +28,7 @@
 // counting sort on the first hit, then each bucket's few entries by insertion), the sorted
 // position stands in the key for the first hit (so that keys never tie), and the survivors
 // are compacted in that order.  Both give the same ntuplets in the same order.  A4 to A6
-// on 64 pileup-200 events: 0.84 ms, against 1.62 ms when the graph ran the separate steps.
+// on 64 pileup-200 events: 0.73 ms, against 1.62 ms when the graph ran the separate steps.
 #include "ptca_internal.cuh"
 
 namespace ptca {
@@ -186,8 +186,8 @@ __device__ uint32_t walk(const Buffers& b, uint32_t l0, unsigned long long t0, u
 // then reserves them and the warp copies them out.  If a batch finds more than the buffer
 // holds, it is walked again and written directly.
 //
-// Bound by the latency of its random reads.  64 pileup-200 events (4.6M ntuplets): 0.50 ms
-// (0.40 traced), against 0.68 when a step read four arrays.  Reducing the cleaning keys here as well holds
+// Bound by the latency of its random reads.  64 pileup-200 events (4.6M ntuplets): 0.40 ms,
+// against 0.68 when a step read four arrays.  Reducing the cleaning keys here as well holds
 // up the walks behind the atomics: 0.75 ms with the keys in link space (0.07 for them in a
 // pass of their own), 1.07 with the keys among all cells, 1.11 if their results are waited
 // for.

@@ -406,6 +406,9 @@ cudaError_t launch_vertices(const Buffers& b, const Params& p, int n_events, int
 // scan of n+1 entries: out[i] = sum(in[0..i)), n = *n_dev
 void launch_scan(const uint32_t* in, uint32_t* out, const unsigned long long* n_dev,
                  uint32_t* part, cudaStream_t s);
+// the same where part[] holds the sums of the blocks' shares (scan_share) already
+void launch_scan_counted(const uint32_t* in, uint32_t* out, const unsigned long long* n_dev,
+                         const uint32_t* part, cudaStream_t s);
 // learned gate: features, tensor-core MLP and link pruning (enabled contexts only);
 // gate_prepare() sets the MLP kernel's shared-memory attribute (call before capture)
 cudaError_t gate_prepare();
@@ -435,6 +438,12 @@ void launch_export_links(const Buffers& b, const Params& p, const Launch& l, int
 // ------------------------------------------------------------ device helpers
 #ifdef __CUDACC__
 constexpr unsigned kFull = 0xffffffffu;
+
+// Entries of one scan block's share of n, a multiple of four so that aligned arrays are read
+// four at a time.
+__device__ __forceinline__ uint64_t scan_share(uint64_t n) {
+  return ((n + kScanBlocks - 1) / kScanBlocks + 3) & ~3ull;
+}
 
 // Correctly rounded float32 operations that the compiler never contracts into FMA.
 __device__ __forceinline__ float fmul(float a, float b) { return __fmul_rn(a, b); }
@@ -692,11 +701,10 @@ constexpr uint32_t kHole = 0xffffffffu;  // marks a reserved but unused slot
 // most of the GPU idle on a single event (41k hits in chunks of 32 keep 1281 of 6080 warps
 // busy), and uneven hits leave the last warps of a batch running alone; small ones pay the
 // chunk's set-up, which is lane-parallel over its hits, more often.  So a chunk is an eighth
-// of an even share of what is left, 1 to 32 hits.  Doublet / link search in us, with this
-// (and a quarter), with 8 hits at most of a fixed sixteenth, and with 32 always: 64
-// pileup-200 events 1432 / 3082 (1467 / 3529), 1607 / 3315, 1656 / 3367; 7 gap-pair events
-// 260 / 492 (252 / 1071), 269 / 747, 392 / 1878; one pileup-200 event 77 / 82, 75 / 83,
-// 342 / 440.
+// of an even share of what is left, 1 to 32 hits.  The whole call in us, with an eighth (a
+// quarter, a sixth, a twelfth; an eighth of at most 16 hits): 64 pileup-200 events 5499 (5645,
+// 5545, 5614; 5514), 7 gap-pair events 1125 (1199, 1104, 1171; 1129), one pileup-200 event 327
+// (328, 333, 333; 333).  With 32 hits always the two searches of that one event alone took 782.
 __device__ __forceinline__ uint32_t search_chunk(uint32_t left, uint32_t warps) {
   return min(32u, max(1u, left / (8u * warps)));
 }
