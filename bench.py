@@ -774,8 +774,8 @@ def run_ours(args):
             trace = ctx.pt_get_trace()
             ctx.pt_set_tracing(False)
             kernels[form] = {k: round(ms / n, 4) for k, (ms, n) in trace.items()}
-            # a scan is two launches, the binning's one
-            launches[form] = sum(n * (2 if k == "scan" else 1)
+            # a scan is two launches, the binning's one, and the doublet step two
+            launches[form] = sum(n * (2 if k in ("scan", "k_doublets") else 1)
                                  for k, (_, n) in trace.items()) // TRACE_STEPS - 1
         total_s = max_over_ranks(sum(step_ms) / 1000.0, dist, dev)
         # end to end through the public call: pinned host in, host out; E2E_THREADS host

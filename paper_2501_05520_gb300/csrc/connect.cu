@@ -61,7 +61,6 @@ static_assert(kQueue >= 63 && (kQueue & (kQueue - 1)) == 0, "queue holds 31 + 32
 // kWindowWraps in x, from x to the outer layer's end and from its start to y; y may carry
 // kWindowExact (window_flag).  Empty where the slot is unused, the outer layer ends inside
 // the inner hit's radius, or none of its r-z extent can pass D2 and D3 with the inner hit.
-constexpr uint32_t kWindowWraps = 0x80000000u;
 __device__ __forceinline__ uint2 forward_window(const Buffers& b, const pt_cuts& cuts,
                                                 const PairTable& pt, int32_t B,
                                                 float bins_per_rad, uint32_t gb, float4 hi,

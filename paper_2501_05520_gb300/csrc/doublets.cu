@@ -32,22 +32,22 @@ constexpr float kHalfPi = 1.57079632679489661923f;
 constexpr int kWarpsPerBlock = 8;
 
 // Azimuthal window of outer hit `ho` (global bin gb, azimuth phi, asin_o = asin(kmax*ro/2),
-// +inf where kmax*ro/2 >= 0.7) towards inner slot k: up to two ranges [r.x, r.y) and
-// [r.z, r.w) of the sorted hits, the first below the second, r.w with kWindowExact or
-// without; empty where the slot is unused, the inner layer has no hit inside the outer hit's
-// radius, or none of its r-z extent can pass D2 and D3 with the outer hit.
-__device__ __forceinline__ uint4 reverse_window(const Buffers& b, const pt_cuts& cuts,
+// +inf where kmax*ro/2 >= 0.7) towards inner slot k of its layer: the range [x, y) of the
+// sorted hits, or, with kWindowWraps in x, from x to the inner layer's end and from its start
+// to y; y may carry kWindowExact (window_flag).  Empty where the inner layer has no hit inside
+// the outer hit's radius, or none of its r-z extent can pass D2 and D3 with the outer hit.
+__device__ __forceinline__ uint2 reverse_window(const Buffers& b, const pt_cuts& cuts,
                                                 const PairTable& pt, int32_t B,
                                                 float bins_per_rad, uint32_t gb, float4 ho,
                                                 float asin_o, float phi, int k) {
   const int el = gb / B;  // event*10 + layer
   const int e = el / kLayers, L = el - e * kLayers;
-  uint4 r = make_uint4(0u, 0u, 0u, 0u);
-  if (k >= pt.n_inner[L]) return r;
+  uint2 r = make_uint2(0u, 0u);
   const int Li = pt.inner[L][k];
   const float ri_min = __uint_as_float(b.layer_rmin[e * kLayers + Li]);
+  const float ri_max = __uint_as_float(b.layer_rmax[e * kLayers + Li]);
   if (!(ho.w > ri_min)) return r;  // D0 fails for every hit of the inner layer
-  if (!rz_box_reachable(cuts, ho.w, ho.z, ri_min, __uint_as_float(b.layer_rmax[e * kLayers + Li]),
+  if (!rz_box_reachable(cuts, ho.w, ho.z, ri_min, ri_max,
                         float_from_order_key(b.layer_zmin[e * kLayers + Li]),
                         float_from_order_key(b.layer_zmax[e * kLayers + Li]), false))
     return r;
@@ -56,33 +56,65 @@ __device__ __forceinline__ uint4 reverse_window(const Buffers& b, const pt_cuts&
     win = fminf(asin_o - b.layer_asin_lo[e * kLayers + Li] + 1e-4f, win);
   const uint32_t base = (uint32_t)(e * kLayers + Li) * (uint32_t)B;
   const int2 w = window_bins(phi, win, bins_per_rad, B);
-  if (w.x < 0) {
-    r.x = b.bin_start[base];
-    r.y = b.bin_start[base + w.y];
-    r.z = b.bin_start[base + B + w.x];
-    r.w = b.bin_start[base + B];
-  } else if (w.y > B) {
-    r.x = b.bin_start[base];
-    r.y = b.bin_start[base + w.y - B];
-    r.z = b.bin_start[base + w.x];
-    r.w = b.bin_start[base + B];
-  } else {
-    r.x = b.bin_start[base + w.x];
-    r.y = b.bin_start[base + w.y];
-  }
-  r.w |= window_flag(cuts, win, bins_per_rad, ho.w, ri_min,
-                     __uint_as_float(b.layer_rmax[e * kLayers + Li]));
+  const uint32_t wraps = w.x < 0 || w.y > B ? kWindowWraps : 0u;
+  r.x = b.bin_start[base + (w.x < 0 ? w.x + B : w.x)] | wraps;
+  r.y = b.bin_start[base + (w.y > B ? w.y - B : w.y)] |
+        window_flag(cuts, win, bins_per_rad, ho.w, ri_min, ri_max);
   return r;
 }
 
+// The windows of sorted hit s on a layer with nin inner layers (global bin gb), given to
+// put(k, window).
+template <class Put>
+__device__ __forceinline__ void reverse_windows(const Buffers& b, const pt_cuts& cuts,
+                                                const PairTable& pt, int32_t B, uint32_t gb,
+                                                float4 ho, int nin, uint32_t n_sorted, Put put) {
+  const float bins_per_rad = (float)B / kTwoPi;
+  const float a = 0.5f * cuts.kmax * ho.w;
+  const float asin_o = a >= 0.7f ? __int_as_float(0x7f800000) : asinf(a);
+  const float phi = azimuth(ho);
+  for (int k = 0; k < nin; ++k) {
+    uint2 rg = reverse_window(b, cuts, pt, B, bins_per_rad, gb, ho, asin_o, phi, k);
+    const uint32_t rx = rg.x & ~kWindowWraps, ry = rg.y & ~kWindowExact;
+    if (!PT_CHECK(b.cnt, (rx <= ry || (rg.x & kWindowWraps)) && rx <= n_sorted && ry <= n_sorted,
+                  DBG_DBL_WINDOW))
+      rg = make_uint2(0u, 0u);
+    put(k, rg);
+  }
+}
+
+// The windows of every sorted hit, one thread per hit, into the slots that the search then
+// overwrites with the hit's segments; the slots that the hit's layer does not use are written
+// empty.  In the search a chunk's windows take the instructions of searching one or two hits,
+// on as few lanes as the chunk has hits.  The whole call in us with the windows found here
+// (in the search): 64 pileup-200 events 5439 (5516), 7 gap-pair events 1109 (1133), one
+// pileup-200 event 320 (326); but one pileup-50 event 188 (185), where the launch costs more,
+// so contexts of fewer than kWindowsMinHits hits have no such launch.
+constexpr int64_t kWindowsMinHits = 32768;
+__global__ void k_windows(Buffers b, pt_cuts cuts, PairTable pt, int32_t B) {
+  pdl_sync();
+  const uint32_t n_sorted = b.bin_start[b.hdr->n_events * kLayers * B];
+  for (uint32_t s = blockIdx.x * blockDim.x + threadIdx.x; s < n_sorted;
+       s += gridDim.x * blockDim.x) {
+    const uint32_t gb = b.hbin[s];
+    const int nin = pt.n_inner[(gb / (uint32_t)B) % kLayers];
+    uint2* seg = b.seg + (uint64_t)s * pt.max_inner;
+    reverse_windows(b, cuts, pt, B, gb, b.hit4[s], nin, n_sorted,
+                    [&](int k, uint2 rg) { seg[k] = rg; });
+    for (int k = nin; k < pt.max_inner; ++k) seg[k] = make_uint2(0u, 0u);
+  }
+}
+
 // Warps take chunks of a few consecutive sorted (outer) hits (search_chunk), the first
-// by their own number, the others from a work counter.  The chunk's windows are found lane-parallel (one hit per lane, all of its loads in flight
-// at once) and kept in shared memory; the warp then searches them hit by hit.
+// by their own number, the others from a work counter.  The chunk's windows are read
+// (WINDOWS: k_windows has run) or found lane-parallel, one hit per lane, and kept in shared
+// memory; the warp then searches them hit by hit.
+template <bool WINDOWS>
 __global__ void __launch_bounds__(kWarpsPerBlock * 32, 5)
     k_doublets(Buffers b, pt_cuts cuts, PairTable pt, int32_t B, uint64_t cap_cells) {
   pdl_wait();
   __shared__ uint32_t st_val[kWarpsPerBlock][kStage];
-  __shared__ uint4 st_rng[kWarpsPerBlock][32][kMaxInner];
+  __shared__ uint2 st_rng[kWarpsPerBlock][32][kMaxInner];
   __shared__ float4 st_hit[kWarpsPerBlock][32];
   __shared__ uint8_t st_nin[kWarpsPerBlock][32];  // inner layers of each hit's layer
   const int lane = lane_id(), wib = threadIdx.x >> 5;
@@ -91,7 +123,6 @@ __global__ void __launch_bounds__(kWarpsPerBlock * 32, 5)
 
   const int E = b.hdr->n_events;
   const uint32_t n_sorted = b.bin_start[E * kLayers * B];
-  const float bins_per_rad = (float)B / kTwoPi;
   WarpChunk ch;
 
   const uint32_t n_warps = gridDim.x * kWarpsPerBlock;
@@ -106,19 +137,15 @@ __global__ void __launch_bounds__(kWarpsPerBlock * 32, 5)
       const uint32_t s = s0 + lane;
       const uint32_t gb = b.hbin[s];
       const float4 ho = b.hit4[s];
-      const float a = 0.5f * cuts.kmax * ho.w;
-      const float asin_o = a >= 0.7f ? __int_as_float(0x7f800000) : asinf(a);
-      const float phi = azimuth(ho);
-      st_hit[wib][lane] = ho;
       const int nin = pt.n_inner[(gb / (uint32_t)B) % kLayers];
+      st_hit[wib][lane] = ho;
       st_nin[wib][lane] = (uint8_t)nin;
-      for (int k = 0; k < nin; ++k) {
-        uint4 rg = reverse_window(b, cuts, pt, B, bins_per_rad, gb, ho, asin_o, phi, k);
-        const uint32_t rw = rg.w & ~kWindowExact;
-        if (!PT_CHECK(b.cnt, rg.x <= rg.y && rg.y <= n_sorted && rg.z <= rw && rw <= n_sorted,
-                      DBG_DBL_WINDOW))
-          rg = make_uint4(0u, 0u, 0u, 0u);
-        st_rng[wib][lane][k] = rg;
+      if (WINDOWS) {
+        for (int k = 0; k < nin; ++k)
+          st_rng[wib][lane][k] = b.seg[(uint64_t)s * pt.max_inner + k];
+      } else {
+        reverse_windows(b, cuts, pt, B, gb, ho, nin, n_sorted,
+                        [&](int k, uint2 rg) { st_rng[wib][lane][k] = rg; });
       }
     }
     __syncwarp();
@@ -130,12 +157,18 @@ __global__ void __launch_bounds__(kWarpsPerBlock * 32, 5)
       const float half_k = 0.5f * cuts.kmax * ho.w;
       // the slots the hit's layer does not use are written empty, so readers need not
       // know the hit's layer
-      if (lane >= nin && lane < pt.max_inner)
+      if (!WINDOWS && lane >= nin && lane < pt.max_inner)
         b.seg[(uint64_t)s * pt.max_inner + lane] = make_uint2(0u, 0u);
       for (int k = 0; k < nin; ++k) {
-        uint4 rg = st_rng[wib][j][k];
-        const float tiny = window_tiny(rg.w);
-        rg.w &= ~kWindowExact;
+        const uint2 win = st_rng[wib][j][k];
+        const float tiny = window_tiny(win.y);
+        uint4 rg = make_uint4(win.x & ~kWindowWraps, win.y & ~kWindowExact, 0u, 0u);
+        if (win.x & kWindowWraps) {
+          // the inner layer's bins: its start up to y, and x up to its end
+          const uint32_t el = b.hbin[s] / (uint32_t)B;
+          const uint32_t first = (el - el % kLayers + pt.inner[el % kLayers][k]) * (uint32_t)B;
+          rg = make_uint4(b.bin_start[first], rg.y, rg.x, b.bin_start[first + B]);
+        }
         uint32_t cnt = 0;
         // pass 1: test, stage up to kStage passing hits, count all; two candidates per
         // lane in flight (both loads issued before either test)
@@ -206,9 +239,16 @@ __global__ void __launch_bounds__(kWarpsPerBlock * 32, 5)
 }  // namespace
 
 void launch_doublets(const Buffers& b, const Params& p, const Launch& l, cudaStream_t s) {
-  PT_TRACE(l, s, "k_doublets",
-           launch_pdl(k_doublets, l.sgrid, kWarpsPerBlock * 32, 0, s, b, p.cuts, p.pairs,
-                      p.phi_bins, (uint64_t)p.max_cells));
+  constexpr unsigned block = kWarpsPerBlock * 32;
+  if (p.max_hits >= kWindowsMinHits)
+    PT_TRACE(l, s, "k_doublets",
+             launch_pdl(k_windows, l.grid, 256, 0, s, b, p.cuts, p.pairs, p.phi_bins),
+             launch_pdl(k_doublets<true>, l.sgrid, block, 0, s, b, p.cuts, p.pairs, p.phi_bins,
+                        (uint64_t)p.max_cells));
+  else
+    PT_TRACE(l, s, "k_doublets",
+             launch_pdl(k_doublets<false>, l.sgrid, block, 0, s, b, p.cuts, p.pairs, p.phi_bins,
+                        (uint64_t)p.max_cells));
 }
 
 }  // namespace ptca

@@ -231,7 +231,7 @@ struct Buffers {
   uint32_t* layer_zmax;      //   z per event layer (~0 and 0 for an empty layer)
   // incoming segments: per sorted (outer) hit and inner-layer slot, the cells ending on
   // the hit from that layer, cells [x, x + y), ordered by inner hit; the table's
-  // max_inner slots per hit, all written
+  // max_inner slots per hit, all written; before the doublet search the hit's windows
   uint2* seg;                // [max_hits*kMaxInner]
   // cells
   uint32_t* cell_in;         // [max_cells] inner hit (sorted index); the outer hit is the
@@ -520,7 +520,8 @@ __device__ __forceinline__ bool doublet_pass(const pt_cuts& c, float4 hi, float4
 // and the half-plane cut the doublet search of 64 pileup-200 events takes 1331 instead of
 // 1434 us, the whole call with it in the link search as well 5735 instead of 5790.
 constexpr float kHalfPlane = 1.569f;  // pi/2, less the azimuth's rounding and that of the cut
-constexpr uint32_t kWindowExact = 0x80000000u;  // a window's flag, in its last word
+constexpr uint32_t kWindowExact = 0x80000000u;  // a window's flags, in its last word
+constexpr uint32_t kWindowWraps = 0x80000000u;  //   and in its first
 __device__ __forceinline__ float window_tiny(uint32_t flagged) {
   return flagged & kWindowExact ? __int_as_float(0x7f800000) : 1e-20f;
 }

@@ -48,17 +48,19 @@ def _event(kmax, scale, n, bins, seed):
     (0.0, 1.0, 100),
 ])
 @pytest.mark.parametrize("bins", [16, 256, 4096])
-def test_cells_and_links(cuts, kmax, scale, n, bins):
+@pytest.mark.parametrize("room", [4096, 65536])  # windows found in the search, or before it
+def test_cells_and_links(cuts, kmax, scale, n, bins, room):
     c = dict(cuts, kmax=kmax / scale, z0max=cuts["z0max"] * scale, rz0=cuts["rz0"] * scale,
              dca_b0=cuts["dca_b0"] * scale, dca_other=cuts["dca_other"] * scale)
     hits = _event(kmax, scale, n, bins, 97 + bins)
     ref = oracle.reconstruct(*hits, c)
     n_hits = len(hits[0])
-    cap = pt.default_capacity(max_events=1, hits_per_event=n_hits, cells_per_event=1 << 20,
+    cap = pt.default_capacity(max_events=1, hits_per_event=room, cells_per_event=1 << 20,
                               links_per_event=1 << 20, ntuplets_per_event=1 << 16, phi_bins=bins)
     with pt.Context(cuts=c, capacity=cap) as ctx:
         ctx.pt_load_batch(np.array([0, n_hits], np.int32), *hits)
         ctx.pt_build_doublets()
+        ctx.pt_build_doublets()  # the search leaves nothing behind that a second one trips on
         ctx.pt_connect_cells()
         ci, co, _ = ctx.pt_get_cells()
         h0, h1, h2, q, _ = ctx.pt_get_links()
