@@ -50,14 +50,14 @@ CONFIG4_SEED0 = 5000  # batch workload: 64 events, pileup ~ Poisson(140) clipped
 # DRAM traffic per event of the main kernels from one ncu capture (8 PU200 events per
 # launch, profiles/), valid only while the kernel's sources hash to the recorded value.
 NCU_TRAFFIC = {
-    "k_doublets": {"bytes_per_event": 24503712, "issue_active_pct": 58.4,
-                   "warp_inst_per_event": 25200120, "sha": "2a8aa9a0d737"},
-    "k_connect": {"bytes_per_event": 22363520, "issue_active_pct": 57.7,
-                  "warp_inst_per_event": 45554002, "sha": "0d56a924773e"},
-    "k_link_targets": {"bytes_per_event": 14528864, "issue_active_pct": 19.2,
-                       "warp_inst_per_event": 840076, "sha": "0d56a924773e"},
-    "k_find_ntuplets": {"bytes_per_event": 35716608, "issue_active_pct": 19.5,
-                        "warp_inst_per_event": 2328577, "sha": "e73b2d03adb5"},
+    "k_doublets": {"bytes_per_event": 5029216, "issue_active_pct": 71.4,
+                   "warp_inst_per_event": 23067719, "sha": "677665fbbed0"},
+    "k_connect": {"bytes_per_event": 31619872, "issue_active_pct": 71.4,
+                  "warp_inst_per_event": 45488219, "sha": "fd6da959980f"},
+    "k_link_targets": {"bytes_per_event": 13895776, "issue_active_pct": 17.9,
+                       "warp_inst_per_event": 773268, "sha": "fd6da959980f"},
+    "k_find_ntuplets": {"bytes_per_event": 23664736, "issue_active_pct": 28.7,
+                        "warp_inst_per_event": 2262945, "sha": "2b7043838416"},
 }
 SMS, SCHEDULERS_PER_SM = 152, 4  # GB300: each scheduler issues one warp instruction a cycle
 

@@ -226,8 +226,9 @@ pt_status pt_fit_tracks(pt_ctx* ctx, int64_t* n_tracks);
  * circle + line fit is the reference; its offsets at the hits, one curvature
  * correction and the multiple-scattering kinks at the interior hits (Highland variances
  * for x0_barrel / x0_disk radiation lengths per layer at normal incidence, with 10 um
- * r-phi and 20 um z / r hit errors) are solved by linear least squares in float64, and
- * the parameters at the closest approach replace the track's; chi2_circle and
+ * r-phi and 20 um z / r hit errors) are solved by linear least squares in pairs of float32
+ * (in float64 for a track whose weights span more than those hold), and the parameters at
+ * the closest approach replace the track's; chi2_circle and
  * chi2_line become the two planes' broken-line chi2 (measurements plus kinks).  A
  * track whose reference is not finite, has |kappa| < 1e-7 /cm or whose hits are not
  * strictly ordered along the reference circle keeps its fit.  Run after pt_fit_tracks
