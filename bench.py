@@ -51,13 +51,13 @@ CONFIG4_SEED0 = 5000  # batch workload: 64 events, pileup ~ Poisson(140) clipped
 # launch, profiles/), valid only while the kernel's sources hash to the recorded value.
 NCU_TRAFFIC = {
     "k_doublets": {"bytes_per_event": 5029216, "issue_active_pct": 71.4,
-                   "warp_inst_per_event": 23067719, "sha": "677665fbbed0"},
+                   "warp_inst_per_event": 23067719, "sha": "2baedfdfb43d"},
     "k_connect": {"bytes_per_event": 31619872, "issue_active_pct": 71.4,
-                  "warp_inst_per_event": 45488219, "sha": "fd6da959980f"},
+                  "warp_inst_per_event": 45488219, "sha": "131890a515aa"},
     "k_link_targets": {"bytes_per_event": 13895776, "issue_active_pct": 17.9,
-                       "warp_inst_per_event": 773268, "sha": "fd6da959980f"},
+                       "warp_inst_per_event": 773268, "sha": "131890a515aa"},
     "k_find_ntuplets": {"bytes_per_event": 23664736, "issue_active_pct": 28.7,
-                        "warp_inst_per_event": 2262945, "sha": "2b7043838416"},
+                        "warp_inst_per_event": 2262945, "sha": "645e5ed24950"},
 }
 SMS, SCHEDULERS_PER_SM = 152, 4  # GB300: each scheduler issues one warp instruction a cycle
 

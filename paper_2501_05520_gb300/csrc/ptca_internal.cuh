@@ -259,7 +259,7 @@ struct Buffers {
                              //   none)
   uint32_t* sv_cnt;          // [max_hits + 1] surviving ntuplets that start at the hit (the
                              //   memory of fb_cnt)
-  uint32_t* sv_start;        // [max_hits + 1]   and the first one's place
+  uint32_t* sv_start;        // [max_hits + 1]   and the first one's place (that of fb_start)
   uint32_t* best_list;       // [max_ntuplets] ntuplets that may survive (kHole: it did not)
   uint8_t* used;             // [max_hits] on a surviving ntuplet of four or more hits
   uint32_t* sv;              // [max_ntuplets] cleaned ntuplets in canonical order

@@ -201,7 +201,7 @@ size_t layout(const pt_capacity& c, char* base, Buffers* b, GateWeights** gate =
   t.nt_next = (uint32_t*)take(T * 4);
   t.nt_head = (uint32_t*)take(N * 4);
   t.sv_cnt = t.fb_cnt;
-  t.sv_start = (uint32_t*)take((N + 1) * 4);
+  t.sv_start = t.fb_start;  // the fishbone step is over when the survivors are counted
   t.best_list = (uint32_t*)take(T * 4);
   t.used = (uint8_t*)take(N);
   t.sv = (uint32_t*)take(T * 4);
