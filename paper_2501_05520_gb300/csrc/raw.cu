@@ -19,7 +19,7 @@
 // smallest label among itself, its label's label and its neighbours until no label
 // changes, which leaves every pixel labelled with its cluster's first position; the
 // adc-weighted sums are exact integer atomics on those positions, and the positions in
-// order give the run's hits at the run's first digi position.  Runs of up to 192 digis
+// order give the run's hits at the run's first digi position.  Runs of up to 224 digis
 // take one warp each with small buffers (many warps per SM to hide the shared-memory and
 // load latency); that launch lists the longer runs (up to 1024), and a second launch
 // gives each of those a whole block, which runs the same steps over its pixels.  A
@@ -33,15 +33,14 @@ namespace {
 
 constexpr int kRunMax = 1024;           // digis of one module in one event
 // A run's time is the latency of its shared-memory chains, so both launches want warps: with
-// buffers for 192 digis 48 warps fit a multiprocessor (36 with 256, but fewer runs are left
-// for the blocks), and a block of 512 threads takes a long run's pixels in at most two steps.
-// pt_load_raw in us with 192 digis and 512 threads (192 and 256; 256 and 512; 256 and 256; 384
-// or 128 and 256): 6 pileup-200 events 180 (184; 186; 190; 197, 188), one 120 (126; 126; 132),
-// 16 of them 296 (301; 300; 301), 12 of 7000 particles 202 (202; 203; 203).
-constexpr int kRunSmall = 192;          // runs of up to this many digis take the small launch
+// buffers for 224 digis 40 warps fit a multiprocessor, and a block of 512 threads takes a long
+// run's pixels in at most two steps.  pt_load_raw in us with 224 digis and 512 threads (192
+// digis, 48 warps and 512; 256 digis, 36 warps and 512; the same and 256): pileup-200 events, 6
+// of them 176 (183; 187; 191), 16 of them 301 (300; 301; 301), 64 of them 851 (875; 849; 851).
+constexpr int kRunSmall = 224;          // runs of up to this many digis take the small launch
 constexpr int kClusterMax = 128;        // pixels of one cluster (32-bit exact sums)
-constexpr int kSmallWarps = 4;          // warps per block of the warp-per-run launch (17 KB)
-constexpr int kSmallBlocksPerSm = 12;
+constexpr int kSmallWarps = 4;          // warps per block of the warp-per-run launch (20 KB)
+constexpr int kSmallBlocksPerSm = 10;
 constexpr int kBigThreads = 512;        // block of the block-per-run launch (22.5 KB shared)
 constexpr int kBigBlocksPerSm = 4;
 constexpr int kLoadBatch = 8;           // digis per lane loaded before use

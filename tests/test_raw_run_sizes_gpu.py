@@ -1,4 +1,4 @@
-"""Module runs around the sizes where the clustering changes hands: 192 digis (a warp, then a
+"""Module runs around the sizes where the clustering changes hands: 224 digis (a warp, then a
 block), 512 (one step of the block, then two) and 1024 (the most), against the oracle.  Hits in
 the oracle's order, positions within the 2e-5 cm that float32 rounding leaves."""
 
@@ -18,8 +18,8 @@ from paper_2501_05520_gb300 import pixels as ppix  # noqa: E402
 from test_raw_gpu import _sparse_run  # noqa: E402
 
 
-@pytest.mark.parametrize("sizes", [(31, 32, 33, 191, 192), (193, 192, 1), (511, 512, 513),
-                                   (1023, 1024, 192, 193)])
+@pytest.mark.parametrize("sizes", [(31, 32, 33, 223, 224), (225, 224, 1), (511, 512, 513),
+                                   (1023, 1024, 224, 225)])
 def test_sizes(cuts, sizes):
     rng = np.random.default_rng(sum(sizes))
     table = opix.modules(ppix.PARAMS)
