@@ -365,8 +365,11 @@ pt_status check_status(pt_ctx* c) {
   return PT_OK;
 }
 
-// Device memory of the context's own GPU, which its kernels may use in place.
-bool own_device_memory(const pt_ctx* c, const void* p) {
+// Device memory of the context's own GPU, aligned as its type wants, which its kernels may
+// use in place (a copy takes any address).
+template <class T>
+bool own_device_memory(const pt_ctx* c, const T* p) {
+  if ((uintptr_t)p % alignof(T)) return false;
   cudaPointerAttributes a;
   if (cudaPointerGetAttributes(&a, p) != cudaSuccess) {
     cudaGetLastError();
