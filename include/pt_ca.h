@@ -337,9 +337,11 @@ pt_status pt_reconstruct_batch(pt_ctx* ctx, int n_events, const int64_t* hit_off
                                int out_on_device);
 
 /* Load a batch and enqueue all GPU stages (doublets, links, ntuplets, fit, export) as
- * one CUDA graph on the context's stream, without synchronising: results stay on the
- * device until a getter (pt_get_ntuplets, pt_get_tracks, ...) is called.  Input
- * validation errors are returned immediately; capacity errors by the next getter. */
+ * one CUDA graph on the context's stream, without waiting for them: results stay on the
+ * device until a getter (pt_get_ntuplets, pt_get_tracks, ...) is called.  The call returns
+ * when the stream has taken the inputs, behind work of the context that is still queued
+ * (pt_load_hits and pt_load_batch likewise).  Input validation errors are returned
+ * immediately; capacity errors by the next getter. */
 pt_status pt_enqueue_batch(pt_ctx* ctx, int n_events, const int64_t* hit_offsets,
                            const float* x, const float* y, const float* z, const uint8_t* layer,
                            int on_device);

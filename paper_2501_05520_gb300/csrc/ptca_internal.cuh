@@ -366,6 +366,9 @@ int64_t server_finished(pt_server* s);
 // counters, status check of that copy, and copies of the cleaned ntuplets, tracks and
 // per-event offsets into host memory, each completion recorded on `done`.
 cudaStream_t ctx_stream(pt_ctx* c);
+// pt_enqueue_batch that returns at once; the caller keeps the inputs until the batch is done.
+pt_status ctx_enqueue_async(pt_ctx* c, int n_events, const int64_t* hit_offsets, const float* x,
+                            const float* y, const float* z, const uint8_t* layer, int on_device);
 pt_status ctx_counters_async(pt_ctx* c, cudaEvent_t done);
 pt_status ctx_read_counters(pt_ctx* c, int64_t* n_ntuplets);
 pt_status ctx_results_async(pt_ctx* c, int64_t S, int32_t* hits, uint8_t* nhits,

@@ -274,7 +274,8 @@ struct pt_ctx {
   pt_track* r_tracks = nullptr;
   int32_t* r_hits = nullptr;
   uint8_t* r_n = nullptr;
-  cudaEvent_t staged = nullptr;
+  cudaEvent_t staged = nullptr;  // the inputs have been copied
+  bool copying = false;          // stage_inputs queued copies from the caller's arrays
   cudaGraphExec_t graph = nullptr;
   // validation staging, allocated on first use
   char* val = nullptr;
@@ -390,10 +391,12 @@ struct Results {
 // Header, offsets and inputs of a batch to the device.  A few copies cost more than they
 // move: one 50-particle event took 30 us to stage in six, so a small batch from the host
 // goes up in one, packed behind the header, and arrays that the caller has on the device
-// are left to the binning pass to copy.
+// are left to the binning pass to copy, by a call that synchronises (`whole`, the one that
+// takes results).  `staged` is recorded behind the copies: a call that returns earlier
+// waits for it (inputs_taken), since the inputs are the caller's again then.
 pt_status stage_inputs(pt_ctx* c, int n_events, const int64_t* off, const float* x,
                        const float* y, const float* z, const uint8_t* layer, int on_device,
-                       const Results& out = {}) {
+                       const Results* whole = nullptr) {
   if (n_events < 1) return fail(PT_ERR_INVALID, "n_events must be >= 1");
   if (n_events > c->cap.max_events)
     return fail(PT_ERR_CAPACITY, "max_events = %lld is too small: %d events given",
@@ -420,6 +423,7 @@ pt_status stage_inputs(pt_ctx* c, int n_events, const int64_t* off, const float*
   h = BatchHeader{};
   h.n_events = n_events;
   h.n_hits = (int32_t)n;
+  const Results out = whole ? *whole : Results{};
   h.out_hits = out.hits;
   h.out_n = out.n;
   h.out_tracks = out.tracks;
@@ -442,7 +446,7 @@ pt_status stage_inputs(pt_ctx* c, int n_events, const int64_t* off, const float*
     h.layer = (const uint8_t*)(h.z + n);
     up = head + (size_t)n * 13;
     copies = false;
-  } else if (n > 0 && on_device && own_device_memory(c, x) && own_device_memory(c, y) &&
+  } else if (n > 0 && whole && on_device && own_device_memory(c, x) && own_device_memory(c, y) &&
              own_device_memory(c, z) && own_device_memory(c, layer)) {
     h.x = x;
     h.y = y;
@@ -459,12 +463,23 @@ pt_status stage_inputs(pt_ctx* c, int n_events, const int64_t* off, const float*
     PT_CUDA(cudaMemcpyAsync(c->B.in_layer, layer, n, k, c->stream));
   }
   PT_CUDA(cudaEventRecord(c->staged, c->stream));
+  c->copying = copies;
   c->n_events = n_events;
   c->n_hits = n;
   c->hit_off.assign(off, off + n_events + 1);
   c->loaded = true;
   c->fitted = false;
   c->vtx_ready = false;
+  return PT_OK;
+}
+
+// Waits until the stream has copied the caller's inputs (in a captured stream they are the
+// replays' to read).
+pt_status inputs_taken(pt_ctx* c) {
+  if (!c->copying) return PT_OK;
+  cudaStreamCaptureStatus st;
+  PT_CUDA(cudaStreamIsCapturing(c->stream, &st));
+  if (st == cudaStreamCaptureStatusNone) PT_CUDA(cudaEventSynchronize(c->staged));
   return PT_OK;
 }
 
@@ -502,6 +517,14 @@ pt_status ensure_graph(pt_ctx* c) {
   return PT_OK;
 }
 
+pt_status launch_graph(pt_ctx* c) {
+  PT_TRY(ensure_graph(c));
+  PT_CUDA(cudaGraphLaunch(c->graph, c->stream));
+  c->fitted = true;
+  c->links_masked = c->masked();  // the graph's link stage ran in the current form
+  return PT_OK;
+}
+
 pt_status need_loaded(pt_ctx* c) {
   if (!c) return fail(PT_ERR_INVALID, "context is NULL");
   if (!c->loaded) return fail(PT_ERR_INVALID, "no hits loaded");
@@ -532,6 +555,13 @@ namespace ptca {
 void set_last_error(const char* msg) { g_err = msg; }
 
 cudaStream_t ctx_stream(pt_ctx* c) { return c->stream; }
+
+pt_status ctx_enqueue_async(pt_ctx* c, int n_events, const int64_t* hit_offsets, const float* x,
+                            const float* y, const float* z, const uint8_t* layer, int on_device) {
+  DeviceGuard guard(c->device);
+  PT_TRY(stage_inputs(c, n_events, hit_offsets, x, y, z, layer, on_device));
+  return launch_graph(c);
+}
 
 pt_status ctx_counters_async(pt_ctx* c, cudaEvent_t done) {
   DeviceGuard guard(c->device);  // the batch's graph ends with the counters' copy
@@ -729,7 +759,8 @@ pt_status pt_load_batch(pt_ctx* c, int n_events, const int64_t* hit_offsets, con
   PT_TRY(stage_inputs(c, n_events, hit_offsets, x, y, z, layer, on_device));
   launch_clear(c->B, c->P, c->L, c->stream);
   launch_bin_hits(c->B, c->P, c->L, c->stream);
-  return last_launch();
+  PT_TRY(last_launch());
+  return inputs_taken(c);
 }
 
 pt_status pt_load_hits(pt_ctx* c, int64_t n, const float* x, const float* y, const float* z,
@@ -1374,12 +1405,8 @@ pt_status pt_enqueue_batch(pt_ctx* c, int n_events, const int64_t* hit_offsets, 
   g_err.clear();
   if (!c) return fail(PT_ERR_INVALID, "context is NULL");
   DeviceGuard guard(c->device);
-  PT_TRY(stage_inputs(c, n_events, hit_offsets, x, y, z, layer, on_device));
-  PT_TRY(ensure_graph(c));
-  PT_CUDA(cudaGraphLaunch(c->graph, c->stream));
-  c->fitted = true;
-  c->links_masked = c->masked();  // the graph's link stage ran in the current form
-  return PT_OK;
+  PT_TRY(ctx_enqueue_async(c, n_events, hit_offsets, x, y, z, layer, on_device));
+  return inputs_taken(c);
 }
 
 pt_status pt_reconstruct_batch(pt_ctx* c, int n_events, const int64_t* hit_offsets,
@@ -1405,11 +1432,8 @@ pt_status pt_reconstruct_batch(pt_ctx* c, int n_events, const int64_t* hit_offse
     out = {c->r_hits, c->r_n, c->r_tracks, c->r_off,
            std::min({cap, (int64_t)c->cap.max_ntuplets, kSmallTracks})};
   }
-  PT_TRY(stage_inputs(c, n_events, hit_offsets, x, y, z, layer, on_device, out));
-  PT_TRY(ensure_graph(c));
-  PT_CUDA(cudaGraphLaunch(c->graph, c->stream));
-  c->fitted = true;
-  c->links_masked = c->masked();  // the graph's link stage ran in the current form
+  PT_TRY(stage_inputs(c, n_events, hit_offsets, x, y, z, layer, on_device, &out));
+  PT_TRY(launch_graph(c));
   PT_CUDA(cudaStreamSynchronize(c->stream));  // the graph ends with the counters' copy
   PT_TRY(check_status(c));
   const int64_t S = (int64_t)c->h_cnt[CNT_SV];

@@ -139,7 +139,7 @@ bool dispatch(pt_server* s, Slot& sl) {
     sl.hoff[e + 1] = o + n;
   }
   s->batches += 1;
-  pt_status st = pt_enqueue_batch(sl.ctx, E, sl.hoff, sl.hx, sl.hy, sl.hz, sl.hl, 0);
+  pt_status st = ctx_enqueue_async(sl.ctx, E, sl.hoff, sl.hx, sl.hy, sl.hz, sl.hl, 0);
   if (st == PT_OK) st = ctx_counters_async(sl.ctx, sl.ev);
   if (st != PT_OK) {
     const std::string m = pt_last_error();
