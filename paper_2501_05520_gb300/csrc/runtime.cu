@@ -1257,9 +1257,15 @@ pt_status pt_gate_score(pt_ctx* c, const float* feat, int64_t n, float* out) {
   DeviceGuard guard(c->device);
   // a status word of its own, so that the loaded batch's status does not leak into the
   // answer; it is zero unless a call timed out, which clears it
-  launch_gate_score(c->gate, feat, n, out, &c->B.cnt[CNT_SCORE_STATUS], c->L.sms,
+  // the kernel reads its rows while it writes scores: where the two share memory, the scores
+  // go to the link stage's feature rows first (32 bytes per link, free after the gate)
+  const char *f0 = (const char*)feat, *s0 = (const char*)out;
+  const bool shared = f0 < s0 + n * 4 && s0 < f0 + n * kGateFeat * 4;
+  float* scores = shared ? (float*)c->B.gate_x : out;
+  launch_gate_score(c->gate, feat, n, scores, &c->B.cnt[CNT_SCORE_STATUS], c->L.sms,
                     c->P.wait_cycles, c->stream);
   PT_TRY(last_launch());
+  if (shared) PT_TRY(copy_out(c, out, scores, (size_t)n * 4, 1));
   PT_CUDA(cudaMemcpyAsync(c->h_cnt, c->B.cnt, CNT_N * 8, cudaMemcpyDeviceToHost, c->stream));
   PT_CUDA(cudaStreamSynchronize(c->stream));
   if (c->h_cnt[CNT_SCORE_STATUS])
