@@ -210,8 +210,8 @@ struct Buffers {
   float* in_y;
   float* in_z;
   uint8_t* in_layer;
-  int32_t* hit_off;          // [max_events + 1], directly after the header; then room for
-                             //   the inputs of a small batch
+  int32_t* hit_off;          // [max_events + 1], directly after the header; a small
+                             //   batch's inputs follow, into hit4, until it is written
   uint32_t* in_bin;          // [max_hits] global bin of input hit (or ~0)
   uint32_t* in_rank;         // [max_hits] rank within the bin
   // hits sorted by (event, layer, phi bin)

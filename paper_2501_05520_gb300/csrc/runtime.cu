@@ -147,11 +147,11 @@ pt_status fail(pt_status st, const char* fmt, ...) {
 
 constexpr size_t kAlign = 256;
 
-// The header, the events' offsets and the inputs of a small batch, which go up in one copy
-// from a pinned block of the same layout.
+// The header and the events' offsets, with the inputs of a small batch behind them: they go up
+// in one copy from a pinned block of the same layout.
+size_t header_bytes(const pt_capacity& c) { return kHeaderBytes + (size_t)(c.max_events + 1) * 4; }
 size_t stage_bytes(const pt_capacity& c) {
-  return kHeaderBytes + (size_t)(c.max_events + 1) * 4 +
-         (size_t)std::min(c.max_hits, kSmallHits) * 13;
+  return header_bytes(c) + (size_t)std::min(c.max_hits, kSmallHits) * 13;
 }
 
 // Carves the workspace; with base == nullptr only computes the size.
@@ -167,8 +167,11 @@ size_t layout(const pt_capacity& c, char* base, Buffers* b, GateWeights** gate =
   const size_t L = (size_t)c.max_links, T = (size_t)c.max_ntuplets;
   const size_t NB = E * kLayers * (size_t)c.phi_bins + 1;
   Buffers t{};
-  t.hdr = (BatchHeader*)take(stage_bytes(c));
+  t.hdr = (BatchHeader*)take(header_bytes(c));
   t.hit_off = (int32_t*)(base ? base + kHeaderBytes : nullptr);
+  // A small batch's inputs (13 bytes a hit) reach from the offsets into the sorted hits, which
+  // are written when the binning pass has copied the inputs to their arrays.
+  t.hit4 = (float4*)take(N * 16);
   t.cnt = (unsigned long long*)take(CNT_N * 8);
   t.in_x = (float*)take(N * 4);
   t.in_y = (float*)take(N * 4);
@@ -176,7 +179,6 @@ size_t layout(const pt_capacity& c, char* base, Buffers* b, GateWeights** gate =
   t.in_layer = (uint8_t*)take(N);
   t.in_bin = (uint32_t*)take(N * 4);
   t.in_rank = (uint32_t*)take(N * 4);
-  t.hit4 = (float4*)take(N * 16);
   t.perm = (uint32_t*)take(N * 4);
   t.hbin = (uint32_t*)take(N * 4);
   t.bin_cnt = (uint32_t*)take(NB * 4);
@@ -393,10 +395,11 @@ struct Results {
 // goes up in one, packed behind the header, and arrays that the caller has on the device
 // are left to the binning pass to copy, by a call that synchronises (`whole`, the one that
 // takes results).  `staged` is recorded behind the copies: a call that returns earlier
-// waits for it (inputs_taken), since the inputs are the caller's again then.
+// waits for it (inputs_taken), since the inputs are the caller's again then.  `repeat`: the
+// chain will run more than once on them (the inputs behind the header last for one run).
 pt_status stage_inputs(pt_ctx* c, int n_events, const int64_t* off, const float* x,
                        const float* y, const float* z, const uint8_t* layer, int on_device,
-                       const Results* whole = nullptr) {
+                       const Results* whole = nullptr, bool repeat = false) {
   if (n_events < 1) return fail(PT_ERR_INVALID, "n_events must be >= 1");
   if (n_events > c->cap.max_events)
     return fail(PT_ERR_CAPACITY, "max_events = %lld is too small: %d events given",
@@ -433,7 +436,7 @@ pt_status stage_inputs(pt_ctx* c, int n_events, const int64_t* off, const float*
   const size_t head = kHeaderBytes + (size_t)(n_events + 1) * 4;
   size_t up = head;
   bool copies = n > 0;
-  if (n > 0 && !on_device && n <= kSmallHits) {
+  if (n > 0 && !on_device && n <= kSmallHits && !repeat) {
     char* p = c->h_stage + head;
     std::memcpy(p, x, n * 4);
     std::memcpy(p + n * 4, y, n * 4);
@@ -1370,7 +1373,7 @@ pt_status pt_autotune(const pt_geometry* geom, const pt_cuts* cuts, const pt_cap
     cudaEvent_t e0, e1;
     cudaEventCreate(&e0);
     cudaEventCreate(&e1);
-    pt_status st = stage_inputs(ctx, n_events, hit_offsets, x, y, z, layer, 0);
+    pt_status st = stage_inputs(ctx, n_events, hit_offsets, x, y, z, layer, 0, nullptr, true);
     for (int j = 0; j < n_bps * n_sbps && st == PT_OK; ++j) {
       const int jb = j / n_sbps, js = j % n_sbps;
       st = pt_set_launch(ctx, blocks_per_sm[jb], search_blocks_per_sm[js]);
