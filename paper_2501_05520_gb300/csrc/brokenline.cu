@@ -33,10 +33,13 @@
 // centimetres, and the normal equations mix weights of 1e6 (hits) and 1e4..1e8 (kinks):
 // 24 bits are too few.  GB300 issues a float64 operation at 1/64 of the float32 rate, so the
 // numbers are pairs of floats (F2, 48 bits: 7 float32 operations for a product, 11 for a
-// sum); a track whose kinks outweigh its hits by more than 1e10 (so that too few of the 48
-// bits are left for the hits), or whose pass leaves the range of float32 anywhere (a result
-// that is not finite), is done in float64 by the same template.  The geometry is written so that
-// nothing cancels: with q = (sin phi0, -cos phi0), a hit p has eps = N / (1 + |kappa0| |p -
+// sum); a track whose kinks outweigh its hits by more than 1e6 (so that too few of the 48
+// bits are left for the hits: kStiffMax), or whose pass leaves the range of float32 anywhere
+// (a result that is not finite), is done in float64 by the same template.  On 211k tracks, of
+// events of 800 to 4400 particles, the errors against a 64-bit reference are the ones that a
+// pass in float64 has (the results of the two differ by at most 6e-8 of a parameter's spread);
+// they come from the turning angle below.  The geometry is written so that nothing cancels:
+// with q = (sin phi0, -cos phi0), a hit p has eps = N / (1 + |kappa0| |p -
 // c|), N = d0 (2 - kappa0 d0) - kappa0 p.p + 2 (kappa0 d0 - 1) p.q, and turning angle
 // atan2(p.(cos phi0, sin phi0) / kappa0, (1 + kappa0 (p.q - d0)) / kappa0^2) (the cross and
 // scalar products of the closest approach and p seen from c), c the circle's centre.  The
@@ -154,9 +157,14 @@ template <class T>
 constexpr bool kPairs = false;
 template <>
 constexpr bool kPairs<F2> = true;
-// Largest weight of a kink in the normal equations that pairs of floats take (1e10 times a
-// hit's).
-constexpr float kStiffMax = 1e16f;
+// Largest weight of a kink in the normal equations that pairs of floats take: 1e6 times a hit's
+// in the transverse plane (1e6 /cm^2) and at most 4e6 times one's in the longitudinal plane
+// (2.5e5 on the barrel, 2.5e5 / cot^2 on a disk, where the kinks lose a factor 1 + cot^2 too).
+// There the solved offsets are within 2e-9 cm of the exact ones (5e-7 of a hit's error), less
+// than the float32 results resolve, and the results equal those of the float64 form to one unit
+// in the last place; at 1e10 the offsets were up to 1e-3 of a hit's error away and z0 40 units.
+// A track of 1 GeV through 2 % of a radiation length has 1e4, one of 2 TeV reaches the limit.
+constexpr float kStiffMax = 1e12f;
 
 // sin and cos of a float32 angle within +-pi (a track's phi0).
 __device__ __forceinline__ void sin_cos(float x, double& s, double& c) { sincos((double)x, &s, &c); }
