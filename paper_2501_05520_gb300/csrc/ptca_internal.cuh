@@ -39,6 +39,7 @@ enum : int {
   CNT_SCORE_STATUS = 9,  // status bits of the standalone gate scoring (pt_gate_score)
   CNT_CELLS_USED = 10,  // cells written (CNT_CELLS counts reserved slots incl. holes)
   CNT_LINKS_USED = 11,  // links written (CNT_LINKS counts reserved slots incl. holes)
+  CNT_SCAN_EV = 13,     // events (size of the scan over per-event vertex counts)
   CNT_VTX = 14,         // vertices of the batch
   CNT_RAW_STATUS = 15,  // raw input: status bits (RAW_*), not reset by the chain
   CNT_RAW_DIGIS = 16,   // raw input: digis of the batch (size of the run-flag scan)
@@ -269,7 +270,8 @@ struct Buffers {
   pt_vertex* vtx_stage;      // [max_ntuplets / 2 + 1] event e's vertices from floor(t0 / 2)
   pt_vertex* vtx;            // [max_ntuplets / 2 + 1] the batch's vertices, events in order
   int32_t* trk_vtx;          // [max_ntuplets] vertex of each track, -1 for none
-  uint32_t* ev_nv;           // [max_events + 1] vertices per event
+  uint32_t* ev_nv;           // [max_events + 1] vertices per event (large batches: scanned in
+                             //   place, vertices before each event)
   int64_t* ev_vtx_off;       // [max_events + 1] vertices before each event
   // learned gate (valid when enabled)
   uint16_t* gate_x;          // [max_links*16] bf16 features per link slot (12 used)

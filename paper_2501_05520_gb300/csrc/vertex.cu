@@ -23,6 +23,8 @@
 // Bound by the latency of the passes of one block.  12 pileup-200 events (9.8k
 // tracks each): 52 + 7 us, against 328 us for the bitonic sort with one thread per vertex
 // and 31 us for a scan and a placing kernel of one block per event.
+#include <algorithm>
+
 #include "ptca_internal.cuh"
 
 namespace ptca {
@@ -36,15 +38,19 @@ constexpr int kVtxBucketMax = 512;                // tracks of one bucket that a
 // keys (8 bytes), buckets / scan array (4 bytes), first track of each vertex (2 bytes)
 constexpr size_t kVtxSmem = (size_t)kVtxMax * 12 + (size_t)kVtxMax / 2 * 2;
 
-// In-place exclusive scan of a[0..kVtxMax) (kVtxPer consecutive entries per thread);
-// returns the total.  All threads of the block take part.
-__device__ uint32_t vtx_block_scan(uint32_t* a, uint32_t* warp_tot) {
+// In-place exclusive scan of a[0, per * kVtxThreads), `per` <= kVtxPer consecutive entries per
+// thread (FULL: kVtxPer of them, read four at a time); returns the total.  All threads of the
+// block take part.
+template <bool FULL>
+__device__ uint32_t vtx_block_scan_of(uint32_t* a, int per, uint32_t* warp_tot) {
+  if (FULL) per = kVtxPer;
   const int t = threadIdx.x, lane = t & 31, w = t >> 5;
   uint32_t loc[kVtxPer];
   uint32_t s = 0;
 #pragma unroll
   for (int i = 0; i < kVtxPer; ++i) {
-    loc[i] = a[t * kVtxPer + i];
+    if (i >= per) break;
+    loc[i] = a[t * per + i];
     s += loc[i];
   }
   const uint32_t inc = warp_incl_scan(s);
@@ -60,12 +66,18 @@ __device__ uint32_t vtx_block_scan(uint32_t* a, uint32_t* warp_tot) {
   uint32_t run = warp_tot[w] + inc - s;
 #pragma unroll
   for (int i = 0; i < kVtxPer; ++i) {
-    a[t * kVtxPer + i] = run;
+    if (i >= per) break;
+    a[t * per + i] = run;
     run += loc[i];
   }
   const uint32_t total = warp_tot[32];
   __syncthreads();
   return total;
+}
+
+__device__ __forceinline__ uint32_t vtx_block_scan(uint32_t* a, int per, uint32_t* warp_tot) {
+  return per == kVtxPer ? vtx_block_scan_of<true>(a, per, warp_tot)
+                        : vtx_block_scan_of<false>(a, per, warp_tot);
 }
 
 // Sorts key[0, n) bitonically, padded to a power of two.
@@ -102,10 +114,15 @@ __global__ void __launch_bounds__(kVtxThreads) k_vertex_event(Buffers b, int32_t
   __shared__ uint32_t warp_tot[33];
   __shared__ uint32_t s_n, s_lo, s_hi, s_full;
   const int e = blockIdx.x, tid = threadIdx.x;
+  if (e == 0 && tid == 0) b.cnt[CNT_SCAN_EV] = (unsigned long long)gridDim.x;
   // the event's tracks, clamped to the cleaned ntuplets of the batch
   const int64_t S = (int64_t)min(b.cnt[CNT_SV], (unsigned long long)cap_nt);
   const int64_t t0 = min(max(b.ev_nt_off[e], (int64_t)0), S);
   const int64_t nt = min(max(b.ev_nt_off[e + 1], t0), S) - t0;
+  // Buckets, and so the length of the scans, follow the event's size, up to four per track:
+  // 1000 events of 200 hits take 33 us, 77 with 16384 buckets for every event.
+  const int per = (int)min((int64_t)kVtxPer, max((int64_t)1, (nt + 255) / 256));
+  const int nb = per * kVtxThreads;  // >= nt, or kVtxMax
   if (tid == 0) {
     s_n = 0;
     s_lo = ~0u;
@@ -113,7 +130,10 @@ __global__ void __launch_bounds__(kVtxThreads) k_vertex_event(Buffers b, int32_t
     s_full = 0;
   }
 #pragma unroll
-  for (int j = 0; j < kVtxPer; ++j) vf[tid + j * kVtxThreads] = 0;
+  for (int j = 0; j < kVtxPer; ++j) {
+    if (j >= per) break;
+    vf[tid + j * kVtxThreads] = 0;
+  }
   __syncthreads();
   // [V1] the tracks that take part, keyed by (z0, position)
   uint32_t zlo = ~0u, zhi = 0;
@@ -150,10 +170,10 @@ __global__ void __launch_bounds__(kVtxThreads) k_vertex_event(Buffers b, int32_t
   const float lo = fmaxf(float_from_order_key(s_lo), -z_range);
   const float hi = fminf(float_from_order_key(s_hi), z_range);
   // buckets per cm (0: all tracks in one bucket); a track's bucket does not fall as z0 grows
-  const float scale = hi > lo ? __fdividef((float)kVtxMax, hi - lo) : 0.0f;
+  const float scale = hi > lo ? __fdividef((float)nb, hi - lo) : 0.0f;
   auto bucket = [&](unsigned long long v) {
     const float x = __fmul_rn(__fsub_rn(float_from_order_key((uint32_t)(v >> 32)), lo), scale);
-    return (uint32_t)min(kVtxMax - 1, max(0, __float2int_rz(x)));
+    return (uint32_t)min(nb - 1, max(0, __float2int_rz(x)));
   };
   {
     unsigned long long v[kVtxPer];
@@ -174,7 +194,7 @@ __global__ void __launch_bounds__(kVtxThreads) k_vertex_event(Buffers b, int32_t
     if (s_full) {
       vtx_bitonic(key, n);
     } else {
-      vtx_block_scan(vf, warp_tot);
+      vtx_block_scan(vf, per, warp_tot);
 #pragma unroll
       for (int j = 0; j < kVtxPer; ++j) {
         if ((uint32_t)tid + j * kVtxThreads >= n) break;
@@ -188,7 +208,7 @@ __global__ void __launch_bounds__(kVtxThreads) k_vertex_event(Buffers b, int32_t
         if (k >= n) break;
         v[j] = key[k];
         const uint32_t bk = bucket(v[j]);
-        const uint32_t first = vf[bk], last = bk + 1 < (uint32_t)kVtxMax ? vf[bk + 1] : n;
+        const uint32_t first = vf[bk], last = bk + 1 < (uint32_t)nb ? vf[bk + 1] : n;
         br[j] = first;
         for (uint32_t q = first; q < last; ++q) br[j] += key[q] < v[j] ? 1u : 0u;
       }
@@ -203,13 +223,13 @@ __global__ void __launch_bounds__(kVtxThreads) k_vertex_event(Buffers b, int32_t
   }
   auto starts = [&](uint32_t k) { return k == 0 || fsub(zk(k), zk(k - 1)) > dz; };
   // a group start whose group holds at least two tracks marks a vertex
-  for (uint32_t k = tid; k < (uint32_t)kVtxMax; k += kVtxThreads) {
+  for (uint32_t k = tid; k < (uint32_t)nb; k += kVtxThreads) {
     uint32_t f = 0;
     if (k + 1 < n && starts(k)) f = !starts(k + 1);
     vf[k] = f;
   }
   __syncthreads();
-  const uint32_t nv = vtx_block_scan(vf, warp_tot);
+  const uint32_t nv = vtx_block_scan(vf, per, warp_tot);
   for (uint32_t k = tid; k < n; k += kVtxThreads)
     if ((k + 1 < n ? vf[k + 1] : nv) > vf[k]) vstart[vf[k]] = (uint16_t)k;
   __syncthreads();
@@ -253,9 +273,13 @@ __global__ void __launch_bounds__(kVtxThreads) k_vertex_event(Buffers b, int32_t
 
 // Event e's vertices to the batch-wide list after those of the events before it; its
 // tracks' vertices become batch-wide indices; per-event offsets as int64 and the total
-// count.  blockIdx.y shares an event's tracks among blocks.
+// count.  blockIdx.y shares an event's tracks among blocks.  A block of up to kPlaceSum events
+// adds up the counts before its own itself; more events have them scanned first (SCANNED,
+// ev_nv[e] = vertices before event e), since those sums grow with the square of the events.
 constexpr int kPlaceThreads = 256;
 constexpr int kPlaceBlocks = 8;
+constexpr int kPlaceSum = 2048;
+template <bool SCANNED>
 __global__ void __launch_bounds__(kPlaceThreads) k_vertex_compact(Buffers b, uint64_t cap_nt) {
   pdl_sync();
   __shared__ uint32_t s_sum[kPlaceThreads / 32];
@@ -263,20 +287,25 @@ __global__ void __launch_bounds__(kPlaceThreads) k_vertex_compact(Buffers b, uin
   const int64_t S = (int64_t)min(b.cnt[CNT_SV], (unsigned long long)cap_nt);
   const int64_t t0 = min(max(b.ev_nt_off[e], (int64_t)0), S);
   const int64_t t1 = min(max(b.ev_nt_off[e + 1], t0), S);
-  uint32_t sum = 0;
-  for (int i = threadIdx.x; i < e; i += kPlaceThreads) sum += b.ev_nv[i];
-  sum = __reduce_add_sync(kFull, sum);
-  if (lane_id() == 0) s_sum[threadIdx.x >> 5] = sum;
-  __syncthreads();
-  uint32_t v0 = 0;
+  uint32_t v0 = 0, nv;
+  if (SCANNED) {
+    v0 = b.ev_nv[e];
+    nv = b.ev_nv[e + 1] - v0;
+  } else {
+    uint32_t sum = 0;
+    for (int i = threadIdx.x; i < e; i += kPlaceThreads) sum += b.ev_nv[i];
+    sum = __reduce_add_sync(kFull, sum);
+    if (lane_id() == 0) s_sum[threadIdx.x >> 5] = sum;
+    __syncthreads();
 #pragma unroll
-  for (int i = 0; i < kPlaceThreads / 32; ++i) v0 += s_sum[i];
-  const uint32_t nv = b.ev_nv[e];
+    for (int i = 0; i < kPlaceThreads / 32; ++i) v0 += s_sum[i];
+    nv = b.ev_nv[e];
+  }
   const uint32_t first = blockIdx.y * kPlaceThreads + threadIdx.x;
-  constexpr uint32_t kStep = kPlaceThreads * kPlaceBlocks;
-  for (uint32_t v = first; v < nv; v += kStep) b.vtx[v0 + v] = b.vtx_stage[t0 / 2 + v];
+  const uint32_t step = kPlaceThreads * gridDim.y;
+  for (uint32_t v = first; v < nv; v += step) b.vtx[v0 + v] = b.vtx_stage[t0 / 2 + v];
 #pragma unroll 4
-  for (int64_t t = t0 + first; t < t1; t += kStep) {
+  for (int64_t t = t0 + first; t < t1; t += step) {
     const int32_t v = b.trk_vtx[t];
     if (v >= 0) b.trk_vtx[t] = v + (int32_t)v0;
   }
@@ -301,9 +330,17 @@ cudaError_t launch_vertices(const Buffers& b, const Params& p, int n_events, int
   PT_TRACE(l, s, "k_vertex_event",
            launch_pdl(k_vertex_event, n_events, kVtxThreads, kVtxSmem, s, b, min_hits, dz,
                       1.25f * p.cuts.z0max, cap_nt));
-  PT_TRACE(l, s, "k_vertex_compact",
-           launch_pdl(k_vertex_compact, dim3(n_events, kPlaceBlocks), kPlaceThreads, 0, s, b,
-                      cap_nt));
+  // blocks for an event's tracks: enough to fill the GPU where the events do not
+  const dim3 grid(n_events, std::max(1, std::min(kPlaceBlocks, kPlaceBlocks * l.sms / n_events)));
+  if (n_events <= kPlaceSum) {
+    PT_TRACE(l, s, "k_vertex_compact",
+             launch_pdl(k_vertex_compact<false>, grid, kPlaceThreads, 0, s, b, cap_nt));
+  } else {
+    PT_TRACE(l, s, "scan",
+             launch_scan(b.ev_nv, b.ev_nv, &b.cnt[CNT_SCAN_EV], b.scan_part, s));
+    PT_TRACE(l, s, "k_vertex_compact",
+             launch_pdl(k_vertex_compact<true>, grid, kPlaceThreads, 0, s, b, cap_nt));
+  }
   return cudaGetLastError();
 }
 
