@@ -41,25 +41,40 @@ __global__ void k_export_candidates(Buffers b) {
   }
 }
 
-// One warp per sorted hit: the cells of its incoming segments, at their own slots (the
-// caller has marked every slot a hole).
+// A warp takes 32 sorted hits, one per lane, and slot by slot writes the cells of their
+// incoming segments, one per lane, at the cells' own slots (the caller has marked every slot a
+// hole): an event of few hits has one or two cells in a segment, a large one a hundred.
+// pt_get_cells on 20000 events of 4 hits 119 us, 150 with a warp per hit.
 __global__ void k_export_cells(Buffers b, int32_t B, int max_inner, uint64_t cap_cells,
                                int32_t* out3) {
   const uint64_t nc = min(b.cnt[CNT_CELLS], (unsigned long long)cap_cells);
   const int E = b.hdr->n_events;
   const uint32_t n_sorted = b.bin_start[E * kLayers * B];
-  const uint32_t nw = gridDim.x * (blockDim.x >> 5);
-  for (uint32_t s = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5); s < n_sorted; s += nw) {
-    const int32_t go = (int32_t)b.perm[s];
+  const uint32_t stride = gridDim.x * blockDim.x, lane = lane_id();
+  for (uint32_t s0 = blockIdx.x * blockDim.x + (threadIdx.x & ~31u); s0 < n_sorted; s0 += stride) {
+    const uint32_t s = s0 + lane;
+    const bool valid = s < n_sorted;
+    const int32_t go = valid ? (int32_t)b.perm[s] : 0;
     const int e = find_event(b.hit_off, E, go);
+    const int32_t off = b.hit_off[e];
     for (int k = 0; k < max_inner; ++k) {
-      const uint2 sg = b.seg[(uint64_t)s * max_inner + k];
-      for (uint32_t i = lane_id(); i < sg.y; i += 32) {
-        const uint64_t c = (uint64_t)sg.x + i;
-        if (c >= nc) break;
-        out3[c * 3 + 0] = (int32_t)b.perm[b.cell_in[c]] - b.hit_off[e];
-        out3[c * 3 + 1] = go - b.hit_off[e];
-        out3[c * 3 + 2] = e;
+      const uint2 sg = valid ? b.seg[(uint64_t)s * max_inner + k] : make_uint2(0u, 0u);
+      const uint32_t end = warp_incl_scan(sg.y), total = __shfl_sync(kFull, end, 31);
+      for (uint32_t i0 = 0; i0 < total; i0 += 32) {
+        const uint32_t i = i0 + lane;
+        uint32_t h = 0;  // the lane whose segment holds the i-th cell
+#pragma unroll
+        for (uint32_t o = 16; o > 0; o >>= 1)
+          if (i >= __shfl_sync(kFull, end, h + o - 1)) h += o;
+        const uint32_t first = __shfl_sync(kFull, sg.x, h);
+        const uint32_t before = __shfl_sync(kFull, end, h) - __shfl_sync(kFull, sg.y, h);
+        const int32_t h_go = __shfl_sync(kFull, go, h), h_off = __shfl_sync(kFull, off, h);
+        const int32_t h_e = __shfl_sync(kFull, e, h);
+        const uint64_t c = (uint64_t)first + (i - before);
+        if (i >= total || c >= nc) continue;
+        out3[c * 3 + 0] = (int32_t)b.perm[b.cell_in[c]] - h_off;
+        out3[c * 3 + 1] = h_go - h_off;
+        out3[c * 3 + 2] = h_e;
       }
     }
   }
