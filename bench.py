@@ -12,8 +12,10 @@ with a context each, so that one batch's copies overlap the other's kernels.
   python bench.py [--gpus N] [--steps K] [--warmup W] [--impl ours|reference]
 
 Under torchrun every rank runs its own replica on its own GPU (events are independent,
-no collective on the data path); rank 0 prints one JSON line.  `--impl reference`
-times the CPU oracle on the host cores on the same workload.
+no collective on the data path); rank 0 prints one JSON line with the rates, the roofline,
+the latencies and the physics of both forms, and writes everything it measured (per kernel,
+per serving rate, the tuning table) to the file of --details, which the line names.
+`--impl reference` times the CPU oracle on the host cores on the same workload.
 """
 
 from __future__ import annotations
@@ -700,6 +702,44 @@ def _serving(pt, rates, seconds: float, gate=None, threads: int = 16,
     return out
 
 
+# A reader of a bounded tail of the output must find the whole line in it.
+LINE_BYTES = 3000
+
+
+def short_line(full: dict, details: str) -> dict:
+    """What rank 0 prints of all that was measured: at most LINE_BYTES as JSON."""
+    line = {k: full[k] for k in
+            ("metric", "value", "unit", "n_gpus", "steps", "warmup", "ms_per_step",
+             "p99_ms_per_step", "higher_is_better", "scaling", "vs_baseline", "dtype", "data",
+             "config", "e2e", "clocks", "gpu_launches", "stages_ms", "broken_line", "raw_input",
+             "cpu_baseline") if full.get(k) is not None or k == "vs_baseline"}
+    line["roofline"] = {k: full["roofline"][k] for k in
+                        ("bound", "kernel", "achieved", "peak", "unit", "frac", "traffic",
+                         "peak_src", "algorithmic_bytes", "launch_ms", "issue_active_pct")}
+    line["gated"] = {k: full["gated"][k] for k in ("value", "ms_per_step", "p99_ms_per_step")}
+    if full["gated"]["e2e"]:
+        line["gated"]["e2e"] = full["gated"]["e2e"]["value"]
+    if full["physics"]["plain"]:
+        line["efficiency"] = {form: round(v["efficiency"], 6)
+                              for form, v in full["physics"].items()}
+    line["batch_workload"] = {form: v["value"] for form, v in full["batch_workload"].items()}
+    line["broken_line"] = full["broken_line"]["ms_per_step"]
+    line["raw_input"] = full["raw_input"]["ms_per_step"]
+    if full.get("latency"):
+        line["latency_p50_p99_ms"] = {k: [round(v["p50_ms"], 4), round(v["p99_ms"], 4)]
+                                      for k, v in full["latency"].items() if "p50_ms" in v}
+    if full.get("serving"):
+        line["serving_p50_p99_ms"] = {
+            form: {f"{r['offered_events_per_s']:g}/s": [round(r["p50_ms"], 3),
+                                                        round(r["p99_ms"], 3)]
+                   for r in full["serving"][form]} for form in ("plain", "gated")}
+    if "cpu_baseline" in line:
+        line["cpu_baseline"] = {k: line["cpu_baseline"][k]
+                                for k in ("value", "unit", "kind", "cores", "sample")}
+    line["details"] = details
+    return line
+
+
 def run_ours(args):
     import torch
     import paper_2501_05520_gb300 as pt
@@ -897,7 +937,12 @@ def run_ours(args):
                 for k in (1, 2, 4)]
         if world == 1 and not args.no_cpu_baseline:
             line["cpu_baseline"] = cpu_baseline()
-        print(json.dumps(line), flush=True)
+        try:
+            with open(args.details, "w") as f:
+                json.dump(line, f, indent=1)
+        except OSError as err:
+            print(f"details not written: {err}", file=sys.stderr)
+        print(json.dumps(short_line(line, os.path.basename(args.details))), flush=True)
     ctx.close()
     for c in e2e_more:
         c.close()
@@ -925,6 +970,8 @@ def main():
     ap.add_argument("--serve-seconds", type=float, default=2.0)
     ap.add_argument("--serve-instances-rate", type=float, default=16000.0,
                     help="offered events/s of the instance-scaling runs")
+    ap.add_argument("--details", default=os.path.join(ROOT, "bench_details.json"),
+                    help="file for everything measured")
     args = ap.parse_args()
     if args.impl == "reference":
         run_reference(args)
