@@ -33,7 +33,7 @@
 // centimetres, and the normal equations mix weights of 1e6 (hits) and 1e4..1e8 (kinks):
 // 24 bits are too few.  GB300 issues a float64 operation at 1/64 of the float32 rate, so the
 // numbers are pairs of floats (F2, 48 bits: 7 float32 operations for a product, 11 for a
-// sum); a track whose kinks outweigh its hits by more than 1e6 (so that too few of the 48
+// sum); a track whose kinks outweigh its hits by more than 1e7 (so that too few of the 48
 // bits are left for the hits: kStiffMax), or whose pass leaves the range of float32 anywhere
 // (a result that is not finite), is done in float64 by the same template.  On 211k tracks, of
 // events of 800 to 4400 particles, the errors against a 64-bit reference are the ones that a
@@ -157,14 +157,16 @@ template <class T>
 constexpr bool kPairs = false;
 template <>
 constexpr bool kPairs<F2> = true;
-// Largest weight of a kink in the normal equations that pairs of floats take: 1e6 times a hit's
-// in the transverse plane (1e6 /cm^2) and at most 4e6 times one's in the longitudinal plane
-// (2.5e5 on the barrel, 2.5e5 / cot^2 on a disk, where the kinks lose a factor 1 + cot^2 too).
-// There the solved offsets are within 2e-9 cm of the exact ones (5e-7 of a hit's error), less
+// Largest weight of a kink in the normal equations that pairs of floats take: 1e7 times a hit's
+// in the transverse plane (1e6 /cm^2) and 4e7 times a barrel hit's in the longitudinal one
+// (2.5e5), less by |cot| / 2 for steep tracks, whose hit errors on a disk, and so the offsets'
+// rounding, grow with it.  There the solved offsets are within 3e-9 cm of the exact ones, less
 // than the float32 results resolve, and the results equal those of the float64 form to one unit
 // in the last place; at 1e10 the offsets were up to 1e-3 of a hit's error away and z0 40 units.
-// A track of 1 GeV through 2 % of a radiation length has 1e4, one of 2 TeV reaches the limit.
-constexpr float kStiffMax = 1e12f;
+// A track of 1 GeV through 2 % of a radiation length has a weight of 1e4, one of 10 TeV reaches
+// the limit; the straight fakes that do make the refit of 64 pileup-200 events, 675k tracks, 458
+// instead of 455 us (510 with a tenth of the limit).
+constexpr float kStiffMax = 1e13f;
 
 // sin and cos of a float32 angle within +-pi (a track's phi0).
 __device__ __forceinline__ void sin_cos(float x, double& s, double& c) { sincos((double)x, &s, &c); }
@@ -420,7 +422,7 @@ __device__ __forceinline__ bool fit_pass(Work<T>& W, pt_track& tr, int n,
       const float a = fmaxf(lead(W.a[i - 1][t]), lead(W.a[i][t]));
       stiff = fmaxf(stiff, W.w[i][t] * a * a);
     }
-    if (!(stiff <= kStiffMax)) {
+    if (!(stiff * fmaxf(1.0f, 0.5f * fabsf(tr.cot_theta)) <= kStiffMax)) {
       tr.chi2_circle = __int_as_float(0x7fffffff);  // not finite: float64
       return true;
     }

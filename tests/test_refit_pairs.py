@@ -134,7 +134,7 @@ def solve_exact(n, wm, w, h, e, bend):
 
 @pytest.mark.parametrize("n", [4, 6])
 @pytest.mark.parametrize("plane,cot", [("transverse", 0.0), ("barrel z", 0.5), ("disk r", 6.0),
-                                       ("barrel and disk", 2.0)])
+                                       ("disk r", 12.0), ("barrel and disk", 2.0)])
 def test_offsets_at_the_limit(plane, cot, n):
     rng = np.random.default_rng(11)
     trials = 12
@@ -144,10 +144,11 @@ def test_offsets_at_the_limit(plane, cot, n):
              "disk r": [cot * SIGMA_L] * n,
              "barrel and disk": [SIGMA_L] * 2 + [cot * SIGMA_L] * (n - 2)}[plane]
     kf = 1.0 if plane == "transverse" else sth2
-    # the kernel's measure: kink weight times the larger inverse step squared, at its limit
+    # the kernel's measure, at its limit: kink weight times the larger inverse step squared,
+    # times |cot| / 2 where that is above 1
     w = np.zeros((n, trials))
     for i in range(1, n - 1):
-        w[i] = (STIFF * np.minimum(h[i - 1], h[i])**2).astype(f32)
+        w[i] = (STIFF / max(1.0, cot / 2) * np.minimum(h[i - 1], h[i])**2).astype(f32)
     wm = [1.0 / (s * s) for s in sigma]
     e = rng.normal(size=(n, trials)) * np.array(sigma)[:, None]
     hp = [F2.of(v) for v in h]
