@@ -46,7 +46,7 @@ namespace {
 constexpr float kTwoPi = 6.28318530717958647692f;
 constexpr float kHalfPi = 1.57079632679489661923f;
 constexpr int kConnWarps = 8;
-constexpr int kConnBlocksPerSm = 4;  // 64 registers per thread
+constexpr int kConnBlocksPerSm = 4;  // up to 64 registers per thread
 constexpr int kOut = 128;            // staged outgoing cells of one piece
 constexpr int kNb = 128;             // slope buckets of a piece (a multiple of 32)
 static_assert(kNb % 32 == 0, "buckets are scanned kNb / 32 per lane");
@@ -209,7 +209,7 @@ __global__ void __launch_bounds__(kConnWarps * 32, kConnBlocksPerSm)
 
   const uint32_t n_warps = gridDim.x * kConnWarps;
   // chunks of sorted middle hits, the first by the warp's number, the others from a work
-  // counter (the chunk in shared memory: the kernel's 64 registers are all in use)
+  // counter (the chunk in shared memory: the kernel has no registers left)
   if (lane == 0) {
     W.per = search_chunk(n_sorted, n_warps);
     W.dyn0 = W.per * n_warps;

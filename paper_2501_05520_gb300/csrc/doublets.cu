@@ -89,7 +89,9 @@ __device__ __forceinline__ void reverse_windows(const Buffers& b, const pt_cuts&
 // on as few lanes as the chunk has hits.  The whole call in us with the windows found here
 // (in the search): 64 pileup-200 events 5439 (5516), 7 gap-pair events 1109 (1133), one
 // pileup-200 event 320 (326); but one pileup-50 event 188 (185), where the launch costs more,
-// so contexts of fewer than kWindowsMinHits hits have no such launch.
+// so contexts of fewer than kWindowsMinHits hits have no such launch.  A small batch in a
+// larger context does: an event of 200 hits 88 us with it and 90 without, of 10139 hits 132 to
+// 137 and 128.
 constexpr int64_t kWindowsMinHits = 32768;
 __global__ void k_windows(Buffers b, pt_cuts cuts, PairTable pt, int32_t B) {
   pdl_sync();
@@ -105,10 +107,10 @@ __global__ void k_windows(Buffers b, pt_cuts cuts, PairTable pt, int32_t B) {
   }
 }
 
-// Warps take chunks of a few consecutive sorted (outer) hits (search_chunk), the first
-// by their own number, the others from a work counter.  The chunk's windows are read
-// (WINDOWS: k_windows has run) or found lane-parallel, one hit per lane, and kept in shared
-// memory; the warp then searches them hit by hit.
+// Warps take chunks of a few consecutive sorted (outer) hits (search_chunk), every one from a
+// work counter.  The chunk's windows are read (WINDOWS: k_windows has run) or found
+// lane-parallel, one hit per lane, and kept in shared memory; the warp then searches them hit
+// by hit.
 template <bool WINDOWS>
 __global__ void __launch_bounds__(kWarpsPerBlock * 32, 5)
     k_doublets(Buffers b, pt_cuts cuts, PairTable pt, int32_t B, uint64_t cap_cells) {

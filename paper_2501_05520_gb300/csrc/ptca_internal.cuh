@@ -167,8 +167,14 @@ struct BatchHeader {
 };
 constexpr size_t kHeaderBytes = 256;  // hit_off follows, and small host inputs follow that
 static_assert(sizeof(BatchHeader) <= kHeaderBytes, "header fits its place");
-constexpr int64_t kSmallHits = 4096;    // host inputs of up to so many hits go up in one copy
-constexpr int64_t kSmallTracks = 4096;  // up to so many results come back without a copy
+// Host inputs of up to kSmallHits hits go up in one copy, packed behind the header: an event
+// of 205 hits 94 us for the whole call instead of 103 with a copy per array, of 3666 hits 120
+// instead of 124, of 7314 no less.  Results of up to kSmallTracks tracks come back in a pinned
+// block instead of in a copy per array: 42 tracks 94 instead of 129 us into ordinary memory
+// and 89 instead of 99 into pinned memory, 3107 tracks 180 instead of 192, but 166 instead of
+// 160 into pinned memory.
+constexpr int64_t kSmallHits = 4096;
+constexpr int64_t kSmallTracks = 4096;
 
 // The layer-pair table of a context, as the kernels read it (a kernel argument):
 // outer[L][k], k < n_outer[L], are the outer layers paired with inner layer L, inner[L][k],
