@@ -383,6 +383,9 @@ pt_status ctx_results_async(pt_ctx* c, int64_t S, int32_t* hits, uint8_t* nhits,
                             pt_track* tracks, int64_t* event_offsets, cudaEvent_t done);
 
 // ------------------------------------------------------------------ launchers
+// device arrays of n hits to the context's input arrays
+void launch_take_inputs(const Buffers& b, const float* x, const float* y, const float* z,
+                        const uint8_t* layer, int64_t n, const Launch& l, cudaStream_t s);
 void launch_clear(const Buffers& b, const Params& p, const Launch& l, cudaStream_t s);
 void launch_bin_hits(const Buffers& b, const Params& p, const Launch& l, cudaStream_t s);
 void launch_doublets(const Buffers& b, const Params& p, const Launch& l, cudaStream_t s);
