@@ -52,14 +52,14 @@ CONFIG4_SEED0 = 5000  # batch workload: 64 events, pileup ~ Poisson(140) clipped
 # DRAM traffic per event of the main kernels from one ncu capture (8 PU200 events per
 # launch, profiles/), valid only while the kernel's sources hash to the recorded value.
 NCU_TRAFFIC = {
-    "k_doublets": {"bytes_per_event": 5030304, "issue_active_pct": 71.5,
-                   "warp_inst_per_event": 23067386, "sha": "364d637539bf"},
-    "k_connect": {"bytes_per_event": 31699392, "issue_active_pct": 71.2,
-                  "warp_inst_per_event": 45494649, "sha": "2bd993a45f34"},
-    "k_link_targets": {"bytes_per_event": 13892704, "issue_active_pct": 17.3,
-                       "warp_inst_per_event": 773766, "sha": "2bd993a45f34"},
-    "k_find_ntuplets": {"bytes_per_event": 23672640, "issue_active_pct": 28.7,
-                        "warp_inst_per_event": 2260666, "sha": "695e7bd16fd6"},
+    "k_doublets": {"bytes_per_event": 5046560, "issue_active_pct": 71.4,
+                   "warp_inst_per_event": 23067895, "sha": "e4e6a90eb06e"},
+    "k_connect": {"bytes_per_event": 31608192, "issue_active_pct": 70.3,
+                  "warp_inst_per_event": 45479427, "sha": "7cdee8bb51c2"},
+    "k_link_targets": {"bytes_per_event": 13900448, "issue_active_pct": 17.9,
+                       "warp_inst_per_event": 773435, "sha": "7cdee8bb51c2"},
+    "k_find_ntuplets": {"bytes_per_event": 23695296, "issue_active_pct": 29.1,
+                        "warp_inst_per_event": 2260772, "sha": "8eb0a36b4912"},
 }
 SMS, SCHEDULERS_PER_SM = 152, 4  # GB300: each scheduler issues one warp instruction a cycle
 
